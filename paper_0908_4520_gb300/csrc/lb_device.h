@@ -117,6 +117,7 @@ struct Launch {
     int n_eq;                 // 1..4
     int upwind;               // 1: second-order upwind streaming (off-lattice sets, 32/64-bit storage)
     int grid;                 // blocks (persistent grid-stride over tiles)
+    int follows;              // 1: a step captured behind another one (programmatic dependent launch)
     cudaStream_t stream;
     const void* args;         // Args<float>/Args<double> matching the unit, or Shape* for kQueryShape
 };

@@ -60,15 +60,17 @@ struct Is16<__nv_bfloat16> : std::true_type {};
 template <>
 struct Is16<__half> : std::true_type {};
 
+// (loads of the populations do not take the read-only path: a step launch may have started, and its
+// caches filled, before the launch that writes them has ended; see await_previous_step)
 template <class S, class R>
 __device__ __forceinline__ R ld1(const S* p, R scale) {
     if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        return __bfloat162float(__ldg(p)) * scale;
+        return __bfloat162float(*p) * scale;
     } else if constexpr (std::is_same<S, __half>::value) {
-        return __half2float(__ldg(p)) * scale;
+        return __half2float(*p) * scale;
     } else {
         (void)scale;
-        return __ldg(p);
+        return *p;
     }
 }
 
@@ -111,19 +113,19 @@ __device__ __forceinline__ void sld2(const S* p, R scale, R& v0, R& v1) {
 template <class S, class R>
 __device__ __forceinline__ void ld2(const S* p, R scale, R& v0, R& v1) {
     if constexpr (std::is_same<S, float>::value) {
-        const float2 t = __ldg(reinterpret_cast<const float2*>(p));
+        const float2 t = *reinterpret_cast<const float2*>(p);
         v0 = t.x;
         v1 = t.y;
     } else if constexpr (std::is_same<S, double>::value) {
-        const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+        const double2 t = *reinterpret_cast<const double2*>(p);
         v0 = t.x;
         v1 = t.y;
     } else if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        const float2 t = __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(p)));
+        const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
         v0 = t.x * scale;
         v1 = t.y * scale;
     } else {
-        const float2 t = __half22float2(__ldg(reinterpret_cast<const __half2*>(p)));
+        const float2 t = __half22float2(*reinterpret_cast<const __half2*>(p));
         v0 = t.x * scale;
         v1 = t.y * scale;
     }
@@ -140,20 +142,6 @@ __device__ __forceinline__ void st1(S* p, R v, R scinv) {
         (void)scinv;
         *p = v;
     }
-}
-
-template <class S, class R>
-__device__ __forceinline__ void st2(S* p, R v0, R v1, R scinv) {
-    if constexpr (std::is_same<S, float>::value) {
-        __stcs(reinterpret_cast<float2*>(p), make_float2(v0, v1));
-    } else if constexpr (std::is_same<S, double>::value) {
-        __stcs(reinterpret_cast<double2*>(p), make_double2(v0, v1));
-    } else if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        __stcs(reinterpret_cast<__nv_bfloat162*>(p), __floats2bfloat162_rn(v0 * scinv, v1 * scinv));
-    } else {
-        __stcs(reinterpret_cast<__half2*>(p), __floats2half2_rn(v0 * scinv, v1 * scinv));
-    }
-    (void)scinv;
 }
 
 template <class S, class R>
@@ -419,7 +407,10 @@ struct Pack<float, 2> {
 #define LB_TMA_BAND -1
 #endif
 #ifndef LB_TMA_BAND_SHIFT
-#define LB_TMA_BAND_SHIFT 4  // band height of the exact-shift sets under LB_TMA_BAND = -1
+// band height of the exact-shift sets under LB_TMA_BAND = -1 (D2Q37 FP32 at 4096^2 and 2048^2, GLUPS:
+// bands of 2 / 3 / 4 / 6 / 8 tile rows 19.63 / 19.65 / 19.40 / 18.91 / 18.44 and 19.63 / 19.77 /
+// 19.43 / 19.58 / 19.36)
+#define LB_TMA_BAND_SHIFT 3
 #endif
 #ifndef LB_TMA_WIDE_WARPS
 #define LB_TMA_WIDE_WARPS 0  // consumer warps of the store-staged kernel (two per tile row); 0: 18, q = 64: 14
@@ -636,10 +627,15 @@ __device__ __forceinline__ R warp_sum(R v) {
     return v;
 }
 
-// Write the lane's V storage values of plane `pl` (pointer to cell (0,0)) at
-// every periodic image of (x, y) inside the ghost rim (not at (x, y) itself).
-template <class S, class R, int V>
-__device__ __forceinline__ void store_images(const Args<R>& A, S* pl, int x, int y, const S (&v)[V]) {
+// The periodic images of the V cells at (x.., y) inside the ghost rim (not (x, y) itself), one
+// after another: img(xi, yi) of each.  A cell near an edge has one to three of them, on a grid
+// narrower than the rim more.  The image is the outer loop and the velocities the inner, unrolled
+// one, so that all q values leave from registers as independent stores: a copy of the stored
+// values, velocity by velocity, was a chain of q dependent memory round trips that every warp of a
+// boundary row waited for (us per level before / after: D2Q16-GH FP64 64 x 1 35.7 / 24.9, D2Q36-GH
+// FP32 256^2 37.6 / 23.6, 1024^2 127 / 76, 2048^2 282 / 235, D2Q64-GH FP32 2048^2 768 / 492).
+template <class R, int V, class F>
+__device__ __forceinline__ void for_images(const Args<R>& A, int x, int y, F&& img) {
     int ylo = y;
     while (ylo - A.ny >= -A.gy) ylo -= A.ny;
     int xlo = x;
@@ -647,56 +643,26 @@ __device__ __forceinline__ void store_images(const Args<R>& A, S* pl, int x, int
     for (int yi = ylo; yi < A.ny + A.gy; yi += A.ny) {
         for (int xi = xlo; xi + V <= A.nx + kGhostX; xi += A.nx) {
             if (xi == x && yi == y) continue;
-            S* q = pl + (long long)yi * A.pitch + xi;
-            if constexpr (V == 2) {
-                store_raw2<S>(q, v[0], v[1]);
-            } else {
-                store_raw<S>(q, v[0]);
-            }
+            img(xi, yi);
         }
     }
 }
 
-// Out-of-line image writer (boundary lanes only), so the unrolled callers stay small.
-// Copy the q values this thread just stored at (x.., y) to their periodic images.
-template <class S, class R, int V>
-__device__ __noinline__ void rim_images(const Args<R>& A, S* dst, int q, int x, int y) {
-    for (int a = 0; a < q; ++a) {
-        S* pl = dst + (long long)a * A.plane + A.origin;
-        const S* p = pl + (long long)y * A.pitch + x;
-        S v[V];
-        v[0] = p[0];
-        if constexpr (V == 2) v[V - 1] = p[1];
-        store_images<S, R, V>(A, pl, x, y, v);
-    }
+// Whether the V cells at (x.., y) have an image in the ghost rim.
+template <class R, int V>
+__device__ __forceinline__ bool has_images(const Args<R>& A, int x, int y) {
+    return x < kGhostX || x + V > A.nx - kGhostX || y < A.gy || y >= A.ny - A.gy;
 }
 
-// The same for the store-staged kernel: the values are taken from the output tile in shared
-// memory (out[a * ostride]), which the TMA store writes to (x, y) itself.
+// Write the lane's value at (x, y) and at every periodic image (round to nearest: used for the
+// initial state).
 template <class S, class R>
-__device__ __noinline__ void rim_images_tile(const Args<R>& A, S* dst, const S* out, int ostride, int q, int x, int y) {
-    for (int a = 0; a < q; ++a) {
-        S* pl = dst + (long long)a * A.plane + A.origin;
-        const S v[1] = {out[a * ostride]};
-        store_images<S, R, 1>(A, pl, x, y, v);
-    }
-}
-
-// Write the lane's values at (x, y) and at every periodic image.
-// (round to nearest: used for the initial state)
-template <class S, class R, int V>
-__device__ __forceinline__ void store_cells(const Args<R>& A, S* pl, int x, int y, const R (&v)[V], R si) {
-    S* p = pl + (long long)y * A.pitch + x;
-    S sv[V];
-    if constexpr (V == 2) {
-        st2<S, R>(p, v[0], v[1], si);
-        sv[0] = p[0];
-        sv[V - 1] = p[1];
-    } else {
-        st1<S, R>(p, v[0], si);
-        sv[0] = p[0];
-    }
-    if (x < kGhostX || x + V > A.nx - kGhostX || y < A.gy || y >= A.ny - A.gy) store_images<S, R, V>(A, pl, x, y, sv);
+__device__ __forceinline__ void store_cell(const Args<R>& A, S* pl, int x, int y, R v, R si) {
+    S sv;
+    st1<S, R>(&sv, v, si);
+    store_raw<S>(pl + (long long)y * A.pitch + x, sv);
+    if (has_images<R, 1>(A, x, y))
+        for_images<R, 1>(A, x, y, [&](int xi, int yi) { store_raw<S>(pl + (long long)yi * A.pitch + xi, sv); });
 }
 
 // ------------------------------------------------------------ collision (shared)
@@ -1050,7 +1016,7 @@ __device__ __forceinline__ CellOut<float> collide_cell_pairs(const Tab<float>& t
 // shared memory, out[a * OSTRIDE] for velocity a, instead of to HBM (the periodic images in
 // the ghost rim are still written here, from that tile).
 template <class VS, int N, class S, class R, int V, int KIND, class T, int OSTRIDE = 0>
-__device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], S* __restrict__ dst, int y,
+__device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], S* dst, int y,
                                               const Lane& g, bool diag, R (&acc)[6], int lane, long long lvl,
                                               R gt, S* out = nullptr) {
     constexpr int Q = VS::Q;
@@ -1127,33 +1093,17 @@ __device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], 
             });
         }
     }
-    if constexpr (STEP && OSTRIDE > 0) {
-        if (g.own) {
-            // the same stochastic rounding stream as the global stores below (same bits)
-            uint32_t r0 = 0;
-            if constexpr (Is16<S>::value) r0 = sr_seed(lvl, (long long)y * A.nx + g.x);
-            static_for<0, Q>([&](auto ac) {
-                constexpr int a = decltype(ac)::value;
-                if constexpr (Is16<S>::value) {
-                    r0 = sr_next(r0);
-                    out[a * OSTRIDE] = to_storage<S, R>(lane_get<0>(ft[a]), store_scale<S, R>(A.tab, a), r0);
-                } else {
-                    out[a * OSTRIDE] = lane_get<0>(ft[a]);
-                }
-            });
-            if (g.x < kGhostX || g.x + V > A.nx - kGhostX || y < A.gy || y >= A.ny - A.gy)
-                rim_images_tile<S, R>(A, dst, out, OSTRIDE, Q, g.x, y);
-        }
-    }
-    if constexpr (STEP && OSTRIDE == 0) {
-        if (g.own) {
-            S* base = dst + A.origin + (long long)y * A.pitch + g.x;
+    if constexpr (STEP) {
+        // The relaxed populations, straight from registers: to the cell (OSTRIDE > 0: to the
+        // output tile) and, for the lanes of a boundary, to its periodic images in the ghost rim.
+        // put(p) writes all q planes at offset p of the first; each call draws the 16-bit rounding
+        // bits anew from the cell's own stream, so every image holds the cell's bits.
+        auto put = [&](S* p, long long stride) {
             uint32_t r0 = 0, r1 = 0;
             if constexpr (Is16<S>::value) {
                 r0 = sr_seed(lvl, (long long)y * A.nx + g.x);
                 r1 = sr_seed(lvl, (long long)y * A.nx + g.x + 1);
             }
-            S* p = base;
             static_for<0, Q>([&](auto ac) {
                 constexpr int a = decltype(ac)::value;
                 const R si = store_scale<S, R>(A.tab, a);
@@ -1174,12 +1124,19 @@ __device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], 
                         store_raw<S>(p, s0);
                     }
                 }
-                p += A.plane;
+                p += stride;
             });
-            // periodic images in the ghost rim (boundary cells only): one out-of-line call
-            // that copies the values just stored, so the velocity loop above stays branch-free
-            if (g.x < kGhostX || g.x + V > A.nx - kGhostX || y < A.gy || y >= A.ny - A.gy)
-                rim_images<S, R, V>(A, dst, Q, g.x, y);
+        };
+        if (g.own) {
+            S* const base = dst + A.origin;
+            if constexpr (OSTRIDE > 0) {
+                put(out, OSTRIDE);
+            } else {
+                put(base + (long long)y * A.pitch + g.x, A.plane);
+            }
+            if (has_images<R, V>(A, g.x, y))
+                for_images<R, V>(A, g.x, y,
+                                 [&](int xi, int yi) { put(base + (long long)yi * A.pitch + xi, A.plane); });
         }
     }
     if constexpr (STEP) {
@@ -1284,6 +1241,14 @@ __device__ __forceinline__ void finish_step(const Args<R>& A, R (&acc)[6], doubl
     }
 }
 
+// Programmatic dependent launch: a step launch may start while the one before it ends (its blocks
+// take the SMs that are free, set up and wait here); what that launch wrote is read only after
+// this.  It then lets the launch after it do the same.  No effect on a launch without the attribute.
+__device__ __forceinline__ void await_previous_step() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ------------------------------------------------------------ register kernel
 // KIND = kStep:    f* (next level) into dst, diagnostics when due.
 // KIND = kStepForced: the same with the body force (lb_params.force_amp != 0).
@@ -1297,13 +1262,14 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
     constexpr int ROWS = Cfg<VS, S>::ROWS;
     constexpr int TW = 32 * V;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const S* __restrict__ src = static_cast<const S*>(A.src);
-    S* __restrict__ dst = static_cast<S*>(A.dst);
+    const S* src = static_cast<const S*>(A.src);
+    S* dst = static_cast<S*>(A.dst);
 
     constexpr bool STEP = (KIND == kStep || KIND == kStepForced);
     long long lvl = 0;
     bool diag = false;
     if constexpr (STEP) {
+        await_previous_step();
         lvl = __ldcg(A.level);
         diag = (A.diag_every > 0) && (lvl % A.diag_every == 0);
     } else {
@@ -1600,6 +1566,7 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
     }
     __syncthreads();
 
+    if constexpr (KIND == kStep) await_previous_step();
     const long long lvl = __ldcg(A.level);
     const bool diag = KIND == kStep && (A.diag_every > 0) && (lvl % A.diag_every == 0);
     R acc[6] = {0, 0, 0, 0, 0, 0};
@@ -1869,13 +1836,28 @@ __global__ void __launch_bounds__(256) lb_init_kernel(const __grid_constant__ Ar
         const R th = A.isothermal ? R(0) : (R)(T - 1.0);
         equilibrium_dev<VS, N, R>(A.tab, drho, (R)rho, (R)ux, (R)uy, th, [&](auto ac, R deq) {
             constexpr int a = decltype(ac)::value;
-            const R v[1] = {deq};
-            store_cells<S, R, 1>(A, dst + (long long)a * A.plane + A.origin, x, y, v, store_scale<S, R>(A.tab, a));
+            store_cell<S, R>(A, dst + (long long)a * A.plane + A.origin, x, y, deq, store_scale<S, R>(A.tab, a));
         });
     }
 }
 
 // ------------------------------------------------------------ dispatch
+// A step launch; `follows` makes it a programmatic dependent of the launch before it.
+template <class R>
+cudaError_t launch_step(void (*kernel)(const Args<R>), const Launch& L, int threads, int smem) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)L.grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = L.stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = L.follows ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, *static_cast<const Args<R>*>(L.args));
+}
+
 template <class VS, int N, class S, class R>
 cudaError_t launch_typed(const Launch& L) {
     using C = Cfg<VS, S>;
@@ -1958,10 +1940,8 @@ cudaError_t launch_typed(const Launch& L) {
     if (L.upwind && (L.kind == kStepTma || L.kind == kMomentsTma)) {
         if constexpr (kUpwTma) {
             using TU = TmaCfg<VS, S, true>;
-            if (L.kind == kStepTma)
-                lb_tma_step_kernel<VS, N, S, true><<<L.grid, TU::THREADS, TU::SMEM, L.stream>>>(A);
-            else
-                lb_tma_step_kernel<VS, N, S, true, kMoments><<<L.grid, TU::THREADS, TU::SMEM, L.stream>>>(A);
+            if (L.kind == kStepTma) return launch_step<R>(lb_tma_step_kernel<VS, N, S, true>, L, TU::THREADS, TU::SMEM);
+            lb_tma_step_kernel<VS, N, S, true, kMoments><<<L.grid, TU::THREADS, TU::SMEM, L.stream>>>(A);
             return cudaGetLastError();
         }
         return cudaErrorNotSupported;
@@ -1970,11 +1950,9 @@ cudaError_t launch_typed(const Launch& L) {
         if constexpr (kUpw) {
             switch (L.kind) {
                 case kStep:
-                    lb_fused_kernel<VS, N, S, R, kStep, true><<<L.grid, C::THREADS, 0, L.stream>>>(A);
-                    return cudaGetLastError();
+                    return launch_step<R>(lb_fused_kernel<VS, N, S, R, kStep, true>, L, C::THREADS, 0);
                 case kStepForced:
-                    lb_fused_kernel<VS, N, S, R, kStepForced, true><<<L.grid, C::THREADS, 0, L.stream>>>(A);
-                    return cudaGetLastError();
+                    return launch_step<R>(lb_fused_kernel<VS, N, S, R, kStepForced, true>, L, C::THREADS, 0);
                 case kMoments:
                     lb_fused_kernel<VS, N, S, R, kMoments, true><<<L.grid, C::THREADS, 0, L.stream>>>(A);
                     return cudaGetLastError();
@@ -1989,11 +1967,9 @@ cudaError_t launch_typed(const Launch& L) {
     }
     switch (L.kind) {
         case kStep:
-            lb_fused_kernel<VS, N, S, R, kStep><<<L.grid, C::THREADS, 0, L.stream>>>(A);
-            break;
+            return launch_step<R>(lb_fused_kernel<VS, N, S, R, kStep>, L, C::THREADS, 0);
         case kStepForced:
-            lb_fused_kernel<VS, N, S, R, kStepForced><<<L.grid, C::THREADS, 0, L.stream>>>(A);
-            break;
+            return launch_step<R>(lb_fused_kernel<VS, N, S, R, kStepForced>, L, C::THREADS, 0);
         case kMoments:
             lb_fused_kernel<VS, N, S, R, kMoments><<<L.grid, C::THREADS, 0, L.stream>>>(A);
             break;
@@ -2001,10 +1977,7 @@ cudaError_t launch_typed(const Launch& L) {
             lb_init_kernel<VS, N, S, R><<<L.grid, 256, 0, L.stream>>>(A);
             break;
         case kStepTma:
-            if constexpr (kTma) {
-                lb_tma_step_kernel<VS, N, S><<<L.grid, T::THREADS, T::SMEM, L.stream>>>(A);
-                break;
-            }
+            if constexpr (kTma) return launch_step<R>(lb_tma_step_kernel<VS, N, S>, L, T::THREADS, T::SMEM);
             return cudaErrorNotSupported;
         case kMomentsTma:
             if constexpr (kTma) {
@@ -2015,8 +1988,7 @@ cudaError_t launch_typed(const Launch& L) {
         case kStepTmaStore:
             if constexpr (kStore) {
                 using TS = TmaCfg<VS, S, false, true>;
-                lb_tma_step_kernel<VS, N, S, false, kStep, true><<<L.grid, TS::THREADS, TS::SMEM, L.stream>>>(A);
-                break;
+                return launch_step<R>(lb_tma_step_kernel<VS, N, S, false, kStep, true>, L, TS::THREADS, TS::SMEM);
             }
             return cudaErrorNotSupported;
         default:
