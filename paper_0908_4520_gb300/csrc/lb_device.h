@@ -29,6 +29,8 @@ struct Tab {
     R hn[kMaxNA][kMaxN + 1];  // He_k(a_i) / k!
     R whn[kMaxNA][kMaxN + 1]; // W_i He_k(a_i) / k!
     R lw[kMaxNA][3];          // Lax-Wendroff weights of f*(x-1), f*(x), f*(x+1)
+    R lwt[3][kMaxNA];         // the same, node index innermost: a pair of neighbouring nodes is one 64-bit operand
+    R whnt[kMaxN + 1][kMaxNA]; // whn, node index innermost
     R uw[kMaxNA][3];          // second-order upwind weights of f*(x-2s), f*(x-s), f*(x), s = sign(a_i)
     R w[kMaxQ];               // quadrature weights
     R winv[kMaxQ];            // 1 / w

@@ -70,7 +70,7 @@ void build_tab(const VelocitySetInfo& vs, double dt, double dx, double scale, lb
         for (int k = 0; k <= lbk::kMaxN; ++k) {
             if (k > 1) fact *= k;
             t.hn[i][k] = (R)(hermite_he(k, vs.axis[i]) / fact);
-            t.whn[i][k] = (R)(wm[i] * hermite_he(k, vs.axis[i]) / fact);
+            t.whnt[k][i] = t.whn[i][k] = (R)(wm[i] * hermite_he(k, vs.axis[i]) / fact);
         }
         const double C = vs.on_lattice ? 0.0 : vs.axis[i] * dt / dx;
         double l0 = 0.5 * C * (1.0 + C), l2 = -0.5 * C * (1.0 - C);
@@ -81,6 +81,7 @@ void build_tab(const VelocitySetInfo& vs, double dt, double dx, double scale, lb
         t.lw[i][0] = (R)l0;
         t.lw[i][1] = (R)(1.0 - l0 - l2);
         t.lw[i][2] = (R)l2;
+        for (int k = 0; k < 3; ++k) t.lwt[k][i] = t.lw[i][k];
         // second-order upwind (Beam-Warming), c = |C|: the two upstream neighbours and the cell
         const double c = std::fabs(C);
         double u0 = 0.5 * c * (c - 1.0), u1 = c * (2.0 - c);

@@ -864,6 +864,30 @@ struct PairCollision {
     static constexpr bool value = VS::kProductWeights && !VS::kOnLattice && VS::NA % 2 == 0;
 };
 
+// Tensor-product Lax-Wendroff of a velocity pair (a, a + 1) of one lane's cell: the y pass over
+// the lane's column (values of the rows y - 1, y, y + 1), then the x pass, whose neighbours'
+// columns come by shuffles.  The pair has one x node and two y nodes, so both passes run as
+// packed f32x2 operations: 6 instead of 12 arithmetic instructions a pair, the same rounding.
+// (32 levels: D2Q36-GH FP32 4096^2 28.7 -> 28.2 ms, D2Q64-GH FP16 2048^2 17.0 -> 16.4 ms.)
+template <class VS, int A_>
+__device__ __forceinline__ f2 lw_y_pair(const Tab<float>& t, f2 fm, f2 f0, f2 fp) {
+    constexpr int iy = VS::iy(A_);
+    const f2 l0 = f2{t.lwt[0][iy], t.lwt[0][iy + 1]}, l1 = f2{t.lwt[1][iy], t.lwt[1][iy + 1]},
+             l2 = f2{t.lwt[2][iy], t.lwt[2][iy + 1]};
+    return vfma(l0, fm, vfma(l1, f0, vmul(l2, fp)));
+}
+template <class VS, int A_>
+__device__ __forceinline__ f2 lw_x_pair(const Tab<float>& t, f2 gl, f2 g, f2 gr) {
+    constexpr int ix = VS::ix(A_);
+    return vfma(vsplat<f2>(t.lw[ix][0]), gl, vfma(vsplat<f2>(t.lw[ix][1]), g, vmul(vsplat<f2>(t.lw[ix][2]), gr)));
+}
+__device__ __forceinline__ f2 shfl_up2(f2 v) {
+    return f2{__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1)};
+}
+__device__ __forceinline__ f2 shfl_down2(f2 v) {
+    return f2{__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1)};
+}
+
 // ow, owlo, hn1lo, whn1lo: the relaxation tables of omega (Tab), the handle's own or, in a
 // batch, the instance's.
 template <class VS, int N, bool COLLIDE, class F>
@@ -971,7 +995,7 @@ __device__ __forceinline__ CellOut<float> collide_cell_pairs(const Tab<float>& t
             QYp[j][0] = f2{t.wm[2 * j], t.wm[2 * j + 1]};
 #pragma unroll
             for (int ky = 1; ky <= N; ++ky)
-                QYp[j][ky] = vmul(f2{t.whn[2 * j][ky], t.whn[2 * j + 1][ky]}, vsplat<f2>(cy[ky]));
+                QYp[j][ky] = vmul(f2{t.whnt[ky][2 * j], t.whnt[ky][2 * j + 1]}, vsplat<f2>(cy[ky]));
             // the first-order factor's small second term (exact momentum identity)
             QYp[j][1] = vfma(f2{whn1lo_t[2 * j], whn1lo_t[2 * j + 1]}, vsplat<f2>(cy[1]), QYp[j][1]);
         }
@@ -1538,6 +1562,8 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
     constexpr int NS = C::NS, NG = C::NG, K = C::K, BW = C::BW, BOX = C::BOX, SLOT = C::SLOT;
     constexpr int STAGE_ELEMS = C::STAGE_BYTES / (int)sizeof(S);
     constexpr int OSTRIDE = WIDE ? ROWS * C::TWO : 0;  // output tile: elements per velocity
+    // Lax-Wendroff with halo lanes: the stencil runs on velocity pairs
+    constexpr bool PAIRS = C::HALO && PairCollision<VS>::value && K % 2 == 0;
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     // TMA destinations must be 128-byte aligned: align the base explicitly
     unsigned char* const smem_raw =
@@ -1670,7 +1696,23 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                     static_for<0, K>([&](auto jc) {
                         constexpr int j = decltype(jc)::value;
                         constexpr int a = grp * K + j;
-                        if constexpr (a < Q) {
+                        if constexpr (a < Q && PAIRS) {
+                            // the stencil is linear: 16-bit values are scaled once, after it
+                            if constexpr (j % 2 == 0) {
+                                const R one = R(1);
+                                const S* rm = st + j * SLOT + trow * BW + c_lw;  // row y - 1 of velocity a
+                                const S* rn = rm + SLOT;                         // and of a + 1
+                                const f2 gv = lw_y_pair<VS, a>(
+                                    A.tab, f2{sld1<S, R>(rm, one), sld1<S, R>(rn, one)},
+                                    f2{sld1<S, R>(rm + BW, one), sld1<S, R>(rn + BW, one)},
+                                    f2{sld1<S, R>(rm + 2 * BW, one), sld1<S, R>(rn + 2 * BW, one)});
+                                f2 v = lw_x_pair<VS, a>(A.tab, shfl_up2(gv), gv, shfl_down2(gv));
+                                if constexpr (Is16<S>::value)
+                                    v = vmul(v, f2{load_scale<S, R>(A.tab, a), load_scale<S, R>(A.tab, a + 1)});
+                                ft[a] = v.x;
+                                ft[a + 1] = v.y;
+                            }
+                        } else if constexpr (a < Q) {
                             const R sc = load_scale<S, R>(A.tab, a);
                             const S* box = st + j * SLOT;
                             if constexpr (UPW) {
@@ -1707,7 +1749,7 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                                 const S* rm = box + trow * BW;
                                 const S* r0 = rm + BW;
                                 const S* rp = r0 + BW;
-                                if constexpr (C::HALO) {
+                                if constexpr (C::HALO) {  // (a set of no pairs)
                                     // y pass of the lane's column; x pass from the neighbours
                                     const R f0 = sld1<S, R>(r0 + c_lw, one);
                                     const R fm = sld1<S, R>(rm + c_lw, one);
