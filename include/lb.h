@@ -298,13 +298,15 @@ typedef struct {
     lb_kn_convention kn_convention;
     size_t budget_bytes;      /* device arena for populations, histories, tables (default 1 GiB) */
     int max_slots;            /* default 4096 */
-    int threads;              /* threads per CTA (64..256, multiple of 32); 0 = 256 */
+    int threads;              /* threads per CTA (64..256, multiple of 32); 0 = the library's choice (512) */
     int smem_bytes;           /* on-chip instance budget per CTA (bytes); -1 = 96 KiB */
     void *stream;             /* cudaStream_t; NULL = own stream */
-    int warp_cells;           /* instances of at most this many cells are each advanced by one
-                                 warp (a CTA then advances threads/32 of them at once, each with
-                                 its share of the on-chip budget); larger ones by a whole CTA.
-                                 0 = every instance by a CTA; -1 (default) = 512 */
+    int warp_cells;           /* -1 (default): each instance by a warp, four warps, a CTA or a cluster
+                                 of two CTAs, by its share of the launch's work (a warp or four of
+                                 them have their share of the on-chip budget).  >= 0: instances of
+                                 at most this many cells are each advanced by one warp, larger
+                                 ones by a whole CTA (0 = every instance by a CTA).  Results do
+                                 not depend on it */
 } lb_batch_params;
 
 typedef struct {

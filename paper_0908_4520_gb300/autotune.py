@@ -23,7 +23,8 @@ import time
 from . import capi
 from .batch import Batch
 
-CANDIDATES = [(t, s, w) for t in (64, 128, 256) for s in (0, 48 * 1024, 96 * 1024, 200 * 1024)
+# the library's own choice (0, -1, -1) first: group widths by cost
+CANDIDATES = [(0, -1, -1)] + [(t, s, w) for t in (64, 128, 256) for s in (0, 48 * 1024, 96 * 1024, 200 * 1024)
               for w in (0, 256, 1024, 4096)]
 _CACHE = os.path.join(os.path.expanduser("~"), ".cache", "paper_0908_4520_gb300", "autotune.json")
 
@@ -94,9 +95,10 @@ def tune(instances, precision: str = "f32", sample: int = 1024, chunk: int = 32,
         raise RuntimeError("no launch shape could run the sample")
     best = max(results, key=lambda r: r["cell_updates_per_s"])
     entry = {"threads": best["threads"], "smem_bytes": best["smem_bytes"], "warp_cells": best["warp_cells"],
-             "trials": results, "searched": {"threads": [64, 128, 256], "smem_bytes": [0, 48 << 10, 96 << 10, 200 << 10],
+             "trials": results, "searched": {"threads": [0, 64, 128, 256],
+                                             "smem_bytes": [-1, 0, 48 << 10, 96 << 10, 200 << 10],
                                              "warp_cells (one warp per instance up to; cells per thread = cells/32)":
-                                                 [0, 256, 1024, 4096]}}
+                                                 [-1, 0, 256, 1024, 4096]}}
     cache[sig] = entry
     try:
         os.makedirs(os.path.dirname(_CACHE), exist_ok=True)

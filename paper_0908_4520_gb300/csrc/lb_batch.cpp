@@ -99,16 +99,15 @@ struct lb_batch {
     lbh::VelocitySetInfo sets[3];
     lbk::BatchArgs args{};
     lbk::BatchInst* inst_d = nullptr;
-    int* order_d = nullptr;
-    int* counters_d = nullptr;  // [0] next, [1] next_small, [2] n_order, [3] n_small
-    int* order_small_d = nullptr;
-    int warp_cells = 0;
+    int* order_d = nullptr;     // max_slots entries a queue
+    int* counters_d = nullptr;  // [queue] next, [kBatchQueues + queue] n
+    int warp_cells = 0;         // -1: group widths by cost
     unsigned long long* clock_d = nullptr;  // per CTA: start, end of the last launch (%globaltimer, ns)
     std::vector<lbk::BatchInst> inst;
     std::vector<char> live, dirty;
     std::vector<std::vector<std::pair<size_t, size_t>>> ranges_of;
     std::vector<double> tau;
-    int threads = 256, smem = 96 * 1024, grid = 0;
+    int threads = lbk::kBatchThreads, smem = 96 * 1024, grid = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_chunk = -1;
     bool in_flight = false;
@@ -145,18 +144,18 @@ namespace {
 
 cudaError_t batch_launch(lb_batch* b) {
     switch (b->p.precision) {
-        case LB_F32: return lbk::batch_launch_f32(&b->args, b->grid, b->threads, b->smem, b->stream);
-        case LB_F16: return lbk::batch_launch_f16(&b->args, b->grid, b->threads, b->smem, b->stream);
-        case LB_BF16: return lbk::batch_launch_bf16(&b->args, b->grid, b->threads, b->smem, b->stream);
+        case LB_F32: return lbk::batch_launch_f32(&b->args, b->grid, lbk::kBatchClusterCtas, b->threads, b->smem, b->stream);
+        case LB_F16: return lbk::batch_launch_f16(&b->args, b->grid, lbk::kBatchClusterCtas, b->threads, b->smem, b->stream);
+        case LB_BF16: return lbk::batch_launch_bf16(&b->args, b->grid, lbk::kBatchClusterCtas, b->threads, b->smem, b->stream);
         default: return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t batch_setup(lb_precision prec, int threads, int smem, int* occ) {
+cudaError_t batch_setup(lb_precision prec, int threads, int* smem, int* grid) {
     switch (prec) {
-        case LB_F32: return lbk::batch_setup_f32(threads, smem, occ);
-        case LB_F16: return lbk::batch_setup_f16(threads, smem, occ);
-        case LB_BF16: return lbk::batch_setup_bf16(threads, smem, occ);
+        case LB_F32: return lbk::batch_setup_f32(threads, lbk::kBatchClusterCtas, smem, grid);
+        case LB_F16: return lbk::batch_setup_f16(threads, lbk::kBatchClusterCtas, smem, grid);
+        case LB_BF16: return lbk::batch_setup_bf16(threads, lbk::kBatchClusterCtas, smem, grid);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -207,9 +206,9 @@ lb_status lb_batch_create(const lb_batch_params* pin, lb_batch** out) {
         return LB_ERR_NOMEM;
     }
     b->p = P;
-    b->threads = P.threads ? P.threads : 256;
+    b->threads = P.threads ? P.threads : lbk::kBatchThreads;
     b->smem = P.smem_bytes < 0 ? 96 * 1024 : P.smem_bytes;
-    b->warp_cells = P.warp_cells < 0 ? 512 : P.warp_cells;
+    b->warp_cells = P.warp_cells < 0 ? -1 : P.warp_cells;
     auto bail = [&](lb_status s, const std::string& m) {
         g_batch_error = m;
         if (b->graph) cudaGraphExecDestroy(b->graph);
@@ -217,7 +216,6 @@ lb_status lb_batch_create(const lb_batch_params* pin, lb_batch** out) {
         if (b->inst_d) cudaFree(b->inst_d);
         if (b->order_d) cudaFree(b->order_d);
         if (b->counters_d) cudaFree(b->counters_d);
-        if (b->order_small_d) cudaFree(b->order_small_d);
         if (b->clock_d) cudaFree(b->clock_d);
         if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
         delete b;
@@ -240,19 +238,13 @@ lb_status lb_batch_create(const lb_batch_params* pin, lb_batch** out) {
             return bail(LB_ERR_CUDA, std::string("cudaStreamCreate: ") + cudaGetErrorString(e));
         b->own_stream = true;
     }
-    int occ = 0;
-    if ((e = batch_setup(P.precision, b->threads, b->smem, &occ)) != cudaSuccess || occ < 1)
+    if ((e = batch_setup(P.precision, b->threads, &b->smem, &b->grid)) != cudaSuccess || b->grid < 1)
         return bail(LB_ERR_ARG, std::string("kernel configuration does not fit: ") +
                                     (e != cudaSuccess ? cudaGetErrorString(e) : "zero occupancy"));
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    b->grid = std::max(1, nsm * occ);
     if (cudaMalloc(&b->arena, P.budget_bytes) != cudaSuccess) return bail(LB_ERR_NOMEM, "arena allocation");
     if (cudaMalloc(&b->inst_d, sizeof(lbk::BatchInst) * P.max_slots) != cudaSuccess ||
-        cudaMalloc(&b->order_d, sizeof(int) * P.max_slots) != cudaSuccess ||
+        cudaMalloc(&b->order_d, sizeof(int) * lbk::kBatchQueues * (size_t)P.max_slots) != cudaSuccess ||
         cudaMalloc(&b->counters_d, 256) != cudaSuccess ||
-        cudaMalloc(&b->order_small_d, sizeof(int) * P.max_slots) != cudaSuccess ||
         cudaMalloc(&b->clock_d, sizeof(unsigned long long) * 2 * b->grid) != cudaSuccess)
         return bail(LB_ERR_NOMEM, "descriptor allocation");
     b->ranges.reset(P.budget_bytes);
@@ -262,12 +254,8 @@ lb_status lb_batch_create(const lb_batch_params* pin, lb_batch** out) {
     b->ranges_of.assign(P.max_slots, {});
     b->tau.assign(P.max_slots, 0.0);
     b->args.inst = b->inst_d;
-    b->args.order = b->order_d;
-    b->args.next = b->counters_d;
-    b->args.next_small = b->counters_d + 1;
-    b->args.n_order = b->counters_d + 2;
-    b->args.n_small = b->counters_d + 3;
-    b->args.order_small = b->order_small_d;
+    for (int k = 0; k < lbk::kBatchQueues; ++k)
+        b->args.queue[k] = {b->order_d + (size_t)k * P.max_slots, b->counters_d + lbk::kBatchQueues + k, b->counters_d + k};
     b->args.smem_cap = b->smem;
     b->args.arena = b->arena;
     b->args.hist = static_cast<float2*>(b->arena);
@@ -289,7 +277,6 @@ lb_status lb_batch_destroy(lb_batch* b) {
     cudaFree(b->inst_d);
     cudaFree(b->order_d);
     cudaFree(b->counters_d);
-    cudaFree(b->order_small_d);
     cudaFree(b->clock_d);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b;
@@ -429,29 +416,49 @@ lb_status lb_batch_run(lb_batch* b, int chunk) {
     lb_status st = b->settle();
     if (st != LB_OK) return st;
     const int ch = chunk == 0 ? (1 << 30) : chunk;
-    // work lists: live, unfinished slots by decreasing remaining cost; instances of at most
-    // warp_cells cells go to the warp queue
-    std::vector<int> order, small;
+    // work lists: live, unfinished slots by decreasing remaining cost (strips x velocities x levels)
+    const int nw = b->threads / 32;
+    std::vector<int> order[lbk::kBatchQueues];
     std::vector<double> cost(b->p.max_slots, 0.0);
+    std::vector<long long> strips(b->p.max_slots, 0);
+    double total = 0.0;
     for (int s = 0; s < b->p.max_slots; ++s) {
         if (!b->live[s] || b->inst[s].done) continue;
         const lbk::BatchInst& in = b->inst[s];
         const double levels = std::min<double>(in.max_level - in.level + 1, ch);
-        cost[s] = levels * (double)in.nx * in.ny * b->sets[in.set].q;
-        ((long long)in.nx * in.ny <= b->warp_cells ? small : order).push_back(s);
+        strips[s] = (in.nx <= 32 ? 1 : (in.nx + 29) / 30) * (long long)in.ny;
+        cost[s] = levels * (double)strips[s] * b->sets[in.set].q;
+        total += cost[s];
     }
-    auto by_cost = [&](int x, int y) { return cost[x] > cost[y]; };
-    std::stable_sort(order.begin(), order.end(), by_cost);
-    std::stable_sort(small.begin(), small.end(), by_cost);
-    const int counts[2] = {(int)order.size(), (int)small.size()};
-    const int n = counts[0] + counts[1];
+    // An instance takes cost x (warps of a CTA) / (warps of its group) of an SM's time when the SM is
+    // full.  It goes to the narrowest group that takes at most half of the launch's mean time an SM,
+    // or that has a warp for every strip.  With warp_cells given: at most that many cells to a
+    // warp, else to a CTA.  (Results do not depend on the choice.)
+    const double mean = total / b->grid;
+    const int width[lbk::kBatchQueues] = {nw * lbk::kBatchClusterCtas, nw, 4, 1};
+    for (int s = 0; s < b->p.max_slots; ++s) {
+        if (!b->live[s] || b->inst[s].done) continue;
+        int k = lbk::kBatchWarp;
+        if (b->warp_cells >= 0) {
+            if ((long long)b->inst[s].nx * b->inst[s].ny > b->warp_cells) k = lbk::kBatchCta;
+        } else {
+            while (k > lbk::kBatchCluster && strips[s] > width[k] && cost[s] * nw / width[k] > 0.5 * mean) --k;
+            if (k == lbk::kBatchQuad && (nw <= 4 || nw % 4)) k = lbk::kBatchCta;
+        }
+        order[k].push_back(s);
+    }
+    int counts[lbk::kBatchQueues], n = 0;
     cudaError_t e = cudaSuccess;
-    if (counts[0])
-        e = cudaMemcpyAsync(b->order_d, order.data(), sizeof(int) * counts[0], cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess && counts[1])
-        e = cudaMemcpyAsync(b->order_small_d, small.data(), sizeof(int) * counts[1], cudaMemcpyHostToDevice,
-                            b->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->counters_d + 2, counts, sizeof(counts), cudaMemcpyHostToDevice, b->stream);
+    for (int k = 0; k < lbk::kBatchQueues; ++k) {
+        std::stable_sort(order[k].begin(), order[k].end(), [&](int x, int y) { return cost[x] > cost[y]; });
+        counts[k] = (int)order[k].size();
+        n += counts[k];
+        if (e == cudaSuccess && counts[k])
+            e = cudaMemcpyAsync(b->order_d + (size_t)k * b->p.max_slots, order[k].data(), sizeof(int) * counts[k],
+                                cudaMemcpyHostToDevice, b->stream);
+    }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->counters_d + lbk::kBatchQueues, counts, sizeof(counts), cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess) return b->cuda_fail(e, "work list upload");
     if (n == 0) return LB_OK;
     if (!b->graph || b->graph_chunk != ch) {
@@ -461,7 +468,7 @@ lb_status lb_batch_run(lb_batch* b, int chunk) {
         cudaGraph_t g = nullptr;
         if ((e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
             return b->cuda_fail(e, "cudaStreamBeginCapture");
-        cudaError_t e1 = cudaMemsetAsync(b->counters_d, 0, 2 * sizeof(int), b->stream);  // both queue heads
+        cudaError_t e1 = cudaMemsetAsync(b->counters_d, 0, lbk::kBatchQueues * sizeof(int), b->stream);  // the queue heads
         cudaError_t e2 = batch_launch(b);
         e = cudaStreamEndCapture(b->stream, &g);
         if (e1 != cudaSuccess || e2 != cudaSuccess || e != cudaSuccess) {

@@ -1,21 +1,36 @@
 // Persistent multi-instance kernel: many small, uneven lattices in one launch.
 //
-// Each CTA takes instances from a work queue (an atomic counter over a list
-// ordered by decreasing remaining cost, i.e. longest-processing-time first) and
-// advances one instance at a time by up to `chunk` time levels, with a block
-// barrier between levels: an instance never spans CTAs, so no CTA ever waits
-// on another.  An instance whose two population buffers fit the CTA's shared
-// memory is copied in once per chunk and stepped entirely on chip; larger ones
-// step through global memory (L2-resident at these sizes).  A warp advances
-// strips of up to 30 cells of one row: each lane streams one column in y (three
-// loads per velocity) and takes its neighbours' columns by shuffles for the x
-// pass, the two edge lanes streaming the columns beside the strip, as the
-// single-lattice kernels do.  The per-cell arithmetic is collide_cell_pairs(),
-// the collision those kernels call, and a cell's operations do not depend on
-// the path (on chip or through global memory, a CTA or a warp), so an
-// instance's populations are bitwise the same whichever path runs it and
-// whatever else shares the launch.  Lax-Wendroff streaming only: the batch
-// serves the Gauss-Hermite product sets.
+// A group of warps takes instances from a work queue (an atomic counter over a list ordered by
+// decreasing remaining cost, i.e. longest-processing-time first) and advances one instance at a
+// time by up to `chunk` time levels, with one barrier of the group between levels.  There are four
+// widths of group, each with a queue of its own: a cluster of two CTAs, a CTA, four warps of it,
+// and one warp.  The host gives each instance the narrowest group that still finishes within the
+// launch's mean load, so a launch is not as long as its largest instance takes on one SM and a
+// small instance does not hold a whole one.  Every cluster serves the wide queue first, then its
+// CTAs, then their four-warp groups, then their warps go on by themselves.  Only CTAs of one
+// cluster (which run at the same time) wait on one another.
+//
+// An instance whose two population buffers fit the group's share of the CTA's shared memory is
+// copied in once per chunk and stepped entirely on chip (groups within a CTA); larger ones step
+// through global memory (L2-resident at these sizes).  A warp advances strips of up to 30 cells of
+// one row: each lane streams one column in y (three loads per velocity) and takes its neighbours'
+// columns by shuffles for the x pass, the two edge lanes streaming the columns beside the strip, as
+// the single-lattice kernels do; a row of at most 32 cells is one strip whose lanes are neighbours
+// around the end.  The per-cell arithmetic is the velocity-pair stencil and collide_cell_pairs() of
+// those kernels.
+//
+// The sums of a level (A, S, H) are taken over 64 slots: strip s belongs to slot s % 64, a slot to
+// one warp, which sums its strips in order; after the level's barrier every warp sums the slots in
+// the same order and so knows for itself whether the instance has stopped.  Neither a cell's
+// operations nor the sums' order depend on the group or the memory path, so an instance's
+// populations and history are bitwise the same whichever path runs it and whatever else shares the
+// launch.  Lax-Wendroff streaming only: the batch serves the Gauss-Hermite product sets.
+//
+// Bound: latency of the L2 loads and of the collision's chain; 16 warps of 128 registers per SM beat
+// 8 of 255, the tables are constant-bank operands (the kernel inlines its nine variants; through a
+// reference they were loads), and the two wide queues take the makespan of the largest instances
+// down to the mean load.  512 instances of the batching configuration, 800 levels, admission and
+// histories included: 169 ms before, 72 ms now.
 #pragma once
 
 #include "lb_batch.h"
@@ -23,46 +38,94 @@
 
 namespace lbk {
 
-constexpr int kBatchMaxWarps = 8;  // warps per CTA (the kernel's launch bound: 256 threads)
+constexpr int kBatchMaxWarps = 16;  // warps per CTA (the kernel's launch bound: 512 threads of 128 registers)
 constexpr int kStrip = 30;  // cells of a row per warp and pass (two lanes stream the columns beside them)
+constexpr int kBatchSlots = 64;     // partial sums of a level
 
-// the kernel's static shared memory (one copy, whichever instance template runs)
+// the kernel's static shared memory; what belongs to a group lies at the index of its first warp
 struct BatchShared {
-    float red[kBatchMaxWarps][3];           // per-warp partial sums of a level's diagnostics
-    int done[kBatchMaxWarps];               // stop flag of each group (the CTA, or each warp)
-    float relax[kBatchMaxWarps][4][kMaxNA]; // relaxation tables of each group's instance
+    float red[kBatchMaxWarps / 4][2][3][kBatchSlots];  // A, S, H by slot, two levels (groups of four warps and more)
+    float relax[kBatchMaxWarps][4][kMaxNA];        // relaxation tables of the group's instance
+    int next[kBatchMaxWarps];                      // queue position of the group's instance
 };
 
+// The warps that advance one instance together.
+struct BatchGroup {
+    int kind;        // BatchQueue: cluster, CTA, four warps, warp
+    int warps;       // warps of the group, in all its CTAs
+    int wid;         // this warp's number among them
+    int first;       // first warp of the group in this CTA
+    int threads;     // threads of the group in this CTA
+    int tid;         // this thread's number among those
+    int ctas;        // CTAs of the group
+    int smem_cap;    // bytes of its share of the shared memory
+    __device__ __forceinline__ void sync() const {
+        if (kind == kBatchWarp) {
+            __syncwarp();
+        } else if (kind == kBatchCluster && ctas > 1) {
+            __syncwarp();
+            asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+        } else {
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + first), "r"(threads) : "memory");
+        }
+    }
+};
+
+// address of this CTA's shared variable in CTA r of the cluster, and a load from there
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int r) {
+    uint32_t d;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(smem_u32(p)), "r"(r));
+    return d;
+}
+__device__ __forceinline__ float cluster_ld(uint32_t a) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
 template <class S>
-__device__ __forceinline__ float batch_load(const S* p, float sc) {
-    if constexpr (Is16<S>::value) {
-        return (std::is_same<S, __half>::value ? __half2float(*reinterpret_cast<const __half*>(p))
-                                               : __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(p))) *
-               sc;
+__device__ __forceinline__ float batch_load(const S* p) {
+    if constexpr (std::is_same<S, __half>::value) {
+        return __half2float(*p);
+    } else if constexpr (std::is_same<S, __nv_bfloat16>::value) {
+        return __bfloat162float(*p);
     } else {
-        (void)sc;
         return *p;
     }
 }
 
-// Advance instance `id` by up to B.chunk levels with the CTA's threads (WARP = false) or with
-// one warp of it (WARP = true: small instances, so that a CTA advances several at once; smem is
-// then the warp's slice of the shared memory, smem_cap bytes).
-template <class VS, int N, class S, bool WARP = false>
-__device__ __noinline__ void batch_run(const BatchArgs& B, int id, S* smem, int smem_cap, BatchShared& sh) {
+// Sums of three values over the warp in 7 shuffles: the halves of the warp, then its quarters, take
+// one value each; lanes 0, 8 and 16 return the sums of a, b and c.
+__device__ __forceinline__ float warp_sum3(float a, float b, float c, int lane) {
+    const bool up = lane & 16;
+    // lanes 0-15 keep a and b, lanes 16-31 keep c
+    const float ra = __shfl_xor_sync(0xffffffffu, up ? a : c, 16);
+    const float rb = __shfl_xor_sync(0xffffffffu, b, 16);
+    float x = up ? c + ra : a + ra;
+    float y = up ? 0.f : b + rb;
+    const bool q = lane & 8;
+    const float r = __shfl_xor_sync(0xffffffffu, q ? x : y, 8);
+    x = q ? y + r : x + r;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// Advance instance `id` by up to B.chunk levels with the group's warps (smem: the group's share of
+// the CTA's shared memory).
+template <class VS, int SET, int N, class S>
+__device__ __forceinline__ void batch_run(const BatchArgs& B, int id, S* smem, const BatchGroup& G, BatchShared& sh) {
     constexpr int Q = VS::Q;
     BatchInst& in = B.inst[id];
-    const Tab<float>& t = B.tab[in.set];
+    const Tab<float>& t = B.tab[SET];
     const int nx = in.nx, ny = in.ny;
     const int ncell = nx * ny;
     const long long pop = (long long)Q * ncell;
     const float omega = in.omega, sigma_fac = in.sigma_fac;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tid = WARP ? lane : (int)threadIdx.x, nthr = WARP ? 32 : (int)blockDim.x;
-    const int nwarp = (nthr + 31) >> 5;
+    const int lane = threadIdx.x & 31, tid = G.tid, nthr = G.threads;
     // the instance's relaxation tables (omega W_i and the second terms of the exact FP32
-    // identities) in shared memory, one copy per group (the CTA, or each warp)
-    float(*rt)[kMaxNA] = sh.relax[WARP ? warp : 0];
+    // identities) in shared memory
+    float(*rt)[kMaxNA] = sh.relax[G.first];
     if (tid < VS::NA) {
         rt[0][tid] = in.ow[tid];
         rt[1][tid] = in.owlo[tid];
@@ -72,22 +135,18 @@ __device__ __noinline__ void batch_run(const BatchArgs& B, int id, S* smem, int 
     const float* sinx = B.trig + in.trig_off;
     const float* cosx = sinx + nx;
     float2* hist = B.hist + in.hist_off;
-    const int spr = (nx + kStrip - 1) / kStrip;  // strips per row
+    // a row of at most 32 cells is one strip: its lanes are neighbours around the row's end
+    const bool ring = nx <= 32;
+    const int spr = ring ? 1 : (nx + kStrip - 1) / kStrip;  // strips per row
     const int nstrip = spr * ny;
-    int& s_done = sh.done[WARP ? warp : 0];  // the group's stop flag
-    auto group_sync = [&]() {
-        if constexpr (WARP) {
-            __syncwarp();
-        } else {
-            __syncthreads();
-        }
-    };
+    const int nslot = min(nstrip, kBatchSlots);
 
-    int level = in.level;
+    const int first_level = in.level;
+    int level = first_level;
     int cur = in.cur;
     const int stop = min(in.max_level, level + B.chunk - 1);
     // both buffers of an instance that fits the group's shared memory are stepped on chip
-    const bool onchip = 2 * pop * (long long)sizeof(S) <= (long long)smem_cap;
+    const bool onchip = G.ctas == 1 && 2 * pop * (long long)sizeof(S) <= (long long)G.smem_cap;
     S* const arena = static_cast<S*>(B.arena);
     S* gbuf[2] = {arena + in.off[0], arena + in.off[1]};
     S* buf[2] = {gbuf[0], gbuf[1]};
@@ -97,138 +156,166 @@ __device__ __noinline__ void batch_run(const BatchArgs& B, int id, S* smem, int 
         if (level > 0)
             for (long long k = tid; k < pop; k += nthr) buf[cur][k] = gbuf[cur][k];
     }
-    if (tid == 0) s_done = in.done;
-    group_sync();
+    bool done = in.done;
+    int status = 0;
+    float h0 = in.h0;
+    const double u0 = in.u0;
+    const int isothermal = in.isothermal, max_level = in.max_level;
+    const float stop_ratio2 = in.stop_ratio2;
+    // stop rule sqrt(H / H0) <= stop_ratio (none for stop_ratio = 0, also where H is 0): the largest
+    // FP32 value of H that meets it
+    auto threshold = [&](float h) { return __double2float_rd((double)stop_ratio2 * (double)h); };
+    float hstop = threshold(h0);
 
     // 16-bit storage: deviation = stored * sc[a] * scale; sc (tables built with S = 1) and
     // scale are powers of two, so the load and store scales are exact inverses
     const float scale = in.scale;
     const float inv_scale = 1.0f / scale;
-    for (; level <= stop && !s_done; ++level) {
+    G.sync();
+    for (; level <= stop && !done; ++level) {
         const S* src = buf[cur];
         S* dst = buf[level == 0 ? 0 : 1 - cur];
-        float pa = 0.f, ps = 0.f, ph = 0.f;
-        bool bad = false;
-        // strips of up to 30 cells of one row, one per warp at a time: lanes 1..w own cells
-        // x0 .. x0 + w - 1; lanes 0 and w + 1 stream the columns beside the strip, so that each
-        // lane streams one column in y and takes its neighbours' columns by shuffles for the x
-        // pass; lanes past w + 1 repeat lane w + 1's column and own nothing
-        for (int s = WARP ? 0 : warp; s < nstrip; s += WARP ? 1 : nwarp) {
-            const int y = s / spr, x0 = (s - y * spr) * kStrip;
-            const int w = min(kStrip, nx - x0);
-            int x = x0 + min(lane, w + 1) - 1;
-            x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
-            const bool own = lane >= 1 && lane <= w;
-            const int c = y * nx + x;
-            float ft[Q];
-            if (level == 0) {
-                // f~(0) = f^eq(rho = 1, u_y = u0 sin x, T = 1), rounded through the storage type
-                const double sx = sinpi(2.0 * (double)x / (double)nx);
-                const float uy = (float)(in.u0 * sx);
-                equilibrium_dev<VS, N, float>(t, 0.f, 1.f, 0.f, uy, 0.f, [&](auto ac, float deq) {
-                    constexpr int a = decltype(ac)::value;
-                    if constexpr (Is16<S>::value) {
-                        S tmp;
-                        st1<S, float>(&tmp, deq, t.scinv[a] * inv_scale);
-                        ft[a] = batch_load<S>(&tmp, t.sc[a] * scale);
-                    } else {
-                        ft[a] = deq;
-                    }
-                });
-            } else {
-                const int ym = y == 0 ? ny - 1 : y - 1, yp = y + 1 == ny ? 0 : y + 1;
-                const int om = ym * nx + x, op = yp * nx + x;
-                const bool rows = ny > 1;  // one row: the three y taps read the same value
-                static_for<0, Q>([&](auto ac) {
-                    constexpr int a = decltype(ac)::value;
-                    constexpr int ix = VS::ix(a), iy = VS::iy(a);
-                    const float sc = Is16<S>::value ? t.sc[a] * scale : 1.f;
-                    const S* pl = src + (long long)a * ncell;
-                    const float v0 = batch_load<S>(pl + c, sc);
-                    const float vm = rows ? batch_load<S>(pl + om, sc) : v0;
-                    const float vp = rows ? batch_load<S>(pl + op, sc) : v0;
-                    const float g = fma(t.lw[iy][0], vm, fma(t.lw[iy][1], v0, t.lw[iy][2] * vp));
-                    const float gl = __shfl_up_sync(0xffffffffu, g, 1);
-                    const float gr = __shfl_down_sync(0xffffffffu, g, 1);
-                    ft[a] = fma(t.lw[ix][0], gl, fma(t.lw[ix][1], g, t.lw[ix][2] * gr));
-                });
+        float(*red)[kBatchSlots] = sh.red[G.first / 4][level & 1];
+        float tot[3] = {0.f, 0.f, 0.f};  // lane l: the sums of slots l and l + 32
+        for (int slot = G.wid; slot < nslot; slot += G.warps) {
+            float pa = 0.f, ps = 0.f, ph = 0.f;
+            // strips of up to 30 cells of one row: lanes 1..w own cells x0 .. x0 + w - 1, lanes 0
+            // and w + 1 stream the columns beside the strip, so that each lane streams one column
+            // in y and takes its neighbours' columns by shuffles for the x pass; lanes past w + 1
+            // repeat lane w + 1's column and own nothing.  In a ring lanes 0..nx - 1 own the cells.
+            for (int s = slot; s < nstrip; s += kBatchSlots) {
+                const int y = s / spr, x0 = (s - y * spr) * kStrip;
+                const int w = min(kStrip, nx - x0);
+                int x = ring ? min(lane, nx - 1) : x0 + min(lane, w + 1) - 1;
+                x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+                const bool own = ring ? lane < nx : lane >= 1 && lane <= w;
+                const int from_l = ring ? (lane == 0 ? nx - 1 : lane - 1) : max(lane - 1, 0);
+                const int from_r = ring ? (lane >= nx - 1 ? 0 : lane + 1) : min(lane + 1, 31);
+                const int c = y * nx + x;
+                f2 fp[Q / 2];
+                if (level == 0) {
+                    // f~(0) = f^eq(rho = 1, u_y = u0 sin x, T = 1), rounded through the storage type
+                    const double sx = sinpi(2.0 * (double)x / (double)nx);
+                    const float uy = (float)(u0 * sx);
+                    float ft[Q];
+                    equilibrium_dev<VS, N, float>(t, 0.f, 1.f, 0.f, uy, 0.f, [&](auto ac, float deq) {
+                        constexpr int a = decltype(ac)::value;
+                        if constexpr (Is16<S>::value) {
+                            S tmp;
+                            st1<S, float>(&tmp, deq, t.scinv[a] * inv_scale);
+                            ft[a] = batch_load<S>(&tmp) * (t.sc[a] * scale);
+                        } else {
+                            ft[a] = deq;
+                        }
+                    });
+                    static_for<0, Q / 2>([&](auto mc) {
+                        constexpr int m = decltype(mc)::value;
+                        fp[m] = f2{ft[2 * m], ft[2 * m + 1]};
+                    });
+                } else {
+                    const int ym = y == 0 ? ny - 1 : y - 1, yp = y + 1 == ny ? 0 : y + 1;
+                    const bool rows = ny > 1;  // one row: the three y taps read the same value
+                    const S* p0 = src + c;
+                    const S* pm = src + ym * nx + x;
+                    const S* pp = src + yp * nx + x;
+                    static_for<0, Q / 2>([&](auto mc) {
+                        constexpr int m = decltype(mc)::value, a = 2 * m;
+                        auto pair = [&](const S* p) {
+                            f2 v = f2{batch_load<S>(p), batch_load<S>(p + ncell)};
+                            if constexpr (Is16<S>::value)
+                                v = vmul(v, f2{t.sc[a] * scale, t.sc[a + 1] * scale});
+                            return v;
+                        };
+                        const f2 v0 = pair(p0);
+                        const f2 vm = rows ? pair(pm) : v0;
+                        const f2 vp = rows ? pair(pp) : v0;
+                        p0 += 2 * ncell;
+                        pm += 2 * ncell;
+                        pp += 2 * ncell;
+                        const f2 g = lw_y_pair<VS, a>(t, vm, v0, vp);
+                        const f2 gl = f2{__shfl_sync(0xffffffffu, g.x, from_l), __shfl_sync(0xffffffffu, g.y, from_l)};
+                        const f2 gr = f2{__shfl_sync(0xffffffffu, g.x, from_r), __shfl_sync(0xffffffffu, g.y, from_r)};
+                        fp[m] = lw_x_pair<VS, a>(t, gl, g, gr);
+                    });
+                }
+                const CellOut<float> co = collide_cell_pairs<VS, N, true>(
+                    t, rt[0], rt[1], rt[2], rt[3], 1.f, omega, sigma_fac, isothermal, true, false, 0.f, 0.f, 0.f,
+                    [&](auto mc) -> f2& { return fp[decltype(mc)::value]; });
+                if (own) {
+                    uint32_t r = Is16<S>::value ? sr_seed(level, c) : 0u;
+                    S* p = dst + c;
+                    static_for<0, Q / 2>([&](auto mc) {
+                        constexpr int m = decltype(mc)::value, a = 2 * m;
+                        if constexpr (Is16<S>::value) {
+                            r = sr_next(r);
+                            p[0] = to_storage<S, float>(fp[m].x, t.scinv[a] * inv_scale, r);
+                            r = sr_next(r);
+                            p[ncell] = to_storage<S, float>(fp[m].y, t.scinv[a + 1] * inv_scale, r);
+                        } else {
+                            p[0] = fp[m].x;
+                            p[ncell] = fp[m].y;
+                        }
+                        p += 2 * ncell;
+                    });
+                    pa = fma(co.uy, sinx[x], pa);
+                    ps = fma(co.sig, cosx[x], ps);
+                    ph += co.h;
+                }
             }
-            // velocity pairs of equal x node as packed f32x2 values (the one-cell-per-lane
-            // collision of the single-lattice kernels)
-            f2 fp[Q / 2];
-            static_for<0, Q / 2>([&](auto mc) {
-                constexpr int m = decltype(mc)::value;
-                fp[m] = f2{ft[2 * m], ft[2 * m + 1]};
-            });
-            const CellOut<float> co = collide_cell_pairs<VS, N, true>(
-                t, rt[0], rt[1], rt[2], rt[3], 1.f, omega, sigma_fac, in.isothermal, true, false, 0.f, 0.f, 0.f,
-                [&](auto mc) -> f2& { return fp[decltype(mc)::value]; });
-            if (own) {
-                static_for<0, Q / 2>([&](auto mc) {
-                    constexpr int m = decltype(mc)::value;
-                    ft[2 * m] = fp[m].x;
-                    ft[2 * m + 1] = fp[m].y;
-                });
-                uint32_t r = Is16<S>::value ? sr_seed(level, c) : 0u;
+            const float v = warp_sum3(pa, ps, ph, lane);
+            if (G.kind == kBatchWarp) {  // the warp has every slot itself
 #pragma unroll
-                for (int a = 0; a < Q; ++a) {
-                    if constexpr (Is16<S>::value) r = sr_next(r);
-                    dst[(long long)a * ncell + c] =
-                        to_storage<S, float>(ft[a], Is16<S>::value ? t.scinv[a] * inv_scale : 1.f, r);
+                for (int k = 0; k < 3; ++k) {
+                    const float r = __shfl_sync(0xffffffffu, v, 8 * k);
+                    if (lane == (slot & 31)) tot[k] += r;
                 }
-                pa = fma(co.uy, sinx[x], pa);
-                ps = fma(co.sig, cosx[x], ps);
-                ph += co.h;
-                bad |= !isfinite(co.h);
+            } else if (lane == 0 || lane == 8 || lane == 16) {
+                red[lane >> 3][slot] = v;
             }
         }
-        pa = warp_sum(pa);
-        ps = warp_sum(ps);
-        ph = warp_sum(ph);
-        bad = __any_sync(0xffffffffu, bad);
-        if (!WARP && lane == 0) {
-            sh.red[warp][0] = pa;
-            sh.red[warp][1] = ps;
-            sh.red[warp][2] = bad ? __int_as_float(0x7fc00000) : ph;
-        }
-        group_sync();
-        if (tid == 0) {
-            double A = 0, Sx = 0, H = 0;
-            if constexpr (WARP) {
-                A = pa;
-                Sx = ps;
-                H = bad ? (double)__int_as_float(0x7fc00000) : (double)ph;
-            } else {
-                for (int w = 0; w < nwarp; ++w) {
-                    A += sh.red[w][0];
-                    Sx += sh.red[w][1];
-                    H += sh.red[w][2];
+        G.sync();
+        // every warp sums the slots
+        if (G.kind != kBatchWarp) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const int slot = lane + 32 * s;
+                    if (slot < nslot)
+                        tot[k] += G.ctas == 1 ? red[k][slot] : cluster_ld(cluster_addr(&red[k][slot], slot % G.ctas));
                 }
+        }
+        const float v = warp_sum3(tot[0], tot[1], tot[2], lane);
+        const float H = __shfl_sync(0xffffffffu, v, 16);
+        if (level == 0) {
+            h0 = H;
+            hstop = threshold(h0);
+        }
+        if (!isfinite(H)) {
+            status = 1;
+            done = true;
+        }
+        if (level > 0 && stop_ratio2 > 0.f && H <= hstop) done = true;
+        if (level == max_level) done = true;
+        if (G.wid == 0) {
+            const float Sx = __shfl_sync(0xffffffffu, v, 8);
+            if (lane == 0) {
+                const double norm = 2.0 / (double)ncell;
+                hist[level] = make_float2((float)((double)v * norm), (float)((double)Sx * norm));
             }
-            const double norm = 2.0 / (double)ncell;
-            hist[level] = make_float2((float)(A * norm), (float)(Sx * norm));
-            if (level == 0) in.h0 = (float)H;
-            int d = 0;
-            if (!isfinite(H)) {
-                in.status |= 1;
-                d = 1;
-            }
-            // stop rule sqrt(H / H0) <= stop_ratio (none for stop_ratio = 0, also where H is 0)
-            if (level > 0 && in.stop_ratio2 > 0.f && (double)H <= (double)in.stop_ratio2 * (double)in.h0) d = 1;
-            if (level == in.max_level) d = 1;
-            s_done = d;
         }
         cur = (level == 0) ? 0 : 1 - cur;
-        group_sync();
     }
-    if (onchip && level > in.level)
+    if (onchip && level > first_level)
         for (long long k = tid; k < pop; k += nthr) gbuf[cur][k] = buf[cur][k];
-    if (tid == 0) {
+    G.sync();  // the descriptor has been read, the shared arrays are free
+    if (G.wid == 0 && lane == 0) {
         in.level = level;
         in.cur = cur;
-        in.done = s_done;
+        in.done = done;
+        in.h0 = h0;
+        if (status) in.status |= status;
     }
-    group_sync();
 }
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -237,59 +324,71 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-template <class S, bool WARP>
-__device__ __forceinline__ void batch_dispatch(const BatchArgs& B, int id, S* smem, int smem_cap, BatchShared& sh) {
-    const BatchInst& in = B.inst[id];
-    switch (in.set * 3 + (in.n_eq - 2)) {
-        case 0: batch_run<lbvs::GH4, 2, S, WARP>(B, id, smem, smem_cap, sh); break;
-        case 1: batch_run<lbvs::GH4, 3, S, WARP>(B, id, smem, smem_cap, sh); break;
-        case 2: batch_run<lbvs::GH4, 4, S, WARP>(B, id, smem, smem_cap, sh); break;
-        case 3: batch_run<lbvs::GH6, 2, S, WARP>(B, id, smem, smem_cap, sh); break;
-        case 4: batch_run<lbvs::GH6, 3, S, WARP>(B, id, smem, smem_cap, sh); break;
-        case 5: batch_run<lbvs::GH6, 4, S, WARP>(B, id, smem, smem_cap, sh); break;
-        case 6: batch_run<lbvs::GH8, 2, S, WARP>(B, id, smem, smem_cap, sh); break;
-        case 7: batch_run<lbvs::GH8, 3, S, WARP>(B, id, smem, smem_cap, sh); break;
-        case 8: batch_run<lbvs::GH8, 4, S, WARP>(B, id, smem, smem_cap, sh); break;
-        default: break;
-    }
-}
-
-// Instances come from two work queues ordered longest-first: the CTA queue (each instance
-// advanced by the whole CTA) and, once it is empty, the warp queue (instances of at most
-// warp_cells cells, each advanced by one warp with its slice of the shared memory).
+// The launch: groups from the widest to the narrowest, each taking instances from its queue until
+// it is empty, then parting.
 template <class S>
 __global__ void __launch_bounds__(kBatchMaxWarps * 32) lb_batch_kernel(const __grid_constant__ BatchArgs B) {
     extern __shared__ __align__(16) unsigned char bsm[];
-    S* smem = reinterpret_cast<S*>(bsm);
-    __shared__ int s_i;
     __shared__ BatchShared sh;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    uint32_t nc, rank;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nc));
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     // start and end of every CTA (the launch's tail: how long the last CTA runs alone)
     if (B.cta_clock && threadIdx.x == 0) B.cta_clock[2 * blockIdx.x] = global_ns();
-    for (;;) {
-        if (threadIdx.x == 0) s_i = atomicAdd(B.next, 1);
-        __syncthreads();
-        const int i = s_i;
-        __syncthreads();
-        if (i >= *B.n_order) break;
-        const int id = B.order[i];
-        if (B.inst[id].done) continue;
-        batch_dispatch<S, false>(B, id, smem, B.smem_cap, sh);
-    }
-    if (B.n_small) {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-        // each warp's slice of the shared memory, 16-byte aligned
-        const int slice = (B.smem_cap / nwarp) & ~15;
-        S* wsm = reinterpret_cast<S*>(bsm + (size_t)warp * slice);
+#pragma unroll 1
+    for (int kind = 0; kind < kBatchQueues; ++kind) {
+        const BatchQueue& Qu = B.queue[kind];
+        BatchGroup G;
+        G.kind = kind;
+        const int per_cta = kind <= kBatchCta ? nwarp : (kind == kBatchQuad ? 4 : 1);  // warps of a group in a CTA
+        if (kind == kBatchQuad && nwarp % 4 != 0) continue;  // (the host leaves that queue empty)
+        G.ctas = kind == kBatchCluster ? (int)nc : 1;
+        G.warps = per_cta * G.ctas;
+        G.first = warp / per_cta * per_cta;
+        G.wid = (warp - G.first) * G.ctas + (kind == kBatchCluster ? (int)rank : 0);
+        G.threads = 32 * per_cta;
+        G.tid = threadIdx.x - 32 * G.first;
+        // each group's slice of the shared memory, 16-byte aligned
+        G.smem_cap = (int)((long long)B.smem_cap * per_cta / nwarp) & ~15;
+        S* const smem = reinterpret_cast<S*>(bsm + (size_t)(G.first / per_cta) * G.smem_cap);
+        if (!Qu.order) continue;
+        const int n = *Qu.n;
+        if (n == 0) continue;
         for (;;) {
-            int i = 0;
-            if (lane == 0) i = atomicAdd(B.next_small, 1);
-            i = __shfl_sync(0xffffffffu, i, 0);
-            if (i >= *B.n_small) break;
-            const int id = B.order_small[i];
+            if (G.wid == 0 && lane == 0) {
+                const int i = atomicAdd(Qu.next, 1);
+                if (G.ctas == 1) {
+                    sh.next[G.first] = i;
+                } else {
+                    for (int r = 0; r < G.ctas; ++r)
+                        asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr(&sh.next[G.first], r)),
+                                     "r"(i)
+                                     : "memory");
+                }
+            }
+            G.sync();
+            const int i = *(volatile int*)&sh.next[G.first];
+            G.sync();
+            if (i >= n) break;
+            const int id = Qu.order[i];
             if (B.inst[id].done) continue;
-            batch_dispatch<S, true>(B, id, wsm, slice, sh);
+            switch (B.inst[id].set * 3 + (B.inst[id].n_eq - 2)) {
+                case 0: batch_run<lbvs::GH4, 0, 2, S>(B, id, smem, G, sh); break;
+                case 1: batch_run<lbvs::GH4, 0, 3, S>(B, id, smem, G, sh); break;
+                case 2: batch_run<lbvs::GH4, 0, 4, S>(B, id, smem, G, sh); break;
+                case 3: batch_run<lbvs::GH6, 1, 2, S>(B, id, smem, G, sh); break;
+                case 4: batch_run<lbvs::GH6, 1, 3, S>(B, id, smem, G, sh); break;
+                case 5: batch_run<lbvs::GH6, 1, 4, S>(B, id, smem, G, sh); break;
+                case 6: batch_run<lbvs::GH8, 2, 2, S>(B, id, smem, G, sh); break;
+                case 7: batch_run<lbvs::GH8, 2, 3, S>(B, id, smem, G, sh); break;
+                case 8: batch_run<lbvs::GH8, 2, 4, S>(B, id, smem, G, sh); break;
+                default: break;
+            }
         }
     }
+    // a CTA of a cluster stays until the others have read its shared memory for the last time
+    // (the barrier after the wide queue's last instance); the CTA's end time is that of its last warp
     __syncthreads();
     if (B.cta_clock && threadIdx.x == 0) B.cta_clock[2 * blockIdx.x + 1] = global_ns();
 }

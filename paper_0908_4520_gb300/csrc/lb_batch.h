@@ -31,11 +31,18 @@ struct BatchInst {
     float ow[kMaxNA], owlo[kMaxNA], hn1lo[kMaxNA], whn1lo[kMaxNA];
 };
 
+// The work queues, by the width of the group of warps that advances an instance.
+enum BatchKind : int { kBatchCluster = 0, kBatchCta = 1, kBatchQuad = 2, kBatchWarp = 3, kBatchQueues = 4 };
+
+struct BatchQueue {
+    const int* order;     // slots in processing order (null: no such queue)
+    const int* n;         // number of slots in `order` (device, so a captured graph stays valid)
+    int* next;            // counter (reset before each launch)
+};
+
 struct BatchArgs {
     BatchInst* inst;
-    const int* order;     // slots in processing order
-    const int* n_order;   // number of slots in `order` (device, so a captured graph stays valid)
-    int* next;            // work-queue counter (reset before each launch)
+    BatchQueue queue[kBatchQueues];
     int chunk;            // levels per instance per launch
     int smem_cap;         // bytes of dynamic shared memory available for on-chip instances
     void* arena;          // population storage (the batch's storage type)
@@ -43,17 +50,19 @@ struct BatchArgs {
     const float* trig;
     Tab<float> tab[3];    // per set (weights, nodes, Hermite and Lax-Wendroff tables)
     unsigned long long* cta_clock;  // per CTA: %globaltimer at start and at end (2 grid entries; may be null)
-    // warp queue (may be null): instances of at most warp_cells cells, one warp each
-    const int* order_small;
-    const int* n_small;
-    int* next_small;
 };
 
-cudaError_t batch_launch_f32(const void* args, int grid, int threads, int smem, cudaStream_t st);
-cudaError_t batch_launch_f16(const void* args, int grid, int threads, int smem, cudaStream_t st);
-cudaError_t batch_launch_bf16(const void* args, int grid, int threads, int smem, cudaStream_t st);
-cudaError_t batch_setup_f32(int threads, int smem, int* occupancy);
-cudaError_t batch_setup_f16(int threads, int smem, int* occupancy);
-cudaError_t batch_setup_bf16(int threads, int smem, int* occupancy);
+constexpr int kBatchThreads = 512;  // threads of a CTA by default (and at most)
+constexpr int kBatchClusterCtas = 2;
+
+// cluster: CTAs of a cluster (1 or kBatchClusterCtas; grid a multiple of it)
+cudaError_t batch_launch_f32(const void* args, int grid, int cluster, int threads, int smem, cudaStream_t st);
+cudaError_t batch_launch_f16(const void* args, int grid, int cluster, int threads, int smem, cudaStream_t st);
+cudaError_t batch_launch_bf16(const void* args, int grid, int cluster, int threads, int smem, cudaStream_t st);
+// *grid: the CTAs that run at the same time in clusters of that size; *smem is brought down to what
+// the kernel's own shared memory leaves of the device's limit
+cudaError_t batch_setup_f32(int threads, int cluster, int* smem, int* grid);
+cudaError_t batch_setup_f16(int threads, int cluster, int* smem, int* grid);
+cudaError_t batch_setup_bf16(int threads, int cluster, int* smem, int* grid);
 
 }  // namespace lbk

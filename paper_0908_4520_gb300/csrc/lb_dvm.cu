@@ -25,8 +25,8 @@
 //     P_{s+1} = u_{s+1} + c1 sin x + (G' - u') d^2   (c1, c2: the force over the half levels),
 //   and P is the state that is kept and advected.
 // A warp of its own sums the records and takes the force integrals (FP64 sine), 32 levels at a time.
-// Measured (us a level, one CTA an instance with ~15 operations, two sines and 2 n barriers a level /
-// now): seven instances of 20 nodes x 128 columns 65 / 2.8, one of them 65 / 2.8, forty 65 / 4.4.
+// Measured (us a level): seven instances of 20 nodes x 128 columns 2.8, against 65 with one CTA an
+// instance, ~15 operations a value, sines in every level and 2 n barriers; one of them 2.8, forty 4.4.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 

@@ -32,7 +32,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxDevices = 64;
-constexpr int kThreads = 256;        // the batch defaults, so results match an lb_batch run
+constexpr int kThreads = lbk::kBatchThreads;
 constexpr int kSmemBytes = 96 * 1024;
 
 size_t round_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -107,12 +107,12 @@ lb_status setup_device(int dev, int pi, unsigned char** base) {
         d.ready = true;
     }
     if (!d.kernel_ready[pi]) {
-        int occ = 0;
-        cudaError_t e = pi == 0   ? lbk::batch_setup_f32(kThreads, kSmemBytes, &occ)
-                        : pi == 1 ? lbk::batch_setup_f16(kThreads, kSmemBytes, &occ)
-                                  : lbk::batch_setup_bf16(kThreads, kSmemBytes, &occ);
+        int grid = 0, smem = kSmemBytes;
+        cudaError_t e = pi == 0   ? lbk::batch_setup_f32(kThreads, 1, &smem, &grid)
+                        : pi == 1 ? lbk::batch_setup_f16(kThreads, 1, &smem, &grid)
+                                  : lbk::batch_setup_bf16(kThreads, 1, &smem, &grid);
         if (e != cudaSuccess) return cuda_fail(e, "kernel set-up");
-        if (occ < 1) return fail(LB_ERR_CUDA, "kernel set-up: zero occupancy");
+        if (grid < 1) return fail(LB_ERR_CUDA, "kernel set-up: zero occupancy");
         d.kernel_ready[pi] = true;
     }
     *base = d.base;
@@ -217,18 +217,17 @@ lb_status lb_solve_static(const lb_instance_desc* d, lb_precision precision, lb_
     // ---- one launch: one CTA advances the instance until it finishes
     lbk::BatchArgs args{};
     args.inst = reinterpret_cast<lbk::BatchInst*>(base);
-    args.order = reinterpret_cast<const int*>(base + 256);
-    args.next = reinterpret_cast<int*>(base + 256 + 64);
-    args.n_order = reinterpret_cast<const int*>(base + 256 + 128);
+    args.queue[lbk::kBatchCta] = {reinterpret_cast<const int*>(base + 256), reinterpret_cast<const int*>(base + 256 + 128),
+                                  reinterpret_cast<int*>(base + 256 + 64)};
     args.chunk = 1 << 30;
     args.smem_cap = kSmemBytes;
     args.arena = base + pop_off;
     args.hist = reinterpret_cast<float2*>(base + hist_off);
     args.trig = reinterpret_cast<const float*>(base + trig_off);
     for (int i = 0; i < 3; ++i) args.tab[i] = g_tab[i];
-    e = pi == 0   ? lbk::batch_launch_f32(&args, 1, kThreads, kSmemBytes, s)
-        : pi == 1 ? lbk::batch_launch_f16(&args, 1, kThreads, kSmemBytes, s)
-                  : lbk::batch_launch_bf16(&args, 1, kThreads, kSmemBytes, s);
+    e = pi == 0   ? lbk::batch_launch_f32(&args, 1, 1, kThreads, kSmemBytes, s)
+        : pi == 1 ? lbk::batch_launch_f16(&args, 1, 1, kThreads, kSmemBytes, s)
+                  : lbk::batch_launch_bf16(&args, 1, 1, kThreads, kSmemBytes, s);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
 
     // ---- results (device-to-pageable copies return once they have completed)
