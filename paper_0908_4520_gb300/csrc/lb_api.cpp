@@ -607,12 +607,13 @@ lb_status lb_create_ex(const lb_params* pin, lb_handle** out) {
         L.args = &h->shape;
         if (h->launch(L) != cudaSuccess) {
             h->shape.V = 1;
+            h->shape.tw = 32;
             h->shape.rows = 8;
             h->shape.threads = 256;
             h->shape.occupancy = 0;
         }
     }
-    const int tw = 32 * h->shape.V;
+    const int tw = h->shape.tw;
     h->gy = upwind ? std::max(h->vs.halo, 2) : h->vs.halo;  // upwind: two upstream rows
     h->pitch = (P.nx + 2 * lbk::kGhostX + 63) / 64 * 64 + LB_PITCH_PAD;
     h->plane = (long long)h->pitch * (P.ny + 2 * h->gy);

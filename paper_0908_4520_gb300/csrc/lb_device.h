@@ -99,7 +99,8 @@ struct Args {
 
 // Launch geometry of a compiled (set, storage) unit.
 struct Shape {
-    int V;          // cells per thread along x (tile width 32 V), register kernels
+    int V;          // cells per thread along x, register kernels
+    int tw;         // cells of a row of their tiles (a warp's)
     int rows;       // warps per block = lattice rows per tile
     int threads;    // 32 * rows
     int occupancy;  // resident blocks per SM of the step kernel

@@ -438,6 +438,11 @@ constexpr int cells_per_lane() {
 template <class VS, class S>
 struct Cfg {
     static constexpr int V = cells_per_lane<VS, S, (LB_CFG_V > 0 ? LB_CFG_V : LB_TMA_V)>();
+    // Lax-Wendroff, one cell per lane, FP32 arithmetic: the warp's edge lanes are halo lanes, as in
+    // the TMA-staged kernel: three loads a velocity instead of six (256^2 D2Q36-GH FP32, 400 levels:
+    // 9.79 -> 6.21 ms)
+    static constexpr bool HALO = !VS::kOnLattice && V == 1 && sizeof(S) <= 4 && LB_PAIR_COLLISION && VS::NA % 2 == 0;
+    static constexpr int TW = HALO ? 30 : 32 * V;  // cells of a warp (upwind streaming: 32 V)
     static constexpr int ROWS = LB_CFG_ROWS;
     static constexpr int THREADS = 32 * ROWS;
     // one cell per lane needs under 128 registers: two blocks (16 warps) per SM
@@ -868,7 +873,6 @@ struct PairCollision {
 // the lane's column (values of the rows y - 1, y, y + 1), then the x pass, whose neighbours'
 // columns come by shuffles.  The pair has one x node and two y nodes, so both passes run as
 // packed f32x2 operations: 6 instead of 12 arithmetic instructions a pair, the same rounding.
-// (32 levels: D2Q36-GH FP32 4096^2 28.7 -> 28.2 ms, D2Q64-GH FP16 2048^2 17.0 -> 16.4 ms.)
 template <class VS, int A_>
 __device__ __forceinline__ f2 lw_y_pair(const Tab<float>& t, f2 fm, f2 f0, f2 fp) {
     constexpr int iy = VS::iy(A_);
@@ -1284,7 +1288,8 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
     constexpr int Q = VS::Q;
     constexpr int V = Cfg<VS, S>::V;
     constexpr int ROWS = Cfg<VS, S>::ROWS;
-    constexpr int TW = 32 * V;
+    constexpr bool HALO = Cfg<VS, S>::HALO && !UPW;
+    constexpr int TW = HALO ? Cfg<VS, S>::TW : 32 * V;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const S* src = static_cast<const S*>(A.src);
     S* dst = static_cast<S*>(A.dst);
@@ -1318,15 +1323,36 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
         if (y >= A.ny) continue;  // warp-uniform
         const int tile_start = tx * TW;
         const int x0 = (tx == A.ntiles_x - 1) ? A.x0_last : tile_start;
-        const Lane g = lane_geometry<V>(lane, x0, tile_start, A.nx);
+        const Lane g = HALO ? halo_lane_geometry(lane, x0, tile_start, A.nx) : lane_geometry<V>(lane, x0, tile_start, A.nx);
 
         using T = typename Pack<R, V>::T;
         T ft[Q];
-        static_for<0, Q>([&](auto ac) {
+        if (HALO && !A.raw) {
+            if constexpr (HALO) {
+                // velocity pairs, as in the TMA-staged kernel (columns past nx + 1 of a grid narrower
+                // than a warp lie in the row's padding and reach no cell)
+                const R one = R(1);
+                const S* p = src + A.origin + (long long)(y - 1) * A.pitch + g.xl;
+                static_for<0, Q / 2>([&](auto mc) {
+                    constexpr int a = 2 * decltype(mc)::value;
+                    const S* pa = p + (long long)a * A.plane;
+                    const S* pb = pa + A.plane;
+                    const f2 gv = lw_y_pair<VS, a>(
+                        A.tab, f2{ld1<S, R>(pa, one), ld1<S, R>(pb, one)},
+                        f2{ld1<S, R>(pa + A.pitch, one), ld1<S, R>(pb + A.pitch, one)},
+                        f2{ld1<S, R>(pa + 2 * A.pitch, one), ld1<S, R>(pb + 2 * A.pitch, one)});
+                    f2 v = lw_x_pair<VS, a>(A.tab, shfl_up2(gv), gv, shfl_down2(gv));
+                    if constexpr (Is16<S>::value)
+                        v = vmul(v, f2{load_scale<S, R>(A.tab, a), load_scale<S, R>(A.tab, a + 1)});
+                    ft[a] = v.x;
+                    ft[a + 1] = v.y;
+                });
+            }
+        } else static_for<0, Q>([&](auto ac) {
             constexpr int a = decltype(ac)::value;
             const R sc = load_scale<S, R>(A.tab, a);
             const S* pl = src + (long long)a * A.plane + A.origin;
-            if (A.raw) {
+            if (HALO || A.raw) {
                 const S* p = pl + (long long)y * A.pitch + g.xl;
                 if constexpr (V == 2) {
                     R v0, v1;
@@ -1915,6 +1941,7 @@ cudaError_t launch_typed(const Launch& L) {
     if (L.kind == kQueryShape) {
         Shape* sh = static_cast<Shape*>(const_cast<void*>(L.args));
         sh->V = C::V;
+        sh->tw = L.upwind ? 32 * C::V : C::TW;
         sh->rows = C::ROWS;
         sh->threads = C::THREADS;
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
