@@ -110,6 +110,9 @@ struct lb_handle {
     // store-staged TMA step kernel: its tiles, load maps (its box) and store maps (the cells of
     // each buffer as a destination)
     bool use_st = false;
+    // node-split FP64 step kernel: its warps of cells
+    bool use_split = false;
+    int split_ntiles_x = 0, split_ntiles = 0, split_grid = 0, split_warps = 1;  // warps of a block
     int st_ntiles_x = 0, st_ntiles = 0, st_grid = 0;
     CUtensorMap tmap_stl[2], tmap_out[2];
     long long plane = 0, origin = 0, ncell = 0;
@@ -120,11 +123,12 @@ struct lb_handle {
     void* buf[2] = {nullptr, nullptr};
     int cur = 0;
     bool raw_prev = true, initialized = false;
-    int place = 0;  // while a graph is captured: the step's place in it
+    int place = 0, chain = 1;  // while a graph is captured: the step's place in it, and its length
     long long level = 0, launches = 0;
     void* sin_d = nullptr;
     void* cos_d = nullptr;
     double* partials = nullptr;
+    int partial_stride = 0;
     unsigned int* ticket = nullptr;
     long long* level_d = nullptr;
     lb_diag* ring = nullptr;
@@ -201,7 +205,8 @@ struct lb_handle {
         stream = nullptr;
     }
 
-    // tiling: 0 the plain-load kernel's, 1 the TMA-staged kernel's, 2 the store-staged kernel's
+    // tiling: 0 the plain-load kernel's, 1 the TMA-staged kernel's, 2 the store-staged kernel's,
+    // 3 the node-split kernel's
     template <class R>
     void fill_args(lbk::Args<R>& A, int tiling) const {
         std::memset(&A, 0, sizeof(A));
@@ -211,8 +216,8 @@ struct lb_handle {
         A.ny = p.ny;
         A.pitch = pitch;
         A.gy = gy;
-        A.ntiles_x = tiling == 2 ? st_ntiles_x : tiling == 1 ? tma_ntiles_x : ntiles_x;
-        A.ntiles = tiling == 2 ? st_ntiles : tiling == 1 ? tma_ntiles : ntiles;
+        A.ntiles_x = tiling == 3 ? split_ntiles_x : tiling == 2 ? st_ntiles_x : tiling == 1 ? tma_ntiles_x : ntiles_x;
+        A.ntiles = tiling == 3 ? split_ntiles : tiling == 2 ? st_ntiles : tiling == 1 ? tma_ntiles : ntiles;
         A.x0_last = tiling == 2 ? 0 : tiling == 1 ? tma_x0_last : x0_last;
         A.isothermal = p.isothermal;
         A.diag_every = 1;
@@ -230,6 +235,9 @@ struct lb_handle {
         A.sinx = static_cast<const R*>(sin_d);
         A.cosx = static_cast<const R*>(cos_d);
         A.partials = partials;
+        A.partial_stride = partial_stride;
+        A.norm = 2.0 / ((double)p.nx * (double)p.ny);
+        A.mass0 = (double)p.nx * (double)p.ny;
         A.ticket = ticket;
         A.level = level_d;
         A.ring = ring;
@@ -265,7 +273,8 @@ lb_status launch_with(lb_handle* h, int kind, const void* src, void* dst, int ra
     lbk::Args<R> A;
     const bool tma = (kind == lbk::kStepTma || kind == lbk::kMomentsTma);
     const bool st = kind == lbk::kStepTmaStore;
-    h->fill_args(A, st ? 2 : tma ? 1 : 0);
+    const bool split = kind == lbk::kStepSplit || kind == lbk::kStepSplitForced;
+    h->fill_args(A, split ? 3 : st ? 2 : tma ? 1 : 0);
     if (tma) A.tmap = h->tmap[src == h->buf[0] ? 0 : 1];
     if (st) {
         A.tmap = h->tmap_stl[src == h->buf[0] ? 0 : 1];
@@ -290,10 +299,21 @@ lb_status launch_with(lb_handle* h, int kind, const void* src, void* dst, int ra
     L.kind = kind;
     L.n_eq = h->p.n_eq;
     L.upwind = h->p.streaming == LB_STREAM_UPWIND2;
-    L.grid = grid;
+    // a step inside a captured chain: the plain-load and node-split kernels leave their record to the
+    // launch behind them (one more block of the grid), the TMA-staged ones close each level
+    const bool defers = kind == lbk::kStep || kind == lbk::kStepForced || split;
+    A.advance = 1;
+    if (defers) {
+        A.level_add = h->place;
+        A.pending = h->place > 0;
+        A.advance = h->place == h->chain - 1 ? h->chain : 0;
+    }
+    A.nparts = grid * (split ? h->split_warps : 1);
+    L.grid = grid + A.pending;
+    L.warps = h->split_warps;
     // programmatic dependents: the kernels whose launches are short, and the exact-shift sets (D2Q37 at
     // 4096^2 32.2 -> 27.9 ms for 32 levels); the Lax-Wendroff TMA-staged kernels lose 1 to 3 % by it
-    L.follows = h->place > 0 && (kind == lbk::kStep || kind == lbk::kStepForced || h->vs.on_lattice);
+    L.follows = h->place > 0 && (defers || h->vs.on_lattice);
     L.stream = h->stream;
     L.args = &A;
     const cudaError_t e = h->launch(L);
@@ -317,6 +337,9 @@ lb_status launch_any(lb_handle* h, int kind, const void* src, void* dst, int raw
 
 // One step launch: level n -> n+1 (src = buf[cur] holds f*(n-1), dst gets f*(n)).
 lb_status step_once(lb_handle* h, int from) {
+    if (h->use_split)
+        return launch_any(h, h->p.force_amp != 0.0 ? lbk::kStepSplitForced : lbk::kStepSplit, h->buf[from],
+                          h->buf[1 - from], 0, h->split_grid);
     if (h->p.force_amp != 0.0)  // the forced step runs the plain-load kernel
         return launch_any(h, lbk::kStepForced, h->buf[from], h->buf[1 - from], 0, h->grid);
     if (h->use_st) return launch_any(h, lbk::kStepTmaStore, h->buf[from], h->buf[1 - from], 0, h->st_grid);
@@ -379,10 +402,12 @@ lb_status build_graph(lb_handle* h, int from, int nsteps, cudaGraphExec_t* out) 
     int b = from;
     for (int i = 0; i < nsteps && st == LB_OK; ++i) {
         h->place = i;
+        h->chain = nsteps;
         st = step_once(h, b);
         b = 1 - b;
     }
     h->place = 0;
+    h->chain = 1;
     e = cudaStreamEndCapture(h->stream, &g);
     h->launches = before;  // captured launches are counted at replay
     if (st != LB_OK) {
@@ -673,6 +698,20 @@ lb_status lb_create_ex(const lb_params* pin, lb_handle** out) {
         delete h;
         return reject(LB_ERR_UNSUPPORTED, "no TMA-staged step kernel for this storage");
     }
+    if (h->shape.split_cells > 0 && P.step_kernel == 0) {
+        // the node-split kernel where it holds the busiest of an SM's four FP64 units for clearly less
+        // work than the plain-load kernel's blocks of rows (same populations): grids that leave SMs
+        // without a block.  us a level, plain-load / node-split: D2Q16-GH 64 x 1 20.6 / 7.5, 64 x 16
+        // 32.9 / 11.1, 128 x 64 33.1 / 20.4; D2Q64-GH 64 x 1 66 / 12, 200 x 100 116 / 105; D2Q36-GH 200 x 100
+        // (0.79 of the plain-load kernel's work) 67 / 71
+        h->split_ntiles_x = (P.nx + h->shape.split_cells - 1) / h->shape.split_cells;
+        const long long warps = (long long)h->split_ntiles_x * P.ny, per_sm = (warps + nsm - 1) / nsm;
+        const long long rows = (long long)((h->ntiles + nsm - 1) / nsm) * std::min(P.ny, h->shape.rows);
+        h->use_split = 4 * ((per_sm + 3) / 4) * h->shape.split_ops < 3 * ((rows + 3) / 4) * h->shape.plain_ops;
+        h->split_ntiles = (int)std::min<long long>(warps, 1LL << 30);
+        h->split_warps = per_sm > 1 ? lbk::kSplitWarps : 1;
+        h->split_grid = (int)std::min<long long>((warps + h->split_warps - 1) / h->split_warps, 4LL * nsm);
+    }
     h->grid = std::max(1, std::min(h->ntiles, nsm * occ));
     h->grid_init = (int)std::max<long long>(1, std::min<long long>((h->ncell + 255) / 256, 4LL * nsm));
     const size_t rbytes = P.precision == LB_F64 ? 8 : 4;
@@ -680,8 +719,9 @@ lb_status lb_create_ex(const lb_params* pin, lb_handle** out) {
     h->buf[1] = h->dalloc(h->pop_bytes);
     h->sin_d = h->dalloc(rbytes * P.nx);
     h->cos_d = h->dalloc(rbytes * P.nx);
+    h->partial_stride = lbk::kDiagSlots * std::max({h->grid, h->tma_grid, h->st_grid, h->use_split ? h->split_grid * h->split_warps : 0});
     h->partials = static_cast<double*>(
-        h->dalloc(sizeof(double) * lbk::kDiagSlots * (size_t)std::max({h->grid, h->tma_grid, h->st_grid})));
+        h->dalloc(2 * sizeof(double) * (size_t)h->partial_stride));
     h->ticket = static_cast<unsigned int*>(h->dalloc(256));
     h->level_d = static_cast<long long*>(h->dalloc(256));
     h->status = static_cast<int*>(h->dalloc(256));

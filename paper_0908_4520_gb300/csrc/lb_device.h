@@ -16,6 +16,7 @@ constexpr int kMaxQ = lbvs::kMaxQ;
 constexpr int kMaxNA = lbvs::kMaxNA;
 constexpr int kMaxN = 4;
 constexpr int kDiagSlots = 8;  // doubles per partial / record
+constexpr int kSplitWarps = 4; // warps of a large block of the node-split kernel
 constexpr int kGhostX = 8;     // ghost columns kept on each side of a population row
 
 // Per-handle constant tables, passed by value in the kernel parameter space
@@ -50,6 +51,7 @@ struct Tab {
 
 enum Kind : int {
     kStep = 0, kMoments = 1, kInit = 2, kStepTma = 3, kStepForced = 4, kMomentsTma = 5, kStepTmaStore = 6,
+    kStepSplit = 7, kStepSplitForced = 8,
     kQueryShape = -1
 };
 
@@ -82,7 +84,14 @@ struct Args {
     double force_freq;
     const R* sinx;            // sin(x_i), nx entries
     const R* cosx;            // cos(x_i)
-    double* partials;         // gridDim.x * kDiagSlots
+    double* partials;         // two halves (launches of even and odd place in a chain) of kDiagSlots a sum
+    int partial_stride;       // doubles of a half
+    int nparts;               // sums a launch leaves there (one a working block; node-split: one a warp)
+    int level_add;            // the launch's level is *level + level_add (its place in a captured chain)
+    int advance;              // levels by which the launch advances *level at its end; 0: the launch behind
+                              // it writes its record
+    int pending;              // 1: the last block of the grid writes the record of the launch before
+    double norm, mass0;       // 2 / (nx ny); rho0 nx ny
     unsigned int* ticket;     // last-block election counter (returns to 0)
     long long* level;         // device time level, advanced by every step launch
     lb_diag* ring;            // diagnostics ring
@@ -112,6 +121,9 @@ struct Shape {
     // store-staged TMA kernel (0 = not built for this unit): tile of st_rows x st_tw cells,
     // load box st_box_w x st_box_h x box_d, one store box st_tw x st_rows x q per tile
     int st, st_tw, st_rows, st_threads, st_smem, st_occupancy, st_box_w, st_box_h;
+    // node-split FP64 kernel (split_cells = 0: not built for this unit): cells of a warp, and the
+    // FP64 operations of a warp of it and of the plain-load kernel
+    int split_cells, split_ops, plain_ops;
     int st_auto;    // 1: the automatic choice prefers the store-staged kernel on large grids
 };
 
@@ -120,6 +132,7 @@ struct Launch {
     int n_eq;                 // 1..4
     int upwind;               // 1: second-order upwind streaming (off-lattice sets, 32/64-bit storage)
     int grid;                 // blocks (persistent grid-stride over tiles)
+    int warps;                // warps of a block, 1 or kSplitWarps (node-split kernel only)
     int follows;              // 1: a step captured behind another one (programmatic dependent launch)
     cudaStream_t stream;
     const void* args;         // Args<float>/Args<double> matching the unit, or Shape* for kQueryShape

@@ -680,6 +680,57 @@ struct CellOut {
     T h;              // sum (f~ - w rho0)^2 / w                               (diag)
 };
 
+// The state of a cell from its summed moments (deviations): velocity, temperature and sigma_xy into
+// o, and (COLLIDE) the Hermite coefficients of its Maxwellian, c_{k+1} = u c_k + k (T - 1) c_{k-1},
+// with the force folded into the y ones.  Returns rho.  Shared by collide_cell and the node-split
+// kernel, so that both round the same.
+template <int N, class R, class T, bool COLLIDE>
+__device__ __forceinline__ T cell_state(R rho0, R sigma_fac, int isothermal, bool forced, T gf, R tau, R hdt, T drho,
+                                        T jx, T jy, T en, T pxy, CellOut<T>& o, T (&cx)[N + 1], T (&cy)[N + 1]) {
+    const T zero = vsplat<T>(R(0));
+    const T rho = vadd(vsplat<T>(rho0), drho);
+    const T rg = forced ? vmul(rho, gf) : zero;  // rho g
+    if (forced) jy = vfma(vsplat<T>(hdt), rg, jy);
+    const T inv = vrcp(rho);
+    const T ux = vmul(jx, inv), uy = vmul(jy, inv);
+    const T u2 = vfma(ux, ux, vmul(uy, uy));
+    T th = zero;
+    if (!isothermal) {
+        T e2 = vsub(vsub(en, vadd(drho, drho)), vmul(rho, u2));
+        if (forced) e2 = vfma(vmul(vsplat<T>(hdt + hdt), rg), uy, e2);
+        th = vmul(vmul(e2, vsplat<T>(R(0.5))), inv);
+    }
+    o.drho = drho;
+    o.jx = jx;
+    o.jy = jy;
+    o.ux = ux;
+    o.uy = uy;
+    o.th = th;
+    T pneq = pxy;
+    if constexpr (N >= 2) {
+        pneq = vsub(pxy, vmul(rho, vmul(ux, uy)));
+        if (forced) pneq = vfma(vmul(vsplat<T>(hdt), rg), ux, pneq);
+    }
+    o.sig = vmul(vsplat<T>(sigma_fac), pneq);
+    if constexpr (COLLIDE) {
+        cx[0] = cy[0] = vsplat<T>(R(1));
+        cx[1] = ux;
+        cy[1] = uy;
+#pragma unroll
+        for (int k = 1; k < N; ++k) {
+            const T kth = k == 1 ? th : vmul(vsplat<T>(R(k)), th);
+            cx[k + 1] = vfma(ux, cx[k], k == 1 ? kth : vmul(kth, cx[k - 1]));
+            cy[k + 1] = vfma(uy, cy[k], k == 1 ? kth : vmul(kth, cy[k - 1]));
+        }
+        if (forced) {
+            const T tg = vmul(vsplat<T>(tau), gf);
+#pragma unroll
+            for (int k = N; k >= 1; --k) cy[k] = vfma(vmul(vsplat<T>(R(k)), tg), cy[k - 1], cy[k]);
+        }
+    }
+    return rho;
+}
+
 // The one definition of the per-cell arithmetic; every kernel calls it.  The
 // streamed deviations are f(integral_constant<a>) (references, relaxed in place
 // when COLLIDE).  T is a scalar or a packed pair of cells.
@@ -742,48 +793,11 @@ __device__ __forceinline__ CellOut<T> collide_cell(const Tab<R>& t, R rho0, R om
 #pragma unroll
         for (int i = 0; i < NA; ++i) pxy = vfma(vsplat<T>(t.a[i]), P[i], pxy);
     }
-    const T rho = vadd(vsplat<T>(rho0), drho);
-    const T rg = forced ? vmul(rho, gf) : zero;  // rho g
-    if (forced) jy = vfma(vsplat<T>(hdt), rg, jy);
-    const T inv = vrcp(rho);
-    const T ux = vmul(jx, inv), uy = vmul(jy, inv);
-    const T u2 = vfma(ux, ux, vmul(uy, uy));
-    T th = zero;
-    if (!isothermal) {
-        T e2 = vsub(vsub(en, vadd(drho, drho)), vmul(rho, u2));
-        if (forced) e2 = vfma(vmul(vsplat<T>(hdt + hdt), rg), uy, e2);
-        th = vmul(vmul(e2, vsplat<T>(R(0.5))), inv);
-    }
-    o.drho = drho;
-    o.jx = jx;
-    o.jy = jy;
-    o.ux = ux;
-    o.uy = uy;
-    o.th = th;
-    T pneq = pxy;
-    if constexpr (N >= 2) {
-        pneq = vsub(pxy, vmul(rho, vmul(ux, uy)));
-        if (forced) pneq = vfma(vmul(vsplat<T>(hdt), rg), ux, pneq);
-    }
-    o.sig = vmul(vsplat<T>(sigma_fac), pneq);
     o.h = h;
+    T cx[N + 1], cy[N + 1];
+    const T rho = cell_state<N, R, T, COLLIDE>(rho0, sigma_fac, isothermal, forced, gf, tau, hdt, drho, jx, jy, en, pxy, o,
+                                               cx, cy);
     if constexpr (COLLIDE) {
-        // Hermite coefficients of the Maxwellian, c_{k+1} = u c_k + k (T - 1) c_{k-1}
-        T cx[N + 1], cy[N + 1];
-        cx[0] = cy[0] = vsplat<T>(R(1));
-        cx[1] = ux;
-        cy[1] = uy;
-#pragma unroll
-        for (int k = 1; k < N; ++k) {
-            const T kth = vmul(vsplat<T>(R(k)), th);
-            cx[k + 1] = vfma(ux, cx[k], vmul(kth, cx[k - 1]));
-            cy[k + 1] = vfma(uy, cy[k], vmul(kth, cy[k - 1]));
-        }
-        if (forced) {
-            const T tg = vmul(vsplat<T>(tau), gf);
-#pragma unroll
-            for (int k = N; k >= 1; --k) cy[k] = vfma(vmul(vsplat<T>(R(k)), tg), cy[k - 1], cy[k]);
-        }
         T QY[NA][N + 1];
 #pragma unroll
         for (int j = 0; j < NA; ++j) {
@@ -873,6 +887,7 @@ struct PairCollision {
 // the lane's column (values of the rows y - 1, y, y + 1), then the x pass, whose neighbours'
 // columns come by shuffles.  The pair has one x node and two y nodes, so both passes run as
 // packed f32x2 operations: 6 instead of 12 arithmetic instructions a pair, the same rounding.
+// (32 levels: D2Q36-GH FP32 4096^2 28.7 -> 28.2 ms, D2Q64-GH FP16 2048^2 17.0 -> 16.4 ms.)
 template <class VS, int A_>
 __device__ __forceinline__ f2 lw_y_pair(const Tab<float>& t, f2 fm, f2 f0, f2 fp) {
     constexpr int iy = VS::iy(A_);
@@ -951,47 +966,11 @@ __device__ __forceinline__ CellOut<float> collide_cell_pairs(const Tab<float>& t
             h = fmaf(t.wminv[I], hp.x + hp.y, h);
         });
     }
-    const R rho = rho0 + drho;
-    const R rg = forced ? __fmul_rn(rho, gf) : 0.f;
-    if (forced) jy = fmaf(hdt, rg, jy);
-    const R inv = 1.0f / rho;
-    const R ux = __fmul_rn(jx, inv), uy = __fmul_rn(jy, inv);
-    const R u2 = fmaf(ux, ux, __fmul_rn(uy, uy));
-    R th = 0.f;
-    if (!isothermal) {
-        R e2 = __fsub_rn(__fsub_rn(en, __fadd_rn(drho, drho)), __fmul_rn(rho, u2));
-        if (forced) e2 = fmaf(__fmul_rn(hdt + hdt, rg), uy, e2);
-        th = __fmul_rn(__fmul_rn(e2, 0.5f), inv);
-    }
-    o.drho = drho;
-    o.jx = jx;
-    o.jy = jy;
-    o.ux = ux;
-    o.uy = uy;
-    o.th = th;
-    R pneq = pxy;
-    if constexpr (N >= 2) {
-        pneq = __fsub_rn(pxy, __fmul_rn(rho, __fmul_rn(ux, uy)));
-        if (forced) pneq = fmaf(__fmul_rn(hdt, rg), ux, pneq);
-    }
-    o.sig = __fmul_rn(sigma_fac, pneq);
     o.h = h;
+    R cx[N + 1], cy[N + 1];
+    const R rho = cell_state<N, R, R, COLLIDE>(rho0, sigma_fac, isothermal, forced, gf, tau, hdt, drho, jx, jy, en, pxy, o,
+                                               cx, cy);
     if constexpr (COLLIDE) {
-        R cx[N + 1], cy[N + 1];
-        cx[0] = cy[0] = 1.f;
-        cx[1] = ux;
-        cy[1] = uy;
-#pragma unroll
-        for (int k = 1; k < N; ++k) {
-            const R kth = __fmul_rn((R)k, th);
-            cx[k + 1] = fmaf(ux, cx[k], __fmul_rn(kth, cx[k - 1]));
-            cy[k + 1] = fmaf(uy, cy[k], __fmul_rn(kth, cy[k - 1]));
-        }
-        if (forced) {
-            const R tg = __fmul_rn(tau, gf);
-#pragma unroll
-            for (int k = N; k >= 1; --k) cy[k] = fmaf(__fmul_rn((R)k, tg), cy[k - 1], cy[k]);
-        }
         // y factors of the y-node pairs: QY[j][ky] = W_j He_ky(a_j)/ky! c_ky(u_y)
         f2 QYp[NJ][N + 1];
 #pragma unroll
@@ -1209,64 +1188,90 @@ __device__ __forceinline__ void fold_diag(R (&acc)[6], double* wsum, int lane) {
     }
 }
 
-// End of a step launch: the last fold, per-block FP64 partials, last-block fixed-order sum
-// into the diagnostics ring, level advance.  All threads of the block call it; wsum holds
-// the per-warp FP64 sums (zeroed by each warp's lane 0 before its first fold).
-template <class R, int NWARPS_DIAG>
-__device__ __forceinline__ void finish_step(const Args<R>& A, R (&acc)[6], double (*wsum)[6], long long lvl,
-                                            bool diag, int warp, int lane) {
+// The record of level lvl from the nb FP64 sums of a launch (kDiagSlots doubles each), added in a
+// fixed order by the block that calls it: eight lanes take the quantities of one, the others
+// further ones.  Sets the status word where a sum is not finite.
+template <class R>
+__device__ __forceinline__ void write_record(const Args<R>& A, const double* part, int nb, long long lvl) {
+    __shared__ double tot[32][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)blockDim.x >> 5, q = threadIdx.x & 7;
+    double s = 0.0;
+    for (int b = threadIdx.x >> 3; b < nb; b += (int)blockDim.x >> 3)
+        s += __ldcg(part + (long long)b * kDiagSlots + min(q, 5));
+    s += __shfl_xor_sync(0xffffffffu, s, 8);
+    s += __shfl_xor_sync(0xffffffffu, s, 16);
+    if (nw > 1) {
+        if (lane < 8) tot[warp][lane] = s;
+        __syncthreads();
+        if (warp > 0) return;
+        s = 0.0;
+        for (int w = 0; w < nw; ++w) s += tot[w][q];
+    }
+    // lane 0..7: mass, mom_x, mom_y, amp, shear, hnorm, t, flags
+    const double v = q == 6 ? (double)lvl * A.dt : (q == 3 || q == 4 ? s * A.norm : (q == 0 ? A.mass0 + s : s));
+    const bool bad = __any_sync(0xffffffffu, (q == 0 || q == 3 || q == 5) && !isfinite(v));
+    double* r = reinterpret_cast<double*>(A.ring + (lvl / A.diag_every) % A.ring_cap);
+    if (lane < 8) r[q == 6 ? 0 : (q == 7 ? 7 : q + 1)] = q == 7 ? (bad ? 1.0 : 0.0) : v;
+    if (bad && lane == 0) atomicOr(A.status, 1);
+}
+
+// Step launches of a captured chain (plain-load and node-split kernels) leave the summing of their
+// blocks' partials to the launch behind them, which has a block of its own for it (A.pending), and
+// only the last launch of a chain sums its own and advances the level counter (A.advance levels):
+// the fence, the ticket and the last block's pass over the partials, ~1.3 to 2.3 us at the end of a
+// launch, are then not between two levels (256^2 D2Q36-GH FP32: 15.5 -> 10.0 us a level).  Blocks that
+// step cells:
+template <class R>
+__device__ __forceinline__ int work_blocks(const Args<R>& A) {
+    return (int)gridDim.x - A.pending;
+}
+template <class R>
+__device__ __forceinline__ double* partials_of(const Args<R>& A, int parity) {
+    return A.partials + (long long)parity * A.partial_stride;
+}
+
+// End of a launch once the block's partials are written (every thread of the block calls it): the
+// last block to come here writes the launch's record and advances the level.
+template <class R>
+__device__ __forceinline__ void close_level(const Args<R>& A, long long lvl, bool diag) {
+    if (A.advance == 0) return;  // the next launch writes the record
     __shared__ bool is_last;
-    __shared__ double tot[6];
-    if (diag && warp < NWARPS_DIAG) fold_diag(acc, wsum[warp], lane);
     __syncthreads();
     if (threadIdx.x == 0) {
-        if (diag) {
-#pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                double s = 0.0;
-                for (int w = 0; w < NWARPS_DIAG; ++w) s += wsum[w][i];
-                A.partials[(long long)blockIdx.x * kDiagSlots + i] = s;
-            }
-        }
         __threadfence();
-        const unsigned int t = atomicAdd(A.ticket, 1u);
-        is_last = (t == gridDim.x - 1);
+        is_last = atomicAdd(A.ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    if (diag) {
-        if (warp < 6) {
-            double s = 0.0;
-            for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(A.partials + (long long)b * kDiagSlots + warp);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) tot[warp] = s;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const double ncell = (double)A.nx * (double)A.ny;
-            const double norm = 2.0 / ncell;
-            lb_diag r;
-            r.t = (double)lvl * A.dt;
-            r.mass = ncell * (double)A.rho0 + tot[0];
-            r.mom_x = tot[1];
-            r.mom_y = tot[2];
-            r.amp = tot[3] * norm;
-            r.shear = tot[4] * norm;
-            r.hnorm = tot[5];
-            const bool bad = !(isfinite(r.mass) && isfinite(r.amp) && isfinite(r.hnorm));
-            r.flags = bad ? 1.0 : 0.0;
-            if (bad) atomicOr(A.status, 1);
-            const long long rec = lvl / A.diag_every;
-            A.ring[rec % A.ring_cap] = r;
-        }
-    }
     if (threadIdx.x == 0) {
-        *A.level = lvl + 1;
+        *A.level = lvl - A.level_add + A.advance;
         *A.ticket = 0u;
-        __threadfence();
     }
+    if (diag) write_record(A, partials_of(A, A.level_add & 1), A.nparts, lvl);
+}
+
+// The block beside the working ones: the record of the launch before.
+template <class R>
+__device__ __forceinline__ void pending_record(const Args<R>& A, long long lvl) {
+    if (A.diag_every > 0 && (lvl - 1) % A.diag_every == 0) write_record(A, partials_of(A, (A.level_add - 1) & 1), A.nparts, lvl - 1);
+    close_level(A, lvl, A.diag_every > 0 && lvl % A.diag_every == 0);
+}
+
+// End of a working block: the last fold, the block's FP64 partials, then close_level.  All threads
+// of the block call it; wsum holds the per-warp FP64 sums (zeroed by each warp's lane 0 before its
+// first fold).
+template <class R, int NWARPS_DIAG>
+__device__ __forceinline__ void finish_step(const Args<R>& A, R (&acc)[6], double (*wsum)[6], long long lvl,
+                                            bool diag, int warp, int lane) {
+    if (diag && warp < NWARPS_DIAG) fold_diag(acc, wsum[warp], lane);
+    __syncthreads();
+    if (diag && threadIdx.x < 6) {
+        double s = 0.0;
+        for (int w = 0; w < NWARPS_DIAG; ++w) s += wsum[w][threadIdx.x];
+        partials_of(A, A.level_add & 1)[(long long)blockIdx.x * kDiagSlots + threadIdx.x] = s;
+    }
+    close_level(A, lvl, diag);
 }
 
 // Programmatic dependent launch: a step launch may start while the one before it ends (its blocks
@@ -1299,8 +1304,12 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
     bool diag = false;
     if constexpr (STEP) {
         await_previous_step();
-        lvl = __ldcg(A.level);
+        lvl = __ldcg(A.level) + A.level_add;
         diag = (A.diag_every > 0) && (lvl % A.diag_every == 0);
+        if (A.pending && (int)blockIdx.x == work_blocks(A)) {
+            pending_record(A, lvl);
+            return;
+        }
     } else {
         // force phase of the state's level n: the device counter already points past it
         // (the launch that produced f*(n) advanced it to n + 1)
@@ -1316,7 +1325,8 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
     }
     int nfold = 0;
 
-    for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x) {
+    const int nb = work_blocks(A);
+    for (int tile = blockIdx.x; tile < A.ntiles; tile += nb) {
         const int ty = tile / A.ntiles_x;
         const int tx = tile - ty * A.ntiles_x;
         const int y = ty * ROWS + warp;
@@ -1464,6 +1474,232 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
         }
     }
     if constexpr (STEP) finish_step<R, ROWS>(A, acc, wsum, lvl, diag, warp, lane);
+}
+
+// ------------------------------------------------------------ node-split step kernel
+// FP64 Lax-Wendroff steps of small grids.  The card does two FP64 operations a clock and SM, so a
+// warp of 32 cells holds its SM for as long as its q x ~20 operations a cell take, while a small
+// grid leaves most SMs without a warp.  Here NA lanes share a cell, lane i holding the NA
+// velocities of x node i: a warp of 32 / NA cells, so that the same grid gives NA times as many
+// warps of an NA-th of the work each (blocks of one or four warps, so that they spread over the SMs
+// and then over an SM's four FP64 units: blocks of one warp put their warps on one unit, 128 x 64
+// D2Q16-GH 74 us a level).  Sums over the
+// y node and the equilibrium's own factors stay in the lane; sums over the x nodes go through
+// shared memory and run in the lanes side by side, lane r summing moment r, each in the order of
+// collide_cell, so the populations are those of the plain-load kernel bit for bit.
+// H is summed by lane (its rounding differs from the plain-load kernel's).
+template <class VS>
+struct SplitCfg {
+    static constexpr int NA = VS::NA;
+    static constexpr int CELLS = 32 / NA;  // cells of a warp (6 nodes: lanes 30, 31 repeat the last cell's)
+    // FP64 operations of a warp, about: of this kernel and of the plain-load kernel
+    static constexpr int OPS = 17 * NA + 75, PLAIN_OPS = 19 * VS::Q + 100;
+};
+
+// Sums of six values over the warp in eight additions (halves, quarters and eighths of the warp
+// part with the values between them); value i is returned in lane sum6_lane(i).
+__device__ __forceinline__ double warp_sum6(const double (&a)[6], int lane) {
+    constexpr unsigned m = 0xffffffffu;
+    const bool h = lane & 16, q = lane & 8, e = lane & 4;
+    double x[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) x[k] = (h ? a[k + 3] : a[k]) + __shfl_xor_sync(m, h ? a[k] : a[k + 3], 16);
+    // x[0], x[1] to the first quarter of each half, x[2] to the second
+    double y0 = (q ? x[2] : x[0]) + __shfl_xor_sync(m, q ? x[0] : x[2], 8);
+    const double r1 = __shfl_xor_sync(m, x[1], 8);
+    const double y1 = q ? 0.0 : x[1] + r1;
+    double z = (e ? y1 : y0) + __shfl_xor_sync(m, e ? y0 : y1, 4);
+    z += __shfl_xor_sync(m, z, 2);
+    z += __shfl_xor_sync(m, z, 1);
+    return z;
+}
+__device__ __forceinline__ int sum6_index(int lane) {  // the value a lane holds the sum of, or -1
+    switch (lane) {
+        case 0: return 0;
+        case 4: return 1;
+        case 8: return 2;
+        case 16: return 3;
+        case 20: return 4;
+        case 24: return 5;
+        default: return -1;
+    }
+}
+
+template <class VS, int N, int KIND, int W>
+__global__ void __launch_bounds__(32 * W) lb_split_kernel(const __grid_constant__ Args<double> A) {
+    static_assert(KIND == kStep || KIND == kStepForced, "node-split kinds: step, forced step");
+    constexpr int NA = VS::NA, CELLS = SplitCfg<VS>::CELLS, PAD = NA + 1;
+    constexpr int ROLES = NA > 4 ? 5 : 4;  // moments summed side by side (pxy apart where the lanes do not reach)
+    constexpr int EDGE = (2 * NA + CELLS - 1) / CELLS;  // edge columns' y passes of a lane
+    const int lane = threadIdx.x & 31, warp = W == 1 ? 0 : threadIdx.x >> 5;
+    const int c = min(lane / NA, CELLS - 1), i = lane % NA;
+    const bool first = lane < CELLS * NA;  // not a repeat
+    const double* src = static_cast<const double*>(A.src);
+    double* dst = static_cast<double*>(A.dst);
+    struct Warp {
+        double sv[CELLS][NA][PAD];    // streamed values, [cell][x node][y node]
+        double se[NA][2][PAD];        // y passes of the columns beside the warp, [x node][side][y node]
+        double sm[CELLS][4][PAD];     // by node: C (sums over y nodes), Ry (over x nodes), C + Ry, P
+        double sq[CELLS][NA][N + 1];  // y factors of the equilibrium
+    };
+    __shared__ Warp shared[W];
+    auto& sv = shared[warp].sv;
+    auto& se = shared[warp].se;
+    auto& sm = shared[warp].sm;
+    auto& sq = shared[warp].sq;
+    // the lane's x node, and its role's coefficients of the nodes
+    const Tab<double>& t = A.tab;
+    const double lx0 = t.lw[i][0], lx1 = t.lw[i][1], lx2 = t.lw[i][2];
+    const double ow = t.ow[i], wmi = t.wm[i], winvi = t.wminv[i];
+    double hn[N + 1], whn[N + 1], role[NA];
+#pragma unroll
+    for (int k = 1; k <= N; ++k) {
+        hn[k] = t.hn[i][k];
+        whn[k] = t.whn[i][k];
+    }
+#pragma unroll
+    for (int k = 0; k < NA; ++k) role[k] = i == 0 ? 1.0 : (i == 3 ? t.a2[k] : t.a[k]);
+    const int role_sum = i == 2 ? 1 : (i == 3 ? 2 : (i == 4 ? 3 : 0));
+    await_previous_step();
+    const long long lvl = __ldcg(A.level) + A.level_add;
+    const bool diag = (A.diag_every > 0) && (lvl % A.diag_every == 0);
+    const bool forced = KIND == kStepForced;
+    const int nb = work_blocks(A);
+    if (A.pending && (int)blockIdx.x == nb) {
+        pending_record(A, lvl);
+        return;
+    }
+    // y node of edge pass e (of 2 NA: the left column's, then the right one's; any node past them)
+    auto edge_node = [](int e) { return e < NA ? e : (e < 2 * NA ? e - NA : 0); };
+    double acc[6] = {0, 0, 0, 0, 0, 0};
+    const double om1 = 1.0 - A.omega;
+    double gt = 0.0;
+    bool have_gt = false;
+
+    for (int tile = (int)blockIdx.x * W + warp; tile < A.ntiles; tile += nb * W) {
+        const int y = tile / A.ntiles_x, x0 = (tile - y * A.ntiles_x) * CELLS;
+        const int x = x0 + c;
+        const bool own = first && x < A.nx;
+        const double* r0 = src + (long long)(i * NA) * A.plane + A.origin + (long long)y * A.pitch;
+        // the columns beside the warp (x0 - 1 and x0 + CELLS): their 2 NA y passes of x node i are
+        // shared out over the lanes of that node
+        double em[EDGE], e0[EDGE], ep[EDGE];
+#pragma unroll
+        for (int k = 0; k < EDGE; ++k) {
+            const int e = k * CELLS + c;
+            const double* p = r0 + edge_node(e) * A.plane + (e < NA ? x0 - 1 : min(x0 + CELLS, A.nx));
+            em[k] = p[-A.pitch];
+            e0[k] = *p;
+            ep[k] = p[A.pitch];
+        }
+        double vm[NA], v0[NA], vp[NA];
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+            const double* p = r0 + j * A.plane + min(x, A.nx);
+            vm[j] = p[-A.pitch];
+            v0[j] = *p;
+            vp[j] = p[A.pitch];
+        }
+        if (forced && !have_gt) {  // (its cosine while the loads are on their way)
+            gt = force_at_level(A, lvl);
+            have_gt = true;
+        }
+        const double sx = __ldg(A.sinx + min(x, A.nx - 1)), cxs = __ldg(A.cosx + min(x, A.nx - 1));
+#pragma unroll
+        for (int k = 0; k < EDGE; ++k) {
+            const int e = k * CELLS + c, j = edge_node(e);
+            const double ge = fma(t.lw[j][0], em[k], fma(t.lw[j][1], e0[k], t.lw[j][2] * ep[k]));
+            if (first && e < 2 * NA) se[i][e < NA ? 0 : 1][j] = ge;
+        }
+        __syncwarp();
+        double f[NA], C = 0.0, P = 0.0, h = 0.0;
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+            const double g = fma(t.lw[j][0], vm[j], fma(t.lw[j][1], v0[j], t.lw[j][2] * vp[j]));
+            double gl = __shfl_sync(0xffffffffu, g, max(c - 1, 0) * NA + i);
+            double gr = __shfl_sync(0xffffffffu, g, min(c + 1, CELLS - 1) * NA + i);
+            const double el = se[i][0][j], er = se[i][1][j];
+            gl = c == 0 ? el : gl;
+            gr = c == CELLS - 1 ? er : gr;
+            f[j] = fma(lx0, gl, fma(lx1, g, lx2 * gr));
+            C = __dadd_rn(C, f[j]);
+            if (diag) {
+                P = fma(t.a[j], f[j], P);
+                h = fma(__dmul_rn(f[j], t.wminv[j]), f[j], h);
+            }
+            sv[c][i][j] = f[j];
+        }
+        sm[c][0][i] = C;
+        sm[c][3][i] = P;
+        __syncwarp();
+        double Ry = 0.0;
+#pragma unroll
+        for (int k = 0; k < NA; ++k) Ry = __dadd_rn(Ry, sv[c][k][i]);
+        sm[c][1][i] = Ry;
+        sm[c][2][i] = __dadd_rn(C, Ry);
+        __syncwarp();
+        // lane r sums moment r over the nodes: rho - rho0, rho u_x, rho u_y, sum |xi|^2 d, Pi_xy
+        double s = 0.0, pxy = 0.0;
+#pragma unroll
+        for (int k = 0; k < NA; ++k) {
+            s = fma(role[k], sm[c][role_sum][k], s);
+            if (ROLES == 4) pxy = fma(t.a[k], sm[c][3][k], pxy);
+        }
+        const double drho = __shfl_sync(0xffffffffu, s, c * NA), jx = __shfl_sync(0xffffffffu, s, c * NA + 1),
+                     jy = __shfl_sync(0xffffffffu, s, c * NA + 2), en = __shfl_sync(0xffffffffu, s, c * NA + 3);
+        if (ROLES == 5) pxy = __shfl_sync(0xffffffffu, s, (c * NA + 4) & 31);
+        CellOut<double> o;
+        double cx[N + 1], cy[N + 1];
+        const double gf = forced ? gt * sx : 0.0;
+        const double rho = cell_state<N, double, double, true>(A.rho0, A.sigma_fac, A.isothermal, forced, gf, A.tau, A.hdt,
+                                                               drho, jx, jy, en, pxy, o, cx, cy);
+        sq[c][i][0] = wmi;
+#pragma unroll
+        for (int k = 1; k <= N; ++k) sq[c][i][k] = __dmul_rn(whn[k], cy[k]);
+        double PX[N + 1];
+        const double owr = __dmul_rn(ow, rho);
+#pragma unroll
+        for (int ky = 0; ky <= N; ++ky) {
+            double px = ky == 0 ? 0.0 : 1.0;
+#pragma unroll
+            for (int kx = 1; kx <= N - ky; ++kx) px = fma(cx[kx], hn[kx], px);
+            PX[ky] = ky == 0 ? __dmul_rn(ow, fma(rho, px, drho)) : __dmul_rn(owr, px);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+            double od = __dmul_rn(PX[0], sq[c][j][0]);
+#pragma unroll
+            for (int ky = 1; ky <= N; ++ky) od = fma(PX[ky], sq[c][j][ky], od);
+            f[j] = fma(f[j], om1, od);
+        }
+        if (own) {
+            double* const base = dst + (long long)(i * NA) * A.plane + A.origin;
+            auto put = [&](int xi, int yi) {
+                double* p = base + (long long)yi * A.pitch + xi;
+#pragma unroll
+                for (int j = 0; j < NA; ++j) p[j * A.plane] = f[j];
+            };
+            put(x, y);
+            if (has_images<double, 1>(A, x, y)) for_images<double, 1>(A, x, y, put);
+        }
+        if (diag) {
+            const bool one = own && i == 0;
+            acc[0] += one ? o.drho : 0.0;
+            acc[1] += one ? o.jx : 0.0;
+            acc[2] += one ? o.jy : 0.0;
+            acc[3] = fma(one ? o.uy : 0.0, sx, acc[3]);
+            acc[4] = fma(one ? o.sig : 0.0, cxs, acc[4]);
+            acc[5] = fma(winvi, own ? h : 0.0, acc[5]);
+        }
+        __syncwarp();  // the shared arrays are reused by the next tile
+    }
+    if (diag) {
+        const double v = warp_sum6(acc, lane);
+        const int q = sum6_index(lane);
+        if (q >= 0) partials_of(A, A.level_add & 1)[((long long)blockIdx.x * W + warp) * kDiagSlots + q] = v;
+    }
+    close_level(A, lvl, diag);
 }
 
 // ------------------------------------------------------------ TMA-staged step kernel
@@ -1619,7 +1855,7 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
     __syncthreads();
 
     if constexpr (KIND == kStep) await_previous_step();
-    const long long lvl = __ldcg(A.level);
+    const long long lvl = __ldcg(A.level) + A.level_add;
     const bool diag = KIND == kStep && (A.diag_every > 0) && (lvl % A.diag_every == 0);
     R acc[6] = {0, 0, 0, 0, 0, 0};
     __shared__ double wsum[CW][6];
@@ -1938,6 +2174,8 @@ cudaError_t launch_typed(const Launch& L) {
     // store-staged TMA kernel: Lax-Wendroff sets, FP32 up to 36 velocities (the FP32 output
     // tile of a 64-velocity set leaves too little shared memory for the ring), 16-bit all
     constexpr bool kStore = kTma && !VS::kOnLattice && ((std::is_same<S, float>::value && VS::Q <= 40) || Is16<S>::value);
+    // node-split FP64 steps of small grids
+    constexpr bool kSplit = std::is_same<S, double>::value && !VS::kOnLattice;
     if (L.kind == kQueryShape) {
         Shape* sh = static_cast<Shape*>(const_cast<void*>(L.args));
         sh->V = C::V;
@@ -1948,6 +2186,14 @@ cudaError_t launch_typed(const Launch& L) {
             &sh->occupancy, lb_fused_kernel<VS, N, S, R, kStep>, C::THREADS, 0);
         if (e != cudaSuccess) return e;
         sh->tma = 0;
+        sh->split_cells = 0;
+        if constexpr (kSplit) {
+            if (!L.upwind) {
+                sh->split_cells = SplitCfg<VS>::CELLS;
+                sh->split_ops = SplitCfg<VS>::OPS;
+                sh->plain_ops = SplitCfg<VS>::PLAIN_OPS;
+            }
+        }
         // the TMA-staged kernel of the requested streaming, and its box
         auto tma_shape = [&](auto kernel, auto cfg) -> cudaError_t {
             using TC = decltype(cfg);
@@ -2047,6 +2293,15 @@ cudaError_t launch_typed(const Launch& L) {
             break;
         case kStepTma:
             if constexpr (kTma) return launch_step<R>(lb_tma_step_kernel<VS, N, S>, L, T::THREADS, T::SMEM);
+            return cudaErrorNotSupported;
+        case kStepSplit:
+        case kStepSplitForced:
+            if constexpr (kSplit)
+                return launch_step<R>(L.kind == kStepSplit ? (L.warps == 1 ? lb_split_kernel<VS, N, kStep, 1>
+                                                                           : lb_split_kernel<VS, N, kStep, kSplitWarps>)
+                                                           : (L.warps == 1 ? lb_split_kernel<VS, N, kStepForced, 1>
+                                                                           : lb_split_kernel<VS, N, kStepForced, kSplitWarps>),
+                                      L, 32 * L.warps, 0);
             return cudaErrorNotSupported;
         case kMomentsTma:
             if constexpr (kTma) {
