@@ -168,6 +168,9 @@ struct lb_handle {
         err = std::string(where) + ": " + cudaGetErrorString(e);
         return LB_ERR_CUDA;
     }
+    // population elements: bytes of one, planes of them
+    size_t elem_bytes() const { return storage_bytes(p.precision) * (size_t)shape.vw; }
+    int planes() const { return vs.q / shape.vw; }
     void* dalloc(size_t bytes) {
         void* ptr = nullptr;
         if (p.alloc) {
@@ -350,15 +353,12 @@ lb_status step_once(lb_handle* h, int from) {
 lb_status encode_maps(lb_handle* h) {
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return h->fail(LB_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
-    CUtensorMapDataType dt;
-    switch (h->p.precision) {
-        case LB_F32: dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT32; break;
-        case LB_BF16: dt = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16; break;
-        case LB_F16: dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT16; break;
-        default: return h->fail(LB_ERR_UNSUPPORTED, "TMA staging is built for 32- and 16-bit storage");
-    }
-    const size_t b = storage_bytes(h->p.precision);
-    const cuuint64_t dims[3] = {(cuuint64_t)h->pitch, (cuuint64_t)(h->p.ny + 2 * h->gy), (cuuint64_t)h->vs.q};
+    // the maps move elements of 4 or 8 bytes, bit for bit
+    const size_t b = h->elem_bytes();
+    if (h->p.precision == LB_F64 || (b != 4 && b != 8))
+        return h->fail(LB_ERR_UNSUPPORTED, "TMA staging is built for 32- and 16-bit storage");
+    const CUtensorMapDataType dt = b == 8 ? CU_TENSOR_MAP_DATA_TYPE_UINT64 : CU_TENSOR_MAP_DATA_TYPE_UINT32;
+    const cuuint64_t dims[3] = {(cuuint64_t)h->pitch, (cuuint64_t)(h->p.ny + 2 * h->gy), (cuuint64_t)h->planes()};
     const cuuint64_t strides[2] = {(cuuint64_t)h->pitch * b, (cuuint64_t)h->plane * b};
     const cuuint32_t box[3] = {(cuuint32_t)h->shape.box_w, (cuuint32_t)h->shape.box_h, (cuuint32_t)h->shape.box_d};
     const cuuint32_t estr[3] = {1, 1, 1};
@@ -374,8 +374,8 @@ lb_status encode_maps(lb_handle* h) {
         // tile of all q velocities per store
         const cuuint32_t lbox[3] = {(cuuint32_t)h->shape.st_box_w, (cuuint32_t)h->shape.st_box_h,
                                     (cuuint32_t)h->shape.box_d};
-        const cuuint64_t odims[3] = {(cuuint64_t)h->p.nx, (cuuint64_t)h->p.ny, (cuuint64_t)h->vs.q};
-        const cuuint32_t obox[3] = {(cuuint32_t)h->shape.st_tw, (cuuint32_t)h->shape.st_rows, (cuuint32_t)h->vs.q};
+        const cuuint64_t odims[3] = {(cuuint64_t)h->p.nx, (cuuint64_t)h->p.ny, (cuuint64_t)h->planes()};
+        const cuuint32_t obox[3] = {(cuuint32_t)h->shape.st_tw, (cuuint32_t)h->shape.st_rows, (cuuint32_t)h->planes()};
         for (int i = 0; i < 2; ++i) {
             CUresult r = enc(&h->tmap_stl[i], dt, 3, h->buf[i], dims, strides, lbox, estr,
                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -631,6 +631,7 @@ lb_status lb_create_ex(const lb_params* pin, lb_handle** out) {
         L.upwind = upwind;  // the TMA-staged kernel (and box) of this streaming
         L.args = &h->shape;
         if (h->launch(L) != cudaSuccess) {
+            h->shape.vw = 1;
             h->shape.V = 1;
             h->shape.tw = 32;
             h->shape.rows = 8;
@@ -647,7 +648,7 @@ lb_status lb_create_ex(const lb_params* pin, lb_handle** out) {
     h->ntiles_x = (P.nx + tw - 1) / tw;
     h->x0_last = P.nx >= tw ? P.nx - tw : 0;
     h->ntiles = h->ntiles_x * ((P.ny + h->shape.rows - 1) / h->shape.rows);
-    h->pop_bytes = (size_t)h->vs.q * h->plane * storage_bytes(P.precision);
+    h->pop_bytes = (size_t)h->planes() * h->plane * h->elem_bytes();
 
     cudaError_t e;
     if (P.stream) {
@@ -845,16 +846,16 @@ long long row_block(const lb_handle* h, int r0) { return (long long)(r0 + h->gy)
 lb_status halo_copy(lb_handle* h, int side, void* dst, const void* src, bool pack) {
     if (!h->initialized) return h->fail(LB_ERR_STATE, "init first");
     if ((side != 0 && side != 1) || (pack ? !dst : !src)) return h->fail(LB_ERR_ARG, "side 0 or 1 and a device buffer");
-    const size_t b = storage_bytes(h->p.precision);
+    const size_t b = h->elem_bytes();
     const size_t block = (size_t)h->gy * h->pitch * b;   // gy whole padded rows of one plane
     const size_t plane = (size_t)h->plane * b;
     char* state = static_cast<char*>(h->buf[h->cur]);
     // pack: boundary rows 0..gy-1 or ny-gy..ny-1; unpack: ghost rows -gy..-1 or ny..ny+gy-1
     const int r0 = pack ? (side == 0 ? 0 : h->p.ny - h->gy) : (side == 0 ? -h->gy : h->p.ny);
     char* rows = state + row_block(h, r0) * (long long)b;
-    const cudaError_t e = pack ? cudaMemcpy2DAsync(dst, block, rows, plane, block, h->vs.q, cudaMemcpyDeviceToDevice,
+    const cudaError_t e = pack ? cudaMemcpy2DAsync(dst, block, rows, plane, block, h->planes(), cudaMemcpyDeviceToDevice,
                                                    h->stream)
-                               : cudaMemcpy2DAsync(rows, plane, src, block, block, h->vs.q, cudaMemcpyDeviceToDevice,
+                               : cudaMemcpy2DAsync(rows, plane, src, block, block, h->planes(), cudaMemcpyDeviceToDevice,
                                                    h->stream);
     if (e != cudaSuccess) return h->cuda_fail(e, pack ? "halo pack" : "halo unpack");
     return LB_OK;
@@ -863,7 +864,7 @@ lb_status halo_copy(lb_handle* h, int side, void* dst, const void* src, bool pac
 
 lb_status lb_halo_bytes(const lb_handle* h, size_t* bytes) {
     if (!h || !bytes) return LB_ERR_ARG;
-    *bytes = (size_t)h->vs.q * h->gy * h->pitch * storage_bytes(h->p.precision);
+    *bytes = (size_t)h->planes() * h->gy * h->pitch * h->elem_bytes();
     return LB_OK;
 }
 

@@ -30,7 +30,7 @@
 // 8 of 255, the tables are constant-bank operands (the kernel inlines its nine variants; through a
 // reference they were loads), and the two wide queues take the makespan of the largest instances
 // down to the mean load.  512 instances of the batching configuration, 800 levels, admission and
-// histories included: 169 ms before, 72 ms now.
+// histories included: 169 ms before, 72 ms, 66 ms with the populations in pairs.
 #pragma once
 
 #include "lb_batch.h"
@@ -114,13 +114,14 @@ __device__ __forceinline__ float warp_sum3(float a, float b, float c, int lane) 
 // Advance instance `id` by up to B.chunk levels with the group's warps (smem: the group's share of
 // the CTA's shared memory).
 template <class VS, int SET, int N, class S>
-__device__ __forceinline__ void batch_run(const BatchArgs& B, int id, S* smem, const BatchGroup& G, BatchShared& sh) {
+__device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem, const BatchGroup& G, BatchShared& sh) {
     constexpr int Q = VS::Q;
     BatchInst& in = B.inst[id];
     const Tab<float>& t = B.tab[SET];
     const int nx = in.nx, ny = in.ny;
     const int ncell = nx * ny;
-    const long long pop = (long long)Q * ncell;
+    using E = typename PairOf<S>::E;  // the populations lie in pairs of velocities, [pair][cell]
+    const long long pop = (long long)(Q / 2) * ncell;
     const float omega = in.omega, sigma_fac = in.sigma_fac;
     const int lane = threadIdx.x & 31, tid = G.tid, nthr = G.threads;
     // the instance's relaxation tables (omega W_i and the second terms of the exact FP32
@@ -146,13 +147,13 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, S* smem, c
     int cur = in.cur;
     const int stop = min(in.max_level, level + B.chunk - 1);
     // both buffers of an instance that fits the group's shared memory are stepped on chip
-    const bool onchip = G.ctas == 1 && 2 * pop * (long long)sizeof(S) <= (long long)G.smem_cap;
+    const bool onchip = G.ctas == 1 && 2 * pop * (long long)sizeof(E) <= (long long)G.smem_cap;
     S* const arena = static_cast<S*>(B.arena);
-    S* gbuf[2] = {arena + in.off[0], arena + in.off[1]};
-    S* buf[2] = {gbuf[0], gbuf[1]};
+    E* gbuf[2] = {reinterpret_cast<E*>(arena + in.off[0]), reinterpret_cast<E*>(arena + in.off[1])};
+    E* buf[2] = {gbuf[0], gbuf[1]};
     if (onchip) {
-        buf[0] = smem;
-        buf[1] = smem + pop;
+        buf[0] = static_cast<E*>(smem);
+        buf[1] = buf[0] + pop;
         if (level > 0)
             for (long long k = tid; k < pop; k += nthr) buf[cur][k] = gbuf[cur][k];
     }
@@ -173,8 +174,8 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, S* smem, c
     const float inv_scale = 1.0f / scale;
     G.sync();
     for (; level <= stop && !done; ++level) {
-        const S* src = buf[cur];
-        S* dst = buf[level == 0 ? 0 : 1 - cur];
+        const E* src = buf[cur];
+        E* dst = buf[level == 0 ? 0 : 1 - cur];
         float(*red)[kBatchSlots] = sh.red[G.first / 4][level & 1];
         float tot[3] = {0.f, 0.f, 0.f};  // lane l: the sums of slots l and l + 32
         for (int slot = G.wid; slot < nslot; slot += G.warps) {
@@ -214,48 +215,57 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, S* smem, c
                     });
                 } else {
                     const int ym = y == 0 ? ny - 1 : y - 1, yp = y + 1 == ny ? 0 : y + 1;
-                    const bool rows = ny > 1;  // one row: the three y taps read the same value
-                    const S* p0 = src + c;
-                    const S* pm = src + ym * nx + x;
-                    const S* pp = src + yp * nx + x;
-                    static_for<0, Q / 2>([&](auto mc) {
-                        constexpr int m = decltype(mc)::value, a = 2 * m;
-                        auto pair = [&](const S* p) {
-                            f2 v = f2{batch_load<S>(p), batch_load<S>(p + ncell)};
-                            if constexpr (Is16<S>::value)
-                                v = vmul(v, f2{t.sc[a] * scale, t.sc[a + 1] * scale});
-                            return v;
-                        };
-                        const f2 v0 = pair(p0);
-                        const f2 vm = rows ? pair(pm) : v0;
-                        const f2 vp = rows ? pair(pp) : v0;
-                        p0 += 2 * ncell;
-                        pm += 2 * ncell;
-                        pp += 2 * ncell;
-                        const f2 g = lw_y_pair<VS, a>(t, vm, v0, vp);
-                        const f2 gl = f2{__shfl_sync(0xffffffffu, g.x, from_l), __shfl_sync(0xffffffffu, g.y, from_l)};
-                        const f2 gr = f2{__shfl_sync(0xffffffffu, g.x, from_r), __shfl_sync(0xffffffffu, g.y, from_r)};
-                        fp[m] = lw_x_pair<VS, a>(t, gl, g, gr);
-                    });
+                    const E* p0 = src + c;
+                    const E* pm = src + ym * nx + x;
+                    const E* pp = src + yp * nx + x;
+                    // one row: the three y taps read the same value (the branch lies outside the velocity
+                    // loop, whose loads it would keep apart)
+                    auto stream = [&](auto rows) {
+                        static_for<0, Q / 2>([&](auto mc) {
+                            constexpr int m = decltype(mc)::value, a = 2 * m;
+                            auto pair = [&](const E* p) {
+                                f2 v = lds_pair<S>(p);  // (plain loads: the arena or shared memory)
+                                if constexpr (Is16<S>::value)
+                                    v = vmul(v, f2{t.sc[a] * scale, t.sc[a + 1] * scale});
+                                return v;
+                            };
+                            const f2 v0 = pair(p0);
+                            f2 vm = v0, vp = v0;
+                            if constexpr (decltype(rows)::value) {
+                                vm = pair(pm);
+                                vp = pair(pp);
+                            }
+                            p0 += ncell;
+                            pm += ncell;
+                            pp += ncell;
+                            const f2 g = lw_y_pair<VS, a>(t, vm, v0, vp);
+                            const f2 gl = f2{__shfl_sync(0xffffffffu, g.x, from_l), __shfl_sync(0xffffffffu, g.y, from_l)};
+                            const f2 gr = f2{__shfl_sync(0xffffffffu, g.x, from_r), __shfl_sync(0xffffffffu, g.y, from_r)};
+                            fp[m] = lw_x_pair<VS, a>(t, gl, g, gr);
+                        });
+                    };
+                    if (ny > 1) {
+                        stream(std::true_type{});
+                    } else {
+                        stream(std::false_type{});
+                    }
                 }
                 const CellOut<float> co = collide_cell_pairs<VS, N, true>(
                     t, rt[0], rt[1], rt[2], rt[3], 1.f, omega, sigma_fac, isothermal, true, false, 0.f, 0.f, 0.f,
                     [&](auto mc) -> f2& { return fp[decltype(mc)::value]; });
                 if (own) {
-                    uint32_t r = Is16<S>::value ? sr_seed(level, c) : 0u;
-                    S* p = dst + c;
+                    uint32_t r0 = 0, r1 = Is16<S>::value ? sr_seed(level, c) : 0u;
+                    E* p = dst + c;
                     static_for<0, Q / 2>([&](auto mc) {
                         constexpr int m = decltype(mc)::value, a = 2 * m;
+                        f2 si = f2{1.f, 1.f};
                         if constexpr (Is16<S>::value) {
-                            r = sr_next(r);
-                            p[0] = to_storage<S, float>(fp[m].x, t.scinv[a] * inv_scale, r);
-                            r = sr_next(r);
-                            p[ncell] = to_storage<S, float>(fp[m].y, t.scinv[a + 1] * inv_scale, r);
-                        } else {
-                            p[0] = fp[m].x;
-                            p[ncell] = fp[m].y;
+                            r0 = sr_next(r1);
+                            r1 = sr_next(r0);
+                            si = f2{t.scinv[a] * inv_scale, t.scinv[a + 1] * inv_scale};
                         }
-                        p += 2 * ncell;
+                        *p = to_storage_pair<S>(fp[m], si, r0, r1);
+                        p += ncell;
                     });
                     pa = fma(co.uy, sinx[x], pa);
                     ps = fma(co.sig, cosx[x], ps);
@@ -351,7 +361,7 @@ __global__ void __launch_bounds__(kBatchMaxWarps * 32) lb_batch_kernel(const __g
         G.tid = threadIdx.x - 32 * G.first;
         // each group's slice of the shared memory, 16-byte aligned
         G.smem_cap = (int)((long long)B.smem_cap * per_cta / nwarp) & ~15;
-        S* const smem = reinterpret_cast<S*>(bsm + (size_t)(G.first / per_cta) * G.smem_cap);
+        void* const smem = bsm + (size_t)(G.first / per_cta) * G.smem_cap;
         if (!Qu.order) continue;
         const int n = *Qu.n;
         if (n == 0) continue;

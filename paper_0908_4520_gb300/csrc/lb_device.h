@@ -55,18 +55,18 @@ enum Kind : int {
     kQueryShape = -1
 };
 
-// Population layout: plane a, row y, column x at
-//   a * plane + origin + y * pitch + x,   origin = gy * pitch + kGhostX,
-// for -kGhostX <= x < nx + kGhostX and -gy <= y < ny + gy: the rim holds the
+// Population layout: plane a, row y, column x at element
+//   a * plane + origin + y * pitch + x,   origin = gy * pitch + kGhostX
+// (an element: one velocity, or the velocities 2 a, 2 a + 1 where Layout<> pairs them), for -kGhostX <= x < nx + kGhostX and -gy <= y < ny + gy: the rim holds the
 // periodic images of the grid, rewritten by every launch that writes the
 // populations, so streaming never wraps an index.
 template <class R>
 struct Args {
     CUtensorMap tmap;         // TMA view of src (step kernel with TMA staging only)
     CUtensorMap tmap_st;      // TMA view of the cells of dst, nx x ny x q (store-staged kernel only)
-    const void* src;          // populations read (storage type), q planes
+    const void* src;          // populations read (storage type)
     void* dst;                // populations written
-    long long plane;          // elements per population plane ((ny + 2 gy) * pitch)
+    long long plane;          // elements per plane ((ny + 2 gy) * pitch)
     long long origin;         // offset of cell (0, 0) in a plane
     int nx, ny, pitch, gy;
     int ntiles_x, ntiles;     // tile grid (tile = rows x 32*V columns)
@@ -108,6 +108,7 @@ struct Args {
 
 // Launch geometry of a compiled (set, storage) unit.
 struct Shape {
+    int vw;         // velocities of a population element (2: pairs), see the population layout
     int V;          // cells per thread along x, register kernels
     int tw;         // cells of a row of their tiles (a warp's)
     int rows;       // warps per block = lattice rows per tile

@@ -160,6 +160,46 @@ __device__ __forceinline__ R store_scale(const Tab<R>& t, int a) {
     return R(1);
 }
 
+// ---------------------------------------------------------------- population elements
+// Lax-Wendroff sets with 32- and 16-bit storage keep two velocities (a, a + 1), a even, side by side:
+// plane a / 2 holds pairs, 8 or 4 bytes a cell.  The kernels collide such pairs as one packed value
+// (collide_cell_pairs), so a pair is one load, one 16-bit conversion pair and one store, and a tile
+// row of a TMA box has half the alignment padding.  The exact-shift sets (a shift of its own for
+// every velocity) and FP64 keep one velocity a plane.
+// (32 levels, one velocity a plane / pairs: D2Q36-GH FP32 4096^2 28.06 / 27.36 ms, D2Q64-GH FP32 2048^2
+// 15.8 / 13.4, FP16 16.2 / 15.4; D2Q16-GH FP32 2502 x 1251, 64 levels 6.31 / 5.60.)
+template <class S>
+struct PairOf {
+    using E = S;
+};
+template <>
+struct PairOf<float> {
+    using E = float2;
+};
+template <>
+struct PairOf<__half> {
+    using E = uint32_t;
+};
+template <>
+struct PairOf<__nv_bfloat16> {
+    using E = uint32_t;
+};
+template <class VS, class S>
+struct Layout {
+    static constexpr bool PAIRED = !VS::kOnLattice && VS::kProductWeights && VS::NA % 2 == 0 && sizeof(S) <= 4;
+    static constexpr int VW = PAIRED ? 2 : 1;               // velocities of an element
+    static constexpr int PLANES = VS::Q / VW;
+    static constexpr int EB = VW * (int)sizeof(S);          // bytes of an element
+    using E = typename std::conditional<PAIRED, typename PairOf<S>::E, S>::type;
+};
+// Scalar view of the populations: value of velocity a at element offset `off` of its plane is
+// base[pop_index(a, plane, off)], neighbours in x lie VW apart.
+template <class VS, class S>
+__device__ __forceinline__ long long pop_index(int a, long long plane, long long off) {
+    constexpr int VW = Layout<VS, S>::VW;
+    return VW * ((a / VW) * plane + off) + a % VW;
+}
+
 // ---------------------------------------------------------------- stochastic rounding
 // 16-bit stores of the step kernels round stochastically (unbiased: the stored
 // value equals the FP32 value in expectation), so per-step changes smaller than
@@ -352,6 +392,46 @@ struct Pack<float, 2> {
     using T = f2;
 };
 
+// A pair of velocities of one cell, unscaled (global memory; shared memory).
+template <class S>
+__device__ __forceinline__ f2 unpack_pair(uint32_t u) {
+    float2 t;
+    if constexpr (std::is_same<S, __half>::value) {
+        t = __half22float2(*reinterpret_cast<const __half2*>(&u));
+    } else {
+        t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u));
+    }
+    return f2{t.x, t.y};
+}
+template <class S>
+__device__ __forceinline__ f2 ld_pair(const typename PairOf<S>::E* p) {
+    if constexpr (std::is_same<S, float>::value) {
+        const float2 t = *p;
+        return f2{t.x, t.y};
+    } else {
+        return unpack_pair<S>(*p);
+    }
+}
+template <class S>
+__device__ __forceinline__ f2 lds_pair(const typename PairOf<S>::E* p) {
+    if constexpr (std::is_same<S, float>::value) {
+        const float2 t = *p;
+        return f2{t.x, t.y};
+    } else {
+        return unpack_pair<S>(*p);
+    }
+}
+// The stored pair (16-bit: stochastically rounded with the random bits of r0, r1).
+template <class S>
+__device__ __forceinline__ typename PairOf<S>::E to_storage_pair(f2 v, f2 si, uint32_t r0, uint32_t r1) {
+    if constexpr (std::is_same<S, float>::value) {
+        return make_float2(v.x, v.y);
+    } else {
+        const f2 h = vmul(v, si);
+        return to_storage16x2<S>(h.x, h.y, r0, r1);
+    }
+}
+
 // ------------------------------------------------------------ configuration
 // Launch shapes, from sweeps at 4096^2 (FP32, N = 3) and 2048^2 (D2Q64, N = 4):
 //  * Lax-Wendroff (Gauss-Hermite product) sets: one cell per lane and many warps
@@ -383,9 +463,6 @@ struct Pack<float, 2> {
 #endif
 #ifndef LB_TMA_EVICT_LAST
 #define LB_TMA_EVICT_LAST 1  // TMA loads keep their lines in L2 for the neighbouring tiles (-3 % DRAM reads)
-#endif
-#ifndef LB_PAIR_COLLISION
-#define LB_PAIR_COLLISION 1  // one cell per lane: collide velocity pairs as packed f32x2 values
 #endif
 #ifndef LB_TMA_HALO
 #define LB_TMA_HALO -1  // -1: per set and storage (see TmaCfg), 0: never, 1: always
@@ -432,7 +509,7 @@ struct Pack<float, 2> {
 // cells per lane along x (FP64 storage: always 1)
 template <class VS, class S, int OVERRIDE>
 constexpr int cells_per_lane() {
-    return sizeof(S) == 8 ? 1 : (OVERRIDE > 0 ? OVERRIDE : (VS::kOnLattice ? 2 : 1));
+    return sizeof(S) == 8 || Layout<VS, S>::PAIRED ? 1 : (OVERRIDE > 0 ? OVERRIDE : 2);
 }
 
 template <class VS, class S>
@@ -441,7 +518,7 @@ struct Cfg {
     // Lax-Wendroff, one cell per lane, FP32 arithmetic: the warp's edge lanes are halo lanes, as in
     // the TMA-staged kernel: three loads a velocity instead of six (256^2 D2Q36-GH FP32, 400 levels:
     // 9.79 -> 6.21 ms)
-    static constexpr bool HALO = !VS::kOnLattice && V == 1 && sizeof(S) <= 4 && LB_PAIR_COLLISION && VS::NA % 2 == 0;
+    static constexpr bool HALO = !VS::kOnLattice && V == 1 && Layout<VS, S>::PAIRED;
     static constexpr int TW = HALO ? 30 : 32 * V;  // cells of a warp (upwind streaming: 32 V)
     static constexpr int ROWS = LB_CFG_ROWS;
     static constexpr int THREADS = 32 * ROWS;
@@ -453,15 +530,17 @@ struct Cfg {
 // 0, 1 and 30, 31 compute the y pass of the two columns on either side of the 28 cells
 // that lanes 2..29 own, and the box carries two extra rows above and below.
 // WIDE: the store-staged variant of the Lax-Wendroff kernel (one cell per lane, halo
-// lanes): two warps share a tile row (FP32: 30 cells each, 60 per row, 240 bytes; 16-bit:
-// 28 cells each - lanes 30, 31 idle - 56 per row, 112 bytes: whole 16-byte TMA granules),
-// the consumer warps write the relaxed populations of the tile (16-bit: stochastically
+// lanes): two warps share a tile row (30 cells each, 60 velocity pairs per row: whole 16-byte TMA
+// granules), the consumer warps write the relaxed populations of the tile (16-bit: stochastically
 // rounded) into a shared-memory output tile, and the producer warp writes it to HBM with
 // one TMA tensor store per tile (cp.async.bulk.tensor, shared -> global), so no thread
 // issues per-velocity global stores and every DRAM sector of the tile is written whole.
 template <class VS, class S, bool UPW = false, bool WIDE = false>
 struct TmaCfg {
     static constexpr bool LW = !VS::kOnLattice;
+    using E = typename Layout<VS, S>::E;
+    static constexpr int VW = Layout<VS, S>::VW, EB = Layout<VS, S>::EB;
+    static_assert(LW == Layout<VS, S>::PAIRED || sizeof(S) == 8, "32/16-bit Lax-Wendroff sets are paired");
     static constexpr int V = cells_per_lane<VS, S, LB_TMA_V>();
     static_assert(!UPW || (LW && V == 1), "upwind TMA staging: Lax-Wendroff sets, one cell per lane");
     static_assert(!WIDE || (LW && V == 1 && !UPW && sizeof(S) <= 4), "store staging: 32/16-bit Lax-Wendroff sets");
@@ -484,24 +563,25 @@ struct TmaCfg {
     // and the barrier cost 5 %: 16.3 against 17.2 GLUPS for D2Q36-GH FP32 at 4096^2)
     static constexpr bool TILE_SYNC =
         LB_TMA_TILE_SYNC > 0 || (LB_TMA_TILE_SYNC < 0 && !WIDE && (HALO || UPW) && sizeof(S) == 4 && VS::Q == 36);
-    // cells a warp produces (store-staged 16-bit: 28, so that a tile row is 7 granules)
-    static constexpr int WCELLS = UPW ? 28 : (WIDE && sizeof(S) == 2 ? 28 : (HALO ? 30 : TW));
+    static constexpr int WCELLS = UPW ? 28 : (HALO ? 30 : TW);  // cells a warp produces
     static constexpr int TWO = WPR * WCELLS;            // cells a tile row produces
     static constexpr int GX = UPW ? 2 : 1;              // stencil reach (columns and rows) of the box
     static constexpr int BAND = LB_TMA_BAND >= 0 ? LB_TMA_BAND : (LW ? 0 : LB_TMA_BAND_SHIFT);  // tile order
-    static constexpr int AL = 16 / (int)sizeof(S);      // TMA x coordinates are multiples of 16 bytes
+    static constexpr int AL = 16 / EB;                  // TMA x coordinates are multiples of 16 bytes
     static_assert(!WIDE || TWO % AL == 0, "store-staged tile rows are whole 16-byte granules");
     static constexpr int BW = WIDE ? TWO + 2 * AL : ((HALO || UPW) ? 32 + AL : (LW ? TW + 2 * AL : TW + AL));
     static constexpr int BH = LW ? ROWS + 2 * GX : ROWS;
-    static constexpr int BOX = BW * BH;                 // elements of one velocity's box
-    // stride of the velocity slots in a stage: dense for one 3-D box (Lax-Wendroff),
+    static constexpr int BOX = BW * BH;                 // elements of one plane's box
+    // stride of the planes' slots in a stage: dense for one 3-D box (Lax-Wendroff),
     // 128-byte aligned for separate boxes (exact shift)
-    static constexpr int SLOT = LW ? BOX : ((BOX * (int)sizeof(S) + 127) / 128 * 128) / (int)sizeof(S);
+    static constexpr int SLOT = LW ? BOX : ((BOX * EB + 127) / 128 * 128) / EB;
     static constexpr int K = LB_TMA_K > 0 ? LB_TMA_K : (LW ? (VS::Q > 40 ? 12 : 6) : 18);  // velocities per stage
+    static_assert(K % VW == 0, "whole elements per stage");
+    static constexpr int KE = K / VW;                   // planes per stage
     static constexpr int NG = (VS::Q + K - 1) / K;      // stages per tile
-    static constexpr int STAGE_BYTES = (K * SLOT * (int)sizeof(S) + 127) / 128 * 128;
-    // output tile of the store-staged kernel: [velocity][row][TWO cells]
-    static constexpr int OUT_BYTES = WIDE ? (VS::Q * ROWS * TWO * (int)sizeof(S) + 127) / 128 * 128 : 0;
+    static constexpr int STAGE_BYTES = (KE * SLOT * EB + 127) / 128 * 128;
+    // output tile of the store-staged kernel: [plane][row][TWO cells]
+    static constexpr int OUT_BYTES = WIDE ? (Layout<VS, S>::PLANES * ROWS * TWO * EB + 127) / 128 * 128 : 0;
     static constexpr int NS_FIT = ((WIDE ? LB_TMA_WIDE_SMEM - OUT_BYTES : LB_TMA_SMEM) - 512) / STAGE_BYTES;
     static constexpr int NS = NS_FIT < LB_TMA_NS_TILES * NG ? NS_FIT : LB_TMA_NS_TILES * NG;
     static constexpr int THREADS = 32 * (CW + 1);       // + one producer warp
@@ -512,7 +592,7 @@ struct TmaCfg {
     static constexpr int MAXREG = MAXREG_FIT > 255 ? 255 : MAXREG_FIT;
     // ring, output tile, full/empty barriers of the ring, tile-done and output-free barriers
     static constexpr int SMEM = NS * STAGE_BYTES + OUT_BYTES + 2 * NS * 8 + 16 + 128;  // + alignment slack
-    static constexpr int BOX_D = LW ? K : 1;            // velocities per TMA box
+    static constexpr int BOX_D = LW ? KE : 1;           // planes per TMA box
 };
 
 // ------------------------------------------------------------ equilibrium
@@ -576,12 +656,10 @@ struct Lane {
 // TMA-staged Lax-Wendroff with one cell per lane: the warp's edge lanes are halo lanes
 // (columns x0 - 1 and x0 + 30), whose y-pass only feeds their neighbours' x-pass, so no
 // lane reads an extra column; lanes 1..30 own cells x0 .. x0 + 29.
-// (own: the number of cells the warp owns, lanes 1..own; 30, or 28 for the store-staged
-// 16-bit kernel, whose lanes 30 and 31 are idle)
-__device__ __forceinline__ Lane halo_lane_geometry(int lane, int x0, int tile_start, int nx, int own = 30) {
+__device__ __forceinline__ Lane halo_lane_geometry(int lane, int x0, int tile_start, int nx) {
     Lane g;
     g.x = x0 - 1 + lane;
-    g.own = lane >= 1 && lane <= own && g.x < nx && g.x >= tile_start;
+    g.own = lane >= 1 && lane <= 30 && g.x < nx && g.x >= tile_start;
     g.xl = g.x;
     return g;
 }
@@ -659,15 +737,17 @@ __device__ __forceinline__ bool has_images(const Args<R>& A, int x, int y) {
     return x < kGhostX || x + V > A.nx - kGhostX || y < A.gy || y >= A.ny - A.gy;
 }
 
-// Write the lane's value at (x, y) and at every periodic image (round to nearest: used for the
+// Write velocity a's value at (x, y) and at every periodic image (round to nearest: used for the
 // initial state).
-template <class S, class R>
-__device__ __forceinline__ void store_cell(const Args<R>& A, S* pl, int x, int y, R v, R si) {
+template <class VS, class S, class R>
+__device__ __forceinline__ void store_cell(const Args<R>& A, S* dst, int a, int x, int y, R v, R si) {
     S sv;
     st1<S, R>(&sv, v, si);
-    store_raw<S>(pl + (long long)y * A.pitch + x, sv);
-    if (has_images<R, 1>(A, x, y))
-        for_images<R, 1>(A, x, y, [&](int xi, int yi) { store_raw<S>(pl + (long long)yi * A.pitch + xi, sv); });
+    auto put = [&](int xi, int yi) {
+        dst[pop_index<VS, S>(a, A.plane, A.origin + (long long)yi * A.pitch + xi)] = sv;
+    };
+    put(x, y);
+    if (has_images<R, 1>(A, x, y)) for_images<R, 1>(A, x, y, put);
 }
 
 // ------------------------------------------------------------ collision (shared)
@@ -878,11 +958,6 @@ __device__ __forceinline__ R force_at_level(const Args<R>& A, long long lvl) {
 // instruction count.  Product-weight Gauss-Hermite sets (NA even), FP32 arithmetic.
 // Moments as in collide_cell, with the y-node sums kept as pairs and the x-node sums
 // reduced when the x node changes; H = sum_ix (1/W_ix) sum_iy d^2 / W_iy.
-template <class VS>
-struct PairCollision {
-    static constexpr bool value = VS::kProductWeights && !VS::kOnLattice && VS::NA % 2 == 0;
-};
-
 // Tensor-product Lax-Wendroff of a velocity pair (a, a + 1) of one lane's cell: the y pass over
 // the lane's column (values of the rows y - 1, y, y + 1), then the x pass, whose neighbours'
 // columns come by shuffles.  The pair has one x node and two y nodes, so both passes run as
@@ -1025,7 +1100,7 @@ __device__ __forceinline__ CellOut<float> collide_cell_pairs(const Tab<float>& t
 template <class VS, int N, class S, class R, int V, int KIND, class T, int OSTRIDE = 0>
 __device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], S* dst, int y,
                                               const Lane& g, bool diag, R (&acc)[6], int lane, long long lvl,
-                                              R gt, S* out = nullptr) {
+                                              R gt, typename Layout<VS, S>::E* out = nullptr) {
     constexpr int Q = VS::Q;
     static_assert(OSTRIDE == 0 || V == 1, "output tile: one cell per lane");
     // body force g_y(x_i, t_n) = gt sin(x_i), gt = A_f cos(phi t_n) (driven standing wave, Sec. 4);
@@ -1059,8 +1134,7 @@ __device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], 
         }
     }
     CellOut<T> co;
-    if constexpr (V == 1 && std::is_same<R, float>::value && PairCollision<VS>::value &&
-                  LB_PAIR_COLLISION) {
+    if constexpr (Layout<VS, S>::PAIRED) {
         // one cell per lane: velocity pairs as packed f32x2 values
         constexpr int NP = Q / 2;
         f2 fp[NP];
@@ -1103,47 +1177,62 @@ __device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], 
     if constexpr (STEP) {
         // The relaxed populations, straight from registers: to the cell (OSTRIDE > 0: to the
         // output tile) and, for the lanes of a boundary, to its periodic images in the ghost rim.
-        // put(p) writes all q planes at offset p of the first; each call draws the 16-bit rounding
+        // put(p) writes all planes at offset p of the first; each call draws the 16-bit rounding
         // bits anew from the cell's own stream, so every image holds the cell's bits.
-        auto put = [&](S* p, long long stride) {
-            uint32_t r0 = 0, r1 = 0;
-            if constexpr (Is16<S>::value) {
-                r0 = sr_seed(lvl, (long long)y * A.nx + g.x);
-                r1 = sr_seed(lvl, (long long)y * A.nx + g.x + 1);
-            }
-            static_for<0, Q>([&](auto ac) {
-                constexpr int a = decltype(ac)::value;
-                const R si = store_scale<S, R>(A.tab, a);
-                if constexpr (Is16<S>::value) {
-                    r0 = sr_next(r0);
-                    r1 = sr_next(r1);
-                }
-                if constexpr (Is16<S>::value && V == 2) {
-                    const T hs = vmul(ft[a], vsplat<T>(si));
-                    __stcs(reinterpret_cast<unsigned int*>(p),
-                           to_storage16x2<S>(lane_get<0>(hs), lane_get<1>(hs), r0, r1));
-                } else {
-                    const S s0 = to_storage<S, R>(lane_get<0>(ft[a]), si, r0);
-                    const S s1 = to_storage<S, R>(lane_get<V - 1>(ft[a]), si, r1);
-                    if constexpr (V == 2) {
-                        store_raw2<S>(p, s0, s1);
-                    } else {
-                        store_raw<S>(p, s0);
+        using E = typename Layout<VS, S>::E;
+        auto put = [&](E* p, long long stride) {
+            if constexpr (Layout<VS, S>::PAIRED) {
+                uint32_t r0 = 0, r1 = 0;
+                if constexpr (Is16<S>::value) r1 = sr_seed(lvl, (long long)y * A.nx + g.x);
+                static_for<0, Q / 2>([&](auto mc) {
+                    constexpr int a = 2 * decltype(mc)::value;
+                    if constexpr (Is16<S>::value) {
+                        r0 = sr_next(r1);
+                        r1 = sr_next(r0);
                     }
-                }
-                p += stride;
-            });
+                    *p = to_storage_pair<S>(f2{ft[a], ft[a + 1]},
+                                            f2{store_scale<S, R>(A.tab, a), store_scale<S, R>(A.tab, a + 1)}, r0, r1);
+                    p += stride;
+                });
+            } else {
+                static_for<0, Q>([&](auto ac) {
+                    constexpr int a = decltype(ac)::value;
+                    if constexpr (V == 2) {
+                        store_raw2<S>(p, lane_get<0>(ft[a]), lane_get<1>(ft[a]));
+                    } else {
+                        *p = ft[a];
+                    }
+                    p += stride;
+                });
+            }
         };
         if (g.own) {
-            S* const base = dst + A.origin;
+            E* const base = reinterpret_cast<E*>(dst) + A.origin;
             if constexpr (OSTRIDE > 0) {
                 put(out, OSTRIDE);
+                if (has_images<R, V>(A, g.x, y))
+                    for_images<R, V>(A, g.x, y,
+                                     [&](int xi, int yi) { put(base + (long long)yi * A.pitch + xi, A.plane); });
             } else {
-                put(base + (long long)y * A.pitch + g.x, A.plane);
+                // the cell, then (lanes of a boundary) its images: one copy of the stores
+                int xi = g.x, yi = y;
+                bool more = has_images<R, V>(A, g.x, y), self = true;
+                for (;;) {
+                    put(base + (long long)yi * A.pitch + xi, A.plane);
+                    if (!more) break;
+                    do {
+                        if (self) {  // to the first position, at the lowest row and column
+                            while (yi - A.ny >= -A.gy) yi -= A.ny;
+                            while (xi - A.nx >= -kGhostX) xi -= A.nx;
+                            self = false;
+                        } else if ((xi += A.nx) + V > A.nx + kGhostX) {
+                            while (xi - A.nx >= -kGhostX) xi -= A.nx;
+                            yi += A.ny;
+                        }
+                    } while (xi == g.x && yi == y);
+                    if (yi >= A.ny + A.gy) break;
+                }
             }
-            if (has_images<R, V>(A, g.x, y))
-                for_images<R, V>(A, g.x, y,
-                                 [&](int xi, int yi) { put(base + (long long)yi * A.pitch + xi, A.plane); });
         }
     }
     if constexpr (STEP) {
@@ -1337,123 +1426,115 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
 
         using T = typename Pack<R, V>::T;
         T ft[Q];
-        if (HALO && !A.raw) {
-            if constexpr (HALO) {
-                // velocity pairs, as in the TMA-staged kernel (columns past nx + 1 of a grid narrower
-                // than a warp lie in the row's padding and reach no cell)
-                const R one = R(1);
-                const S* p = src + A.origin + (long long)(y - 1) * A.pitch + g.xl;
+        if constexpr (HALO) {
+            // velocity pairs, as in the TMA-staged kernel (columns past nx + 1 of a grid narrower
+            // than a warp lie in the row's padding and reach no cell)
+            using E = typename Layout<VS, S>::E;
+            const E* p = reinterpret_cast<const E*>(src) + A.origin + (long long)y * A.pitch + g.xl;
+            // (the initial state is read as it is; the branch lies outside the velocity loop, whose
+            // loads it would keep apart)
+            auto put = [&](auto mc, f2 v) {
+                constexpr int a = 2 * decltype(mc)::value;
+                // the stencil is linear: 16-bit values are scaled once, after it
+                if constexpr (Is16<S>::value)
+                    v = vmul(v, f2{load_scale<S, R>(A.tab, a), load_scale<S, R>(A.tab, a + 1)});
+                ft[a] = v.x;
+                ft[a + 1] = v.y;
+            };
+            if (A.raw) {
+                static_for<0, Q / 2>([&](auto mc) {
+                    put(mc, ld_pair<S>(p));
+                    p += A.plane;
+                });
+            } else {
                 static_for<0, Q / 2>([&](auto mc) {
                     constexpr int a = 2 * decltype(mc)::value;
-                    const S* pa = p + (long long)a * A.plane;
-                    const S* pb = pa + A.plane;
-                    const f2 gv = lw_y_pair<VS, a>(
-                        A.tab, f2{ld1<S, R>(pa, one), ld1<S, R>(pb, one)},
-                        f2{ld1<S, R>(pa + A.pitch, one), ld1<S, R>(pb + A.pitch, one)},
-                        f2{ld1<S, R>(pa + 2 * A.pitch, one), ld1<S, R>(pb + 2 * A.pitch, one)});
-                    f2 v = lw_x_pair<VS, a>(A.tab, shfl_up2(gv), gv, shfl_down2(gv));
-                    if constexpr (Is16<S>::value)
-                        v = vmul(v, f2{load_scale<S, R>(A.tab, a), load_scale<S, R>(A.tab, a + 1)});
-                    ft[a] = v.x;
-                    ft[a + 1] = v.y;
+                    const f2 gv = lw_y_pair<VS, a>(A.tab, ld_pair<S>(p - A.pitch), ld_pair<S>(p), ld_pair<S>(p + A.pitch));
+                    put(mc, lw_x_pair<VS, a>(A.tab, shfl_up2(gv), gv, shfl_down2(gv)));
+                    p += A.plane;
                 });
             }
-        } else static_for<0, Q>([&](auto ac) {
-            constexpr int a = decltype(ac)::value;
-            const R sc = load_scale<S, R>(A.tab, a);
-            const S* pl = src + (long long)a * A.plane + A.origin;
-            if (HALO || A.raw) {
-                const S* p = pl + (long long)y * A.pitch + g.xl;
-                if constexpr (V == 2) {
-                    R v0, v1;
-                    ld2<S, R>(p, sc, v0, v1);
-                    ft[a] = pack_lanes<T, R>(v0, v1);
+        } else {
+            static_for<0, Q>([&](auto ac) {
+                constexpr int a = decltype(ac)::value;
+                constexpr int VW = Layout<VS, S>::VW;
+                const R sc = load_scale<S, R>(A.tab, a);
+                const S* pl = src + pop_index<VS, S>(a, A.plane, A.origin);
+                if (A.raw) {
+                    const S* p = pl + VW * ((long long)y * A.pitch + g.xl);
+                    if constexpr (V == 2) {
+                        R v0, v1;
+                        ld2<S, R>(p, sc, v0, v1);
+                        ft[a] = pack_lanes<T, R>(v0, v1);
+                    } else {
+                        ft[a] = ld1<S, R>(p, sc);
+                    }
+                } else if constexpr (VS::kOnLattice) {
+                    // exact shift: f~_a(x, y) = f*_a(x - ex, y - ey)
+                    constexpr int ex = VS::ex(a), ey = VS::ey(a);
+                    const S* p = pl + (long long)(y - ey) * A.pitch + g.xl - ex;
+                    if constexpr (V == 2 && (ex % 2 == 0)) {
+                        R v0, v1;
+                        ld2<S, R>(p, sc, v0, v1);
+                        ft[a] = pack_lanes<T, R>(v0, v1);
+                    } else if constexpr (V == 2) {
+                        ft[a] = pack_lanes<T, R>(ld1<S, R>(p, sc), ld1<S, R>(p + 1, sc));
+                    } else {
+                        ft[a] = ld1<S, R>(p, sc);
+                    }
+                } else if constexpr (UPW) {
+                    // tensor-product second-order upwind (Beam-Warming), one cell per lane: y pass
+                    // over the cell's row and the two upstream rows, x pass by shuffles from the two
+                    // upstream lanes; the two lanes at the warp's downstream edge compute the two
+                    // upstream columns outside the warp
+                    static_assert(V == 1 && !Is16<S>::value, "upwind streaming: one cell per lane, 32/64-bit");
+                    constexpr int ix = VS::ix(a), iy = VS::iy(a);
+                    constexpr int sx = VS::axis_sign(ix), sy = VS::axis_sign(iy);
+                    const R yf = A.tab.uw[iy][0], yn = A.tab.uw[iy][1], ys = A.tab.uw[iy][2];
+                    const R xf = A.tab.uw[ix][0], xn = A.tab.uw[ix][1], xs = A.tab.uw[ix][2];
+                    const S* r0 = pl + VW * (long long)y * A.pitch;
+                    const S* rn = r0 - VW * (long long)sy * A.pitch;
+                    const S* rf = r0 - VW * 2LL * sy * A.pitch;
+                    const R one = R(1);
+                    // lanes past the grid read the images of columns 0 and 1 (nx, nx + 1)
+                    const int xu = VW * min(g.x, A.nx + 1);
+                    const R gv = fma(yf, ld1<S, R>(rf + xu, one), fma(yn, ld1<S, R>(rn + xu, one),
+                                                                     ys * ld1<S, R>(r0 + xu, one)));
+                    // extra column: x0 - 2 + (lane & 1) (lanes 30, 31) for sx > 0,
+                    // x0 + 32 + (lane & 1) (lanes 0, 1) for sx < 0, clamped into the rim
+                    const int xe = VW * (sx > 0 ? x0 - 2 + (lane & 1) : min(x0 + 32 + (lane & 1), A.nx + 1));
+                    const R ge = fma(yf, ld1<S, R>(rf + xe, one), fma(yn, ld1<S, R>(rn + xe, one),
+                                                                     ys * ld1<S, R>(r0 + xe, one)));
+                    R g1, g2;
+                    if constexpr (sx > 0) {
+                        g1 = __shfl_up_sync(0xffffffffu, gv, 1);
+                        g2 = __shfl_up_sync(0xffffffffu, gv, 2);
+                        const R e2 = __shfl_sync(0xffffffffu, ge, 30);  // column x0 - 2
+                        const R e1 = __shfl_sync(0xffffffffu, ge, 31);  // column x0 - 1
+                        if (lane == 0) { g1 = e1; g2 = e2; }
+                        if (lane == 1) g2 = e1;
+                    } else {
+                        g1 = __shfl_down_sync(0xffffffffu, gv, 1);
+                        g2 = __shfl_down_sync(0xffffffffu, gv, 2);
+                        const R e1 = __shfl_sync(0xffffffffu, ge, 0);   // column x0 + 32
+                        const R e2 = __shfl_sync(0xffffffffu, ge, 1);   // column x0 + 33
+                        if (lane == 31) { g1 = e1; g2 = e2; }
+                        if (lane == 30) g2 = e1;
+                    }
+                    ft[a] = fma(xf, g2, fma(xn, g1, xs * gv));
                 } else {
-                    ft[a] = ld1<S, R>(p, sc);
-                }
-            } else if constexpr (VS::kOnLattice) {
-                // exact shift: f~_a(x, y) = f*_a(x - ex, y - ey)
-                constexpr int ex = VS::ex(a), ey = VS::ey(a);
-                const S* p = pl + (long long)(y - ey) * A.pitch + g.xl - ex;
-                if constexpr (V == 2 && (ex % 2 == 0)) {
-                    R v0, v1;
-                    ld2<S, R>(p, sc, v0, v1);
-                    ft[a] = pack_lanes<T, R>(v0, v1);
-                } else if constexpr (V == 2) {
-                    ft[a] = pack_lanes<T, R>(ld1<S, R>(p, sc), ld1<S, R>(p + 1, sc));
-                } else {
-                    ft[a] = ld1<S, R>(p, sc);
-                }
-            } else if constexpr (UPW) {
-                // tensor-product second-order upwind (Beam-Warming), one cell per lane: y pass
-                // over the cell's row and the two upstream rows, x pass by shuffles from the two
-                // upstream lanes; the two lanes at the warp's downstream edge compute the two
-                // upstream columns outside the warp
-                static_assert(V == 1 && !Is16<S>::value, "upwind streaming: one cell per lane, 32/64-bit");
-                constexpr int ix = VS::ix(a), iy = VS::iy(a);
-                constexpr int sx = VS::axis_sign(ix), sy = VS::axis_sign(iy);
-                const R yf = A.tab.uw[iy][0], yn = A.tab.uw[iy][1], ys = A.tab.uw[iy][2];
-                const R xf = A.tab.uw[ix][0], xn = A.tab.uw[ix][1], xs = A.tab.uw[ix][2];
-                const S* r0 = pl + (long long)y * A.pitch;
-                const S* rn = r0 - (long long)sy * A.pitch;
-                const S* rf = r0 - 2LL * sy * A.pitch;
-                const R one = R(1);
-                // lanes past the grid read the images of columns 0 and 1 (nx, nx + 1)
-                const int xu = min(g.x, A.nx + 1);
-                const R gv = fma(yf, ld1<S, R>(rf + xu, one), fma(yn, ld1<S, R>(rn + xu, one),
-                                                                 ys * ld1<S, R>(r0 + xu, one)));
-                // extra column: x0 - 2 + (lane & 1) (lanes 30, 31) for sx > 0,
-                // x0 + 32 + (lane & 1) (lanes 0, 1) for sx < 0, clamped into the rim
-                const int xe = sx > 0 ? x0 - 2 + (lane & 1) : min(x0 + 32 + (lane & 1), A.nx + 1);
-                const R ge = fma(yf, ld1<S, R>(rf + xe, one), fma(yn, ld1<S, R>(rn + xe, one),
-                                                                 ys * ld1<S, R>(r0 + xe, one)));
-                R g1, g2;
-                if constexpr (sx > 0) {
-                    g1 = __shfl_up_sync(0xffffffffu, gv, 1);
-                    g2 = __shfl_up_sync(0xffffffffu, gv, 2);
-                    const R e2 = __shfl_sync(0xffffffffu, ge, 30);  // column x0 - 2
-                    const R e1 = __shfl_sync(0xffffffffu, ge, 31);  // column x0 - 1
-                    if (lane == 0) { g1 = e1; g2 = e2; }
-                    if (lane == 1) g2 = e1;
-                } else {
-                    g1 = __shfl_down_sync(0xffffffffu, gv, 1);
-                    g2 = __shfl_down_sync(0xffffffffu, gv, 2);
-                    const R e1 = __shfl_sync(0xffffffffu, ge, 0);   // column x0 + 32
-                    const R e2 = __shfl_sync(0xffffffffu, ge, 1);   // column x0 + 33
-                    if (lane == 31) { g1 = e1; g2 = e2; }
-                    if (lane == 30) g2 = e1;
-                }
-                ft[a] = fma(xf, g2, fma(xn, g1, xs * gv));
-            } else {
-                // tensor-product Lax-Wendroff: y pass in registers, x pass by shuffles;
-                // the warp's two edge lanes take their outer neighbour from one extra column
-                constexpr int ix = VS::ix(a), iy = VS::iy(a);
-                const R ly0 = A.tab.lw[iy][0], ly1 = A.tab.lw[iy][1], ly2 = A.tab.lw[iy][2];
-                const R lx0 = A.tab.lw[ix][0], lx1 = A.tab.lw[ix][1], lx2 = A.tab.lw[ix][2];
-                const S* r0 = pl + (long long)y * A.pitch;
-                const S* rm = r0 - A.pitch;
-                const S* rp = r0 + A.pitch;
-                // the stencil is linear: 16-bit values are scaled once, after it (as in the
-                // TMA-staged kernel, so the two give the same bits)
-                const R one = R(1);
-                const int xe = (lane == 31) ? min(x0 + TW, A.nx) : x0 - 1;
-                const R ge = fma(ly0, ld1<S, R>(rm + xe, one), fma(ly1, ld1<S, R>(r0 + xe, one), ly2 * ld1<S, R>(rp + xe, one)));
-                if constexpr (V == 2) {
-                    R a0v, a1v, b0v, b1v, c0v, c1v;
-                    ld2<S, R>(r0 + g.xl, one, a0v, a1v);
-                    ld2<S, R>(rm + g.xl, one, b0v, b1v);
-                    ld2<S, R>(rp + g.xl, one, c0v, c1v);
-                    const T gv = vfma(vsplat<T>(ly0), pack_lanes<T, R>(b0v, b1v),
-                                      vfma(vsplat<T>(ly1), pack_lanes<T, R>(a0v, a1v),
-                                           vmul(vsplat<T>(ly2), pack_lanes<T, R>(c0v, c1v))));
-                    const R gv0 = lane_get<0>(gv), gv1 = lane_get<1>(gv);
-                    R gl = __shfl_up_sync(0xffffffffu, gv1, 1);
-                    R gr = __shfl_down_sync(0xffffffffu, gv0, 1);
-                    gl = (lane == 0) ? ge : gl;
-                    gr = (lane == 31) ? ge : gr;
-                    ft[a] = pack_lanes<T, R>(fma(lx0, gl, fma(lx1, gv0, lx2 * gv1)),
-                                             fma(lx0, gv0, fma(lx1, gv1, lx2 * gr)));
-                } else {
+                    // tensor-product Lax-Wendroff (FP64): y pass in registers, x pass by shuffles; the
+                    // warp's two edge lanes take their outer neighbour from one extra column
+                    static_assert(V == 1 && VW == 1, "one cell per lane, one velocity a plane");
+                    constexpr int ix = VS::ix(a), iy = VS::iy(a);
+                    const R ly0 = A.tab.lw[iy][0], ly1 = A.tab.lw[iy][1], ly2 = A.tab.lw[iy][2];
+                    const R lx0 = A.tab.lw[ix][0], lx1 = A.tab.lw[ix][1], lx2 = A.tab.lw[ix][2];
+                    const S* r0 = pl + (long long)y * A.pitch;
+                    const S* rm = r0 - A.pitch;
+                    const S* rp = r0 + A.pitch;
+                    const R one = R(1);
+                    const int xe = (lane == 31) ? min(x0 + TW, A.nx) : x0 - 1;
+                    const R ge = fma(ly0, ld1<S, R>(rm + xe, one), fma(ly1, ld1<S, R>(r0 + xe, one), ly2 * ld1<S, R>(rp + xe, one)));
                     const R f0 = ld1<S, R>(r0 + g.xl, one);
                     const R fm = ld1<S, R>(rm + g.xl, one);
                     const R fp = ld1<S, R>(rp + g.xl, one);
@@ -1464,9 +1545,8 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
                     gr = (lane == 31) ? ge : gr;
                     ft[a] = fma(lx0, gl, fma(lx1, gv, lx2 * gr));
                 }
-                if constexpr (Is16<S>::value) ft[a] = vmul(ft[a], vsplat<T>(sc));
-            }
-        });
+            });
+        }
         collide_store<VS, N, S, R, V, KIND>(A, ft, dst, y, g, diag, acc, lane, lvl, gt);
         if (STEP && diag && ++nfold == kDiagFold) {  // warp-uniform
             fold_diag(acc, wsum[warp], lane);
@@ -1822,16 +1902,15 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
     using C = TmaCfg<VS, S, UPW, WIDE>;
     constexpr int Q = VS::Q, V = C::V, ROWS = C::ROWS, CW = C::CW, TW = C::TW, AL = C::AL;
     constexpr int NS = C::NS, NG = C::NG, K = C::K, BW = C::BW, BOX = C::BOX, SLOT = C::SLOT;
-    constexpr int STAGE_ELEMS = C::STAGE_BYTES / (int)sizeof(S);
-    constexpr int OSTRIDE = WIDE ? ROWS * C::TWO : 0;  // output tile: elements per velocity
-    // Lax-Wendroff with halo lanes: the stencil runs on velocity pairs
-    constexpr bool PAIRS = C::HALO && PairCollision<VS>::value && K % 2 == 0;
+    using E = typename C::E;
+    constexpr int STAGE_ELEMS = C::STAGE_BYTES / C::EB, KE = C::KE;
+    constexpr int OSTRIDE = WIDE ? ROWS * C::TWO : 0;  // output tile: elements per plane
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     // TMA destinations must be 128-byte aligned: align the base explicitly
     unsigned char* const smem_raw =
         smem_dyn + ((128u - (smem_u32(smem_dyn) & 127u)) & 127u);
-    S* const stages = reinterpret_cast<S*>(smem_raw);
-    S* const otile = reinterpret_cast<S*>(smem_raw + NS * C::STAGE_BYTES);
+    E* const stages = reinterpret_cast<E*>(smem_raw);
+    E* const otile = reinterpret_cast<E*>(smem_raw + NS * C::STAGE_BYTES);
     uint64_t* const full = reinterpret_cast<uint64_t*>(smem_raw + NS * C::STAGE_BYTES + C::OUT_BYTES);
     uint64_t* const empty = full + NS;
     uint64_t* const tdone = empty + NS;  // store-staged: the consumers have filled the output tile
@@ -1887,13 +1966,13 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                     if (A.withhold_stage && blockIdx.x == 0 && tile == (int)blockIdx.x && grp == 0) continue;
                     const int a0 = grp * K;
                     const int na = (Q - a0) < K ? (Q - a0) : K;
-                    S* dstage = stages + (long long)s * STAGE_ELEMS;
+                    E* dstage = stages + (long long)s * STAGE_ELEMS;
                     if constexpr (C::LW) {
-                        mbar_arrive_expect_tx(&full[s], (uint32_t)(K * BOX * sizeof(S)));
+                        mbar_arrive_expect_tx(&full[s], (uint32_t)(KE * BOX * C::EB));
                         const int xs = WIDE ? x0 - AL + kGhostX : ((x0 - C::GX + kGhostX) / AL) * AL;
-                        tma_load_3d(dstage, &A.tmap, &full[s], xs, y0 - C::GX + A.gy, a0);
+                        tma_load_3d(dstage, &A.tmap, &full[s], xs, y0 - C::GX + A.gy, grp * KE);
                     } else {
-                        mbar_arrive_expect_tx(&full[s], (uint32_t)(na * BOX * sizeof(S)));
+                        mbar_arrive_expect_tx(&full[s], (uint32_t)(na * BOX * C::EB));
                         for (int j = 0; j < na; ++j) {
                             const int a = a0 + j;
                             const int xs = ((x0 - VS::ex(a) + kGhostX) / AL) * AL;
@@ -1936,7 +2015,7 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
             const int x0 = (!WIDE && tx == A.ntiles_x - 1) ? A.x0_last : tile_start;
             const int y = ty * ROWS + trow;
             const Lane g = UPW      ? upwind_lane_geometry(lane, x0, tile_start, A.nx)
-                           : C::HALO ? halo_lane_geometry(lane, x0, tile_start, A.nx, C::WCELLS)
+                           : C::HALO ? halo_lane_geometry(lane, x0, tile_start, A.nx)
                                      : lane_geometry<V>(lane, x0, tile_start, A.nx);
             using T = typename Pack<R, V>::T;
             T ft[Q];
@@ -1945,7 +2024,7 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
             // whose y-pass the two warp-edge lanes need (x0 - 1 for lane 0, x0 + TW for lane 31)
             // (store-staged: the box starts AL columns left of the tile row)
             const int r_lw = WIDE ? AL - 1 + half * C::WCELLS : (x0 - 1 + kGhostX) & (AL - 1);
-            const int c_lw = C::HALO ? r_lw + lane : r_lw + 1 + lane * V;
+            const int c_lw = C::HALO ? r_lw + lane : r_lw + 1 + lane;
             const int ce_lw = (lane == 31) ? r_lw + 1 + TW : r_lw;
             static_for<0, NG>([&](auto gc) {
                 constexpr int grp = decltype(gc)::value;
@@ -1954,112 +2033,77 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                     if (!ok) *abort_flag = 1;
                 }
                 if (ok) {
-                    const S* st = stages + (long long)st_i * STAGE_ELEMS;
-                    static_for<0, K>([&](auto jc) {
-                        constexpr int j = decltype(jc)::value;
-                        constexpr int a = grp * K + j;
-                        if constexpr (a < Q && PAIRS) {
-                            // the stencil is linear: 16-bit values are scaled once, after it
-                            if constexpr (j % 2 == 0) {
-                                const R one = R(1);
-                                const S* rm = st + j * SLOT + trow * BW + c_lw;  // row y - 1 of velocity a
-                                const S* rn = rm + SLOT;                         // and of a + 1
-                                const f2 gv = lw_y_pair<VS, a>(
-                                    A.tab, f2{sld1<S, R>(rm, one), sld1<S, R>(rn, one)},
-                                    f2{sld1<S, R>(rm + BW, one), sld1<S, R>(rn + BW, one)},
-                                    f2{sld1<S, R>(rm + 2 * BW, one), sld1<S, R>(rn + 2 * BW, one)});
-                                f2 v = lw_x_pair<VS, a>(A.tab, shfl_up2(gv), gv, shfl_down2(gv));
+                    const E* st = stages + (long long)st_i * STAGE_ELEMS;
+                    if constexpr (C::LW) {
+                        static_for<0, KE>([&](auto jc) {
+                            constexpr int j = decltype(jc)::value;
+                            constexpr int a = grp * K + 2 * j;
+                            if constexpr (a < Q) {
+                                // the pair (a, a + 1); the stencil is linear: 16-bit values are scaled
+                                // once, after it
+                                const E* box = st + j * SLOT;
+                                f2 v;
+                                if constexpr (UPW) {
+                                    // second-order upwind: y pass over the lane's column in the cell's
+                                    // row and its two upstream rows (box row of row y: trow + 2), x pass
+                                    // from the two upstream lanes (the same operation order as the
+                                    // plain-load kernel, so the two give the same bits); the y nodes of a
+                                    // pair may lie on either side of 0
+                                    constexpr int ix = VS::ix(a), iy = VS::iy(a);
+                                    constexpr int sx = VS::axis_sign(ix), sa = VS::axis_sign(iy), sb = VS::axis_sign(iy + 1);
+                                    const int c = ((x0 - 2 + kGhostX) & (AL - 1)) + lane;
+                                    const E* r0 = box + (trow + 2) * BW + c;
+                                    auto upstream = [&](int k) {
+                                        if constexpr (sa == sb) {
+                                            return lds_pair<S>(r0 - k * sa * BW);
+                                        } else {
+                                            return f2{reinterpret_cast<const float*>(r0 - k * sa * BW)[0],
+                                                      reinterpret_cast<const float*>(r0 - k * sb * BW)[1]};
+                                        }
+                                    };
+                                    auto uw = [&](int k) { return f2{A.tab.uw[iy][k], A.tab.uw[iy + 1][k]}; };
+                                    const f2 gv = vfma(uw(0), upstream(2), vfma(uw(1), upstream(1), vmul(uw(2), lds_pair<S>(r0))));
+                                    const f2 g1 = sx > 0 ? shfl_up2(gv) : shfl_down2(gv);
+                                    f2 g2;
+                                    if constexpr (sx > 0) {
+                                        g2 = f2{__shfl_up_sync(0xffffffffu, gv.x, 2), __shfl_up_sync(0xffffffffu, gv.y, 2)};
+                                    } else {
+                                        g2 = f2{__shfl_down_sync(0xffffffffu, gv.x, 2), __shfl_down_sync(0xffffffffu, gv.y, 2)};
+                                    }
+                                    v = vfma(vsplat<f2>(A.tab.uw[ix][0]), g2,
+                                             vfma(vsplat<f2>(A.tab.uw[ix][1]), g1, vmul(vsplat<f2>(A.tab.uw[ix][2]), gv)));
+                                } else {
+                                    auto column = [&](int c) {
+                                        const E* rm = box + trow * BW + c;  // row y - 1
+                                        return lw_y_pair<VS, a>(A.tab, lds_pair<S>(rm), lds_pair<S>(rm + BW),
+                                                                lds_pair<S>(rm + 2 * BW));
+                                    };
+                                    const f2 gv = column(c_lw);
+                                    f2 gl = shfl_up2(gv), gr = shfl_down2(gv);
+                                    if constexpr (!C::HALO) {
+                                        // all 32 lanes own cells: the edge lanes take their outer
+                                        // column's y pass from an extra read
+                                        const f2 ge = column(ce_lw);
+                                        gl = lane == 0 ? ge : gl;
+                                        gr = lane == 31 ? ge : gr;
+                                    }
+                                    v = lw_x_pair<VS, a>(A.tab, gl, gv, gr);
+                                }
                                 if constexpr (Is16<S>::value)
                                     v = vmul(v, f2{load_scale<S, R>(A.tab, a), load_scale<S, R>(A.tab, a + 1)});
                                 ft[a] = v.x;
                                 ft[a + 1] = v.y;
                             }
-                        } else if constexpr (a < Q) {
-                            const R sc = load_scale<S, R>(A.tab, a);
-                            const S* box = st + j * SLOT;
-                            if constexpr (UPW) {
-                                // second-order upwind: y pass over the lane's column in the cell's
-                                // row and its two upstream rows (box row of row y: warp + 2), x pass
-                                // from the two upstream lanes (the same operation order as the
-                                // plain-load kernel, so the two give the same bits)
-                                const R one = R(1);
-                                constexpr int ix = VS::ix(a), iy = VS::iy(a);
-                                constexpr int sx = VS::axis_sign(ix), sy = VS::axis_sign(iy);
-                                const R yf = A.tab.uw[iy][0], yn = A.tab.uw[iy][1], ys = A.tab.uw[iy][2];
-                                const R xf = A.tab.uw[ix][0], xn = A.tab.uw[ix][1], xs = A.tab.uw[ix][2];
-                                const int c = ((x0 - 2 + kGhostX) & (AL - 1)) + lane;
-                                const S* r0 = box + (trow + 2) * BW;
-                                const S* rn = r0 - sy * BW;
-                                const S* rf = r0 - 2 * sy * BW;
-                                const R gv = fma(yf, sld1<S, R>(rf + c, one),
-                                                 fma(yn, sld1<S, R>(rn + c, one), ys * sld1<S, R>(r0 + c, one)));
-                                R g1, g2;
-                                if constexpr (sx > 0) {
-                                    g1 = __shfl_up_sync(0xffffffffu, gv, 1);
-                                    g2 = __shfl_up_sync(0xffffffffu, gv, 2);
-                                } else {
-                                    g1 = __shfl_down_sync(0xffffffffu, gv, 1);
-                                    g2 = __shfl_down_sync(0xffffffffu, gv, 2);
-                                }
-                                ft[a] = fma(xf, g2, fma(xn, g1, xs * gv));
-                            } else if constexpr (C::LW) {
-                                // the stencil is linear: 16-bit values are scaled once, after it
-                                const R one = R(1);
-                                constexpr int ix = VS::ix(a), iy = VS::iy(a);
-                                const R ly0 = A.tab.lw[iy][0], ly1 = A.tab.lw[iy][1], ly2 = A.tab.lw[iy][2];
-                                const R lx0 = A.tab.lw[ix][0], lx1 = A.tab.lw[ix][1], lx2 = A.tab.lw[ix][2];
-                                const S* rm = box + trow * BW;
-                                const S* r0 = rm + BW;
-                                const S* rp = r0 + BW;
-                                if constexpr (C::HALO) {  // (a set of no pairs)
-                                    // y pass of the lane's column; x pass from the neighbours
-                                    const R f0 = sld1<S, R>(r0 + c_lw, one);
-                                    const R fm = sld1<S, R>(rm + c_lw, one);
-                                    const R fp = sld1<S, R>(rp + c_lw, one);
-                                    const R gv = fma(ly0, fm, fma(ly1, f0, ly2 * fp));
-                                    const R gl = __shfl_up_sync(0xffffffffu, gv, 1);
-                                    const R gr = __shfl_down_sync(0xffffffffu, gv, 1);
-                                    ft[a] = fma(lx0, gl, fma(lx1, gv, lx2 * gr));
-                                } else if constexpr (V == 2) {
-                                    const R ge = fma(ly0, sld1<S, R>(rm + ce_lw, one),
-                                                     fma(ly1, sld1<S, R>(r0 + ce_lw, one),
-                                                         ly2 * sld1<S, R>(rp + ce_lw, one)));
-                                    // y pass on the lane's two cells as one packed pair
-                                    R a0v, a1v, b0v, b1v, c0v, c1v;
-                                    sld2<S, R>(r0 + c_lw, one, a0v, a1v);
-                                    sld2<S, R>(rm + c_lw, one, b0v, b1v);
-                                    sld2<S, R>(rp + c_lw, one, c0v, c1v);
-                                    const T gv = vfma(vsplat<T>(ly0), pack_lanes<T, R>(b0v, b1v),
-                                                      vfma(vsplat<T>(ly1), pack_lanes<T, R>(a0v, a1v),
-                                                           vmul(vsplat<T>(ly2), pack_lanes<T, R>(c0v, c1v))));
-                                    const R gv0 = lane_get<0>(gv), gv1 = lane_get<1>(gv);
-                                    R gl = __shfl_up_sync(0xffffffffu, gv1, 1);
-                                    R gr = __shfl_down_sync(0xffffffffu, gv0, 1);
-                                    gl = (lane == 0) ? ge : gl;
-                                    gr = (lane == 31) ? ge : gr;
-                                    ft[a] = pack_lanes<T, R>(fma(lx0, gl, fma(lx1, gv0, lx2 * gv1)),
-                                                             fma(lx0, gv0, fma(lx1, gv1, lx2 * gr)));
-                                } else {
-                                    // one cell per lane, all 32 lanes own cells: the edge lanes
-                                    // take their outer column's y pass from an extra read
-                                    const R ge = fma(ly0, sld1<S, R>(rm + ce_lw, one),
-                                                     fma(ly1, sld1<S, R>(r0 + ce_lw, one),
-                                                         ly2 * sld1<S, R>(rp + ce_lw, one)));
-                                    const R f0 = sld1<S, R>(r0 + c_lw, one);
-                                    const R fm = sld1<S, R>(rm + c_lw, one);
-                                    const R fp = sld1<S, R>(rp + c_lw, one);
-                                    const R gv = fma(ly0, fm, fma(ly1, f0, ly2 * fp));
-                                    R gl = __shfl_up_sync(0xffffffffu, gv, 1);
-                                    R gr = __shfl_down_sync(0xffffffffu, gv, 1);
-                                    gl = (lane == 0) ? ge : gl;
-                                    gr = (lane == 31) ? ge : gr;
-                                    ft[a] = fma(lx0, gl, fma(lx1, gv, lx2 * gr));
-                                }
-                                if constexpr (Is16<S>::value) ft[a] = vmul(ft[a], vsplat<T>(sc));
-                            } else {
+                        });
+                    } else {
+                        static_for<0, K>([&](auto jc) {
+                            constexpr int j = decltype(jc)::value;
+                            constexpr int a = grp * K + j;
+                            if constexpr (a < Q) {
                                 constexpr int ex = VS::ex(a);
+                                const R sc = load_scale<S, R>(A.tab, a);
                                 const int r = (x0 - ex + kGhostX) & (AL - 1);
-                                const S* p = box + trow * BW + r + lane * V;
+                                const S* p = reinterpret_cast<const S*>(st + j * SLOT) + trow * BW + r + lane * V;
                                 if constexpr (V == 2 && (ex % 2 == 0)) {
                                     R v0, v1;
                                     sld2<S, R>(p, sc, v0, v1);
@@ -2070,8 +2114,8 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                                     ft[a] = sld1<S, R>(p, sc);
                                 }
                             }
-                        }
-                    });
+                        });
+                    }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&empty[st_i]);
                 }
@@ -2140,7 +2184,7 @@ __global__ void __launch_bounds__(256) lb_init_kernel(const __grid_constant__ Ar
         const R th = A.isothermal ? R(0) : (R)(T - 1.0);
         equilibrium_dev<VS, N, R>(A.tab, drho, (R)rho, (R)ux, (R)uy, th, [&](auto ac, R deq) {
             constexpr int a = decltype(ac)::value;
-            store_cell<S, R>(A, dst + (long long)a * A.plane + A.origin, x, y, deq, store_scale<S, R>(A.tab, a));
+            store_cell<VS, S, R>(A, dst, a, x, y, deq, store_scale<S, R>(A.tab, a));
         });
     }
 }
@@ -2178,6 +2222,7 @@ cudaError_t launch_typed(const Launch& L) {
     constexpr bool kSplit = std::is_same<S, double>::value && !VS::kOnLattice;
     if (L.kind == kQueryShape) {
         Shape* sh = static_cast<Shape*>(const_cast<void*>(L.args));
+        sh->vw = Layout<VS, S>::VW;
         sh->V = C::V;
         sh->tw = L.upwind ? 32 * C::V : C::TW;
         sh->rows = C::ROWS;
