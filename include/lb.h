@@ -426,8 +426,8 @@ lb_status lb_solve_static(const lb_instance_desc *desc, lb_precision precision,
  * queued as they arrive; each lb_server_step admits queued requests while the
  * device-memory budget allows, advances every admitted request by one chunk of
  * levels (small requests as slots of one continuously batched persistent
- * launch, large ones as lattices of their own on a second stream, so the two
- * kinds overlap on the device), and retires the finished ones with their FP64
+ * launch, large ones as lattices on streams of their own, so that all of them
+ * overlap on the device), and retires the finished ones with their FP64
  * decay-rate fit.  Finished requests are collected with lb_server_poll.
  * ------------------------------------------------------------------------- */
 typedef struct lb_server lb_server;

@@ -1,6 +1,6 @@
 // C-ABI of the request loop (lb_server_*): a FIFO queue, admission by device
 // memory, continuous batching of small requests in one lb_batch, large
-// requests on lattices of their own (second stream), retirement with FP64
+// requests on lattices of their own (a stream each), retirement with FP64
 // decay fits.
 #include <cuda_runtime.h>
 
@@ -73,7 +73,6 @@ double shear_ratio(const std::vector<double>& amp, const std::vector<double>& sh
 struct lb_server {
     lb_server_params p{};
     lb_batch* batch = nullptr;
-    cudaStream_t large_stream = nullptr;
     std::deque<lb_request> queue;
     std::vector<SmallJob> small;
     std::vector<LargeJob> large;
@@ -114,7 +113,9 @@ lb_status admit_large(lb_server* s, const lb_request& r, double now, bool* admit
     lp.precision = s->p.batch.precision;
     lp.kn_convention = s->p.batch.kn_convention;
     lp.diag_capacity = r.desc.max_steps + 2;
-    lp.stream = s->large_stream;
+    // a stream of its own (the handle's): the levels of one lattice follow one another, and while one
+    // waits for its last blocks, its launch and its first loads another one's level has the SMs
+    lp.stream = nullptr;
     lb_handle* h = nullptr;
     lb_status st = lb_create_ex(&lp, &h);
     if (st != LB_OK) return s->fail(st, std::string("large request: ") + lb_last_error(nullptr));
@@ -155,15 +156,9 @@ lb_status lb_server_create(const lb_server_params* p, lb_server** out) {
     lb_server* s = new (std::nothrow) lb_server();
     if (!s) return LB_ERR_NOMEM;
     s->p = *p;
-    if (cudaStreamCreateWithFlags(&s->large_stream, cudaStreamNonBlocking) != cudaSuccess) {
-        delete s;
-        g_server_error = "stream creation";
-        return LB_ERR_CUDA;
-    }
     const lb_status st = lb_batch_create(&p->batch, &s->batch);
     if (st != LB_OK) {
         g_server_error = std::string("batch: ") + lb_batch_last_error(nullptr);
-        cudaStreamDestroy(s->large_stream);
         delete s;
         return st;
     }
@@ -175,7 +170,6 @@ lb_status lb_server_destroy(lb_server* s) {
     if (!s) return LB_OK;
     for (auto& j : s->large) lb_destroy(j.h);
     lb_batch_destroy(s->batch);
-    cudaStreamDestroy(s->large_stream);
     delete s;
     return LB_OK;
 }
