@@ -435,7 +435,7 @@ __device__ __forceinline__ typename PairOf<S>::E to_storage_pair(f2 v, f2 si, ui
 // ------------------------------------------------------------ configuration
 // Launch shapes, from sweeps at 4096^2 (FP32, N = 3) and 2048^2 (D2Q64, N = 4):
 //  * Lax-Wendroff (Gauss-Hermite product) sets: one cell per lane and many warps
-//    (19 consumer rows, or 15 for q = 64), 6 velocities per TMA stage (12 for q = 64);
+//    (19 consumer rows, or 15 and 11 for q = 64), stages of 6 velocities to a whole tile;
 //  * exact-shift sets: two cells per lane (packed f32x2), 11 consumer rows (13 for
 //    q <= 25), 18 velocities per stage.
 // The plain-load kernel takes the same cells per lane as the TMA-staged one, so the
@@ -464,11 +464,8 @@ __device__ __forceinline__ typename PairOf<S>::E to_storage_pair(f2 v, f2 si, ui
 #ifndef LB_TMA_EVICT_LAST
 #define LB_TMA_EVICT_LAST 1  // TMA loads keep their lines in L2 for the neighbouring tiles (-3 % DRAM reads)
 #endif
-#ifndef LB_TMA_HALO
-#define LB_TMA_HALO -1  // -1: per set and storage (see TmaCfg), 0: never, 1: always
-#endif
 #ifndef LB_TMA_NS_TILES
-#define LB_TMA_NS_TILES 2  // ring depth cap, in tiles of stages
+#define LB_TMA_NS_TILES 0  // ring depth cap, in tiles of stages (0: see TmaCfg)
 #endif
 #ifndef LB_TMA_SMEM
 #define LB_TMA_SMEM (200 * 1024)
@@ -548,34 +545,46 @@ struct TmaCfg {
     // (exact shift at 4096^2 FP32, 11 / 13 rows, GLUPS: D2Q37 18.3 / 16.8, D2Q25 21.3 / 22.3,
     // D2Q21 25.4 / 27.7, D2Q17 41.6 / 42.1, D2Q16 44.7 / 45.1, D2Q9 68.6 / 72.6)
     static constexpr int CW = WIDE ? (LB_TMA_WIDE_WARPS > 0 ? LB_TMA_WIDE_WARPS : (VS::Q > 40 ? 14 : 18))
-                                   : (LB_TMA_ROWS > 0 ? LB_TMA_ROWS : (LW ? (VS::Q > 40 ? 15 : 19) : (VS::Q > 30 ? 11 : 13)));
+                                   : (LB_TMA_ROWS > 0 ? LB_TMA_ROWS
+                                      : !LW           ? (VS::Q > 30 ? 11 : 13)
+                                      : VS::Q > 40    ? (sizeof(S) == 2 ? 11 : 15)
+                                                      : 19);
     static constexpr int WPR = WIDE ? 2 : 1;            // consumer warps per tile row
     static constexpr int ROWS = CW / WPR;               // lattice rows of a tile
     static_assert(CW % WPR == 0, "whole tile rows");
     static constexpr int TW = 32 * V;
-    // Edge lanes as halo lanes (30 cells a row) and a per-tile barrier of the consumer warps,
-    // chosen per set and storage by the sweep at 4096^2 / 2048^2 (GLUPS, no halo / halo /
-    // halo + barrier): D2Q16 FP32 29.5 / 35.5 / 30.4; D2Q36 FP32 12.5 / 9.6 / 14.5; D2Q36
-    // 16-bit 12.1 / 15.9 / 14.4; D2Q64 FP32 5.38 / 4.95 / 4.97; D2Q64 16-bit 4.37 / 6.40 / 6.28.
-    static constexpr bool FP32_Q64 = sizeof(S) == 4 && VS::Q > 40;
-    static constexpr bool HALO = WIDE || (!UPW && LW && V == 1 && (LB_TMA_HALO > 0 || (LB_TMA_HALO < 0 && !FP32_Q64)));
-    // (store-staged: no per-tile barrier; without per-velocity stores the warps stay together,
-    // and the barrier cost 5 %: 16.3 against 17.2 GLUPS for D2Q36-GH FP32 at 4096^2)
+    // Edge lanes as halo lanes: 30 cells a row (D2Q64-GH FP32 at 2048^2, us a level: 32 cells and an
+    // extra column's reads 405, halo lanes 372; FP16 555 / 469).
+    static constexpr bool HALO = LW && V == 1 && !UPW;
+    // A per-tile barrier of the consumer warps keeps the ring's stages together where many warps store
+    // for themselves; the store-staged kernel loses by it (16.3 against 17.2 GLUPS for D2Q36-GH FP32
+    // at 4096^2), and so do the other sets.
     static constexpr bool TILE_SYNC =
-        LB_TMA_TILE_SYNC > 0 || (LB_TMA_TILE_SYNC < 0 && !WIDE && (HALO || UPW) && sizeof(S) == 4 && VS::Q == 36);
+        LB_TMA_TILE_SYNC > 0 || (LB_TMA_TILE_SYNC < 0 && !WIDE && LW && sizeof(S) == 4 && VS::Q == 36);
     static constexpr int WCELLS = UPW ? 28 : (HALO ? 30 : TW);  // cells a warp produces
     static constexpr int TWO = WPR * WCELLS;            // cells a tile row produces
     static constexpr int GX = UPW ? 2 : 1;              // stencil reach (columns and rows) of the box
     static constexpr int BAND = LB_TMA_BAND >= 0 ? LB_TMA_BAND : (LW ? 0 : LB_TMA_BAND_SHIFT);  // tile order
     static constexpr int AL = 16 / EB;                  // TMA x coordinates are multiples of 16 bytes
     static_assert(!WIDE || TWO % AL == 0, "store-staged tile rows are whole 16-byte granules");
-    static constexpr int BW = WIDE ? TWO + 2 * AL : ((HALO || UPW) ? 32 + AL : (LW ? TW + 2 * AL : TW + AL));
+    static constexpr int BW = WIDE ? TWO + 2 * AL : (LW ? 32 + AL : TW + AL);
     static constexpr int BH = LW ? ROWS + 2 * GX : ROWS;
     static constexpr int BOX = BW * BH;                 // elements of one plane's box
     // stride of the planes' slots in a stage: dense for one 3-D box (Lax-Wendroff),
     // 128-byte aligned for separate boxes (exact shift)
     static constexpr int SLOT = LW ? BOX : ((BOX * EB + 127) / 128 * 128) / EB;
-    static constexpr int K = LB_TMA_K > 0 ? LB_TMA_K : (LW ? (VS::Q > 40 ? 12 : 6) : 18);  // velocities per stage
+    // Velocities per stage, in us a level: 16-bit sets take a whole tile a stage (D2Q64-GH 2048^2, 15
+    // rows: 12 / 16 / 32 / 64 velocities 469 / 445 / 418 / 391, with 11 rows and no spills 382;
+    // D2Q36-GH 4096^2 6 / 12 / 18 / 36 889 / 819 / 814 / 811; D2Q16-GH 4096^2 6 / 8 / 16 453 / 432 /
+    // 411), FP32 D2Q16-GH 8 (4096^2 and 2502 x 1251, 6 / 8 / 16: 388 / 364 / 361 and 83.7 / 79.2 / 80.0,
+    // three tiles of stages), D2Q64-GH 16 (2048^2, 8 / 12 / 16: 391 / 372 / 369), store-staged D2Q36-GH 6
+    // (4096^2, 6 / 12 / 18: 818 / 818 / 821).
+    static constexpr int K = LB_TMA_K > 0          ? LB_TMA_K
+                             : !LW                 ? 18
+                             : WIDE || UPW         ? (VS::Q > 40 ? 12 : 6)
+                             : sizeof(S) == 2      ? VS::Q
+                             : VS::Q > 40          ? 16
+                                                   : (VS::Q > 16 ? 6 : 8);
     static_assert(K % VW == 0, "whole elements per stage");
     static constexpr int KE = K / VW;                   // planes per stage
     static constexpr int NG = (VS::Q + K - 1) / K;      // stages per tile
@@ -583,7 +592,9 @@ struct TmaCfg {
     // output tile of the store-staged kernel: [plane][row][TWO cells]
     static constexpr int OUT_BYTES = WIDE ? (Layout<VS, S>::PLANES * ROWS * TWO * EB + 127) / 128 * 128 : 0;
     static constexpr int NS_FIT = ((WIDE ? LB_TMA_WIDE_SMEM - OUT_BYTES : LB_TMA_SMEM) - 512) / STAGE_BYTES;
-    static constexpr int NS = NS_FIT < LB_TMA_NS_TILES * NG ? NS_FIT : LB_TMA_NS_TILES * NG;
+    static constexpr int NS_TILES = LB_TMA_NS_TILES > 0 ? LB_TMA_NS_TILES
+                                    : LW && !WIDE && !UPW && VS::Q == 16 ? (sizeof(S) == 2 ? 4 : 3) : 2;
+    static constexpr int NS = NS_FIT < NS_TILES * NG ? NS_FIT : NS_TILES * NG;
     static constexpr int THREADS = 32 * (CW + 1);       // + one producer warp
     // registers a thread may hold: each SM sub-partition's 16384 registers are shared by
     // ceil(warps / 4) warps of the block (255 for 8 warps, 168 for 9..12, 128 for 13..16)
@@ -2020,12 +2031,10 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
             using T = typename Pack<R, V>::T;
             T ft[Q];
             bool ok = !*abort_flag;
-            // Lax-Wendroff: column of this lane's first cell in the box row, and the column
-            // whose y-pass the two warp-edge lanes need (x0 - 1 for lane 0, x0 + TW for lane 31)
-            // (store-staged: the box starts AL columns left of the tile row)
+            // Lax-Wendroff: the lane's column in the box row (column x0 - 1 for lane 0; store-staged: the
+            // box starts AL columns left of the tile row)
             const int r_lw = WIDE ? AL - 1 + half * C::WCELLS : (x0 - 1 + kGhostX) & (AL - 1);
-            const int c_lw = C::HALO ? r_lw + lane : r_lw + 1 + lane;
-            const int ce_lw = (lane == 31) ? r_lw + 1 + TW : r_lw;
+            const int c_lw = r_lw + lane;
             static_for<0, NG>([&](auto gc) {
                 constexpr int grp = decltype(gc)::value;
                 if (ok) {
@@ -2078,15 +2087,7 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                                         return lw_y_pair<VS, a>(A.tab, lds_pair<S>(rm), lds_pair<S>(rm + BW),
                                                                 lds_pair<S>(rm + 2 * BW));
                                     };
-                                    const f2 gv = column(c_lw);
-                                    f2 gl = shfl_up2(gv), gr = shfl_down2(gv);
-                                    if constexpr (!C::HALO) {
-                                        // all 32 lanes own cells: the edge lanes take their outer
-                                        // column's y pass from an extra read
-                                        const f2 ge = column(ce_lw);
-                                        gl = lane == 0 ? ge : gl;
-                                        gr = lane == 31 ? ge : gr;
-                                    }
+                                    const f2 gv = column(c_lw), gl = shfl_up2(gv), gr = shfl_down2(gv);
                                     v = lw_x_pair<VS, a>(A.tab, gl, gv, gr);
                                 }
                                 if constexpr (Is16<S>::value)
@@ -2288,6 +2289,7 @@ cudaError_t launch_typed(const Launch& L) {
                     sh->st_smem = TS::SMEM;
                     sh->st_box_w = TS::BW;
                     sh->st_box_h = TS::BH;
+                    sh->st_box_d = TS::BOX_D;
                     // measured at 4096^2 (GLUPS, TMA-staged / store-staged): D2Q36-GH N = 3 13.8 /
                     // 16.2, N = 2 11.4 / 16.9, N = 1 9.8 / 18.1; D2Q16-GH N = 2 38.2 / 31.5
                     sh->st_auto = (sizeof(S) == 4 && VS::Q > 16) ? 1 : 0;
