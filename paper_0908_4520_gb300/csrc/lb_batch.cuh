@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(kBatchMaxWarps * 32) lb_batch_kernel(const __g
         if (!Qu.order) continue;
         const int n = *Qu.n;
         if (n == 0) continue;
+        if (G.ctas > 1) G.sync();  // every CTA of the cluster runs before its shared memory is written
         for (;;) {
             if (G.wid == 0 && lane == 0) {
                 const int i = atomicAdd(Qu.next, 1);
