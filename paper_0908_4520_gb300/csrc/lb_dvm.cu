@@ -25,8 +25,8 @@
 //     P_{s+1} = u_{s+1} + c1 sin x + (G' - u') d^2   (c1, c2: the force over the half levels),
 //   and P is the state that is kept and advected.
 // A warp of its own sums the records and takes the force integrals (FP64 sine), 32 levels at a time.
-// Measured (us a level): seven instances of 20 nodes x 128 columns 2.8, against 65 with one CTA an
-// instance, ~15 operations a value, sines in every level and 2 n barriers; one of them 2.8, forty 4.4.
+// Measured (us a level): seven instances of 20 nodes x 128 columns 2.6, against 65 with one CTA an
+// instance, ~15 operations a value, sines in every level and 2 n barriers; one of them 2.4, forty 4.3.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -46,9 +46,10 @@ constexpr int kDvmThreads = 32 * (kDvmWarps + 1);
 constexpr int kDvmNodes = 8;         // nodes a lane holds at most
 constexpr int kDvmMaxCluster = 8;
 #ifndef LB_DVM_FILL
-// lanes of a CTA that the columns fill at least (two warps), where the nodes allow: the sums over the
-// nodes cost a lane more the fewer nodes it holds
-#define LB_DVM_FILL 64
+// lanes of a CTA that the columns fill at least, where the nodes allow: four warps, one for each of the
+// SM's FP64 units (us a level of 20 nodes x 128 columns, seven instances, 64 / 128 / 256: 2.90 / 2.58 /
+// 2.59)
+#define LB_DVM_FILL 128
 #endif
 constexpr int kDvmFill = LB_DVM_FILL;
 constexpr int kDvmForceLevels = 32;  // levels of force integrals taken at a time (one a lane)
@@ -270,7 +271,7 @@ lb_status lb_dvm_run_forced(int n_inst, const double* tau, int n_nodes, int nx, 
     int nc = 1;
     auto shape = [&]() {
         A.max_cols = (nx + nc - 1) / nc;
-        // lanes a column: enough for kDvmNodes nodes a lane, then up to two warps of the CTA
+        // lanes a column: enough for kDvmNodes nodes a lane, then up to four warps of the CTA
         A.kg = 1;
         while (A.kg * kDvmNodes < n_nodes || (A.kg < 8 && 2 * A.kg <= n_nodes && A.max_cols * A.kg < kDvmFill)) A.kg *= 2;
         for (A.log_kg = 0; (1 << A.log_kg) < A.kg;) ++A.log_kg;
