@@ -458,9 +458,6 @@ __device__ __forceinline__ typename PairOf<S>::E to_storage_pair(f2 v, f2 si, ui
 #ifndef LB_TMA_K
 #define LB_TMA_K 0
 #endif
-#ifndef LB_TMA_TILE_SYNC
-#define LB_TMA_TILE_SYNC -1  // -1: per set and storage (see TmaCfg), 0: never, 1: always
-#endif
 #ifndef LB_TMA_EVICT_LAST
 #define LB_TMA_EVICT_LAST 1  // TMA loads keep their lines in L2 for the neighbouring tiles (-3 % DRAM reads)
 #endif
@@ -556,11 +553,9 @@ struct TmaCfg {
     // Edge lanes as halo lanes: 30 cells a row (D2Q64-GH FP32 at 2048^2, us a level: 32 cells and an
     // extra column's reads 405, halo lanes 372; FP16 555 / 469).
     static constexpr bool HALO = LW && V == 1 && !UPW;
-    // A per-tile barrier of the consumer warps keeps the ring's stages together where many warps store
-    // for themselves; the store-staged kernel loses by it (16.3 against 17.2 GLUPS for D2Q36-GH FP32
-    // at 4096^2), and so do the other sets.
-    static constexpr bool TILE_SYNC =
-        LB_TMA_TILE_SYNC > 0 || (LB_TMA_TILE_SYNC < 0 && !WIDE && LW && sizeof(S) == 4 && VS::Q == 36);
+    // (No per-tile barrier of the consumer warps, which would keep the ring's stages together: with
+    // populations in pairs D2Q36-GH FP32 takes 965 us a level with it and 838 without at 4094 x 4096,
+    // upwind at 2048^2 271 and 224.)
     static constexpr int WCELLS = UPW ? 28 : (HALO ? 30 : TW);  // cells a warp produces
     static constexpr int TWO = WPR * WCELLS;            // cells a tile row produces
     static constexpr int GX = UPW ? 2 : 1;              // stencil reach (columns and rows) of the box
@@ -577,14 +572,14 @@ struct TmaCfg {
     // rows: 12 / 16 / 32 / 64 velocities 469 / 445 / 418 / 391, with 11 rows and no spills 382;
     // D2Q36-GH 4096^2 6 / 12 / 18 / 36 889 / 819 / 814 / 811; D2Q16-GH 4096^2 6 / 8 / 16 453 / 432 /
     // 411), FP32 D2Q16-GH 8 (4096^2 and 2502 x 1251, 6 / 8 / 16: 388 / 364 / 361 and 83.7 / 79.2 / 80.0,
-    // three tiles of stages), D2Q64-GH 16 (2048^2, 8 / 12 / 16: 391 / 372 / 369), store-staged D2Q36-GH 6
-    // (4096^2, 6 / 12 / 18: 818 / 818 / 821).
+    // three tiles of stages), D2Q36-GH 12 (4094 x 4096, 6 / 12 / 18: 838 / 786 / 793), D2Q64-GH 16 (2048^2,
+    // 8 / 12 / 16: 391 / 372 / 369), store-staged D2Q36-GH 6 (4096^2, 6 / 12 / 18: 818 / 818 / 821).
     static constexpr int K = LB_TMA_K > 0          ? LB_TMA_K
                              : !LW                 ? 18
                              : WIDE || UPW         ? (VS::Q > 40 ? 12 : 6)
                              : sizeof(S) == 2      ? VS::Q
                              : VS::Q > 40          ? 16
-                                                   : (VS::Q > 16 ? 6 : 8);
+                                                   : (VS::Q > 16 ? 12 : 8);
     static_assert(K % VW == 0, "whole elements per stage");
     static constexpr int KE = K / VW;                   // planes per stage
     static constexpr int NG = (VS::Q + K - 1) / K;      // stages per tile
@@ -2147,13 +2142,6 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                                                         R(0));
             }
             if (diag && (ti % kDiagFold) == kDiagFold - 1) fold_diag(acc, wsum[warp], lane);  // warp-uniform
-            if constexpr (C::TILE_SYNC) {
-                // keep the consumer warps within one tile of each other, so a stage is
-                // released (and refilled) as soon as the last of them has read it; every
-                // consumer warp reaches this barrier once per tile (its waits are bounded)
-                asm volatile("bar.sync 1, %0;" ::"r"(CW * 32) : "memory");
-                if (*abort_flag) ok = false;
-            }
             if (!ok) break;
         }
     }
