@@ -9,7 +9,7 @@ CUDA runtime.  Rebuilds only what changed.
 Supported build options (environment variables):
 
 * ``LB_EXTRA_NVCC``: extra nvcc flags for every unit, e.g. the launch-shape
-  overrides of ``csrc/lb_kernels.cuh`` (``-DLB_TMA_K=9``, ``-DLB_TMA_BAND=0``,
+  overrides of ``csrc/lb_kernels.cuh`` (``-DLB_TMA_K=12``, ``-DLB_TMA_BAND=0``,
   ``-DLB_TMA_WIDE_SMEM=...``; each macro there states its default and what was
   measured for it);
 * ``LB_BUILD_TAG``: build into ``_build_<tag>/`` and ``liblb_<tag>.so`` instead,

@@ -371,11 +371,11 @@ lb_status encode_maps(lb_handle* h) {
     if (h->use_st) {
         // loads: the whole padded buffer, the store-staged kernel's box; stores: the nx x ny
         // cells of each buffer (the rim is written by the kernel's own image stores), one
-        // tile of all q velocities per store
+        // warp's row segment of all planes per store
         const cuuint32_t lbox[3] = {(cuuint32_t)h->shape.st_box_w, (cuuint32_t)h->shape.st_box_h,
                                     (cuuint32_t)h->shape.st_box_d};
         const cuuint64_t odims[3] = {(cuuint64_t)h->p.nx, (cuuint64_t)h->p.ny, (cuuint64_t)h->planes()};
-        const cuuint32_t obox[3] = {(cuuint32_t)h->shape.st_tw, (cuuint32_t)h->shape.st_rows, (cuuint32_t)h->planes()};
+        const cuuint32_t obox[3] = {(cuuint32_t)h->shape.st_cells, 1, (cuuint32_t)h->planes()};
         for (int i = 0; i < 2; ++i) {
             CUresult r = enc(&h->tmap_stl[i], dt, 3, h->buf[i], dims, strides, lbox, estr,
                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,

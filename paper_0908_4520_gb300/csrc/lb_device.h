@@ -120,8 +120,8 @@ struct Shape {
     int tma_tw;     // cells a tile row produces (32 V, or 30 with halo lanes)
     int box_w, box_h, box_d;  // tensor-map box (x, y, planes)
     // store-staged TMA kernel (0 = not built for this unit): tile of st_rows x st_tw cells,
-    // load box st_box_w x st_box_h x st_box_d, one store box st_tw x st_rows x all planes per tile
-    int st, st_tw, st_rows, st_threads, st_smem, st_occupancy, st_box_w, st_box_h, st_box_d;
+    // load box st_box_w x st_box_h x st_box_d, store boxes of st_cells x 1 x all planes, one a warp
+    int st, st_cells, st_tw, st_rows, st_threads, st_smem, st_occupancy, st_box_w, st_box_h, st_box_d;
     // node-split FP64 kernel (split_cells = 0: not built for this unit): cells of a warp, and the
     // FP64 operations of a warp of it and of the plain-load kernel
     int split_cells, split_ops, plain_ops;

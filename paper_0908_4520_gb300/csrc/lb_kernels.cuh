@@ -31,7 +31,7 @@
 // neighbours and sit in L2.  Populations carry a rim of periodic images (ghost columns and
 // rows), rewritten by every store, so no read ever wraps.
 //
-// Two step kernels share the collision code and give bitwise-identical results:
+// Three step kernels share the collision code and give bitwise-identical results:
 //  * lb_tma_step_kernel (the hot path): one producer warp streams, per group of
 //    velocities, the tile's source box (with its halo) from HBM into a ring of
 //    shared-memory stages with cp.async.bulk.tensor, completion tracked by
@@ -40,6 +40,8 @@
 //    on expiry the kernel flags LB_ERR_TIMEOUT in the status word and returns.
 //  * lb_fused_kernel: plain coalesced loads from global memory (moments read-back,
 //    the first level, FP64 storage and grids too small for the TMA tiles).
+//  * lb_split_kernel: FP64 Lax-Wendroff steps of grids that leave FP64 units idle, a lane
+//    for every x node of a cell.
 #pragma once
 
 #include <cuda.h>
@@ -471,10 +473,9 @@ __device__ __forceinline__ typename PairOf<S>::E to_storage_pair(f2 v, f2 si, ui
 #define LB_TMA_MINB 1
 #endif
 #ifndef LB_TMA_BAND
-// TMA kernel tile order: -1 per set, 0 row-major, B > 0 column-major in bands of B tile rows.
-// Measured at 4096^2 FP32 (same box; row-major / bands of 4, 8, 16): D2Q37 12.6 / 18.2 / 16.7 /
-// 14.6 GLUPS, D2Q36-GH 14.8 / 7.7 / 7.6 / 7.4, D2Q16-GH 38.5 / 35.3 / 32.4 / 31.2, D2Q36-GH FP16
-// 16.8 / 15.6 / 11.8 / 14.8: bands for the exact-shift sets, row-major for Lax-Wendroff
+// TMA kernel tile order: -1 per set, 0 row-major, B > 0 column-major in bands of B tile rows: bands for
+// the exact-shift sets, whose boxes are displaced by up to max|e| rows (row-major order cost D2Q37 a third
+// of its rate at 4096^2), row-major for Lax-Wendroff (bands cost up to half)
 #define LB_TMA_BAND -1
 #endif
 #ifndef LB_TMA_BAND_SHIFT
@@ -487,16 +488,13 @@ __device__ __forceinline__ typename PairOf<S>::E to_storage_pair(f2 v, f2 si, ui
 #define LB_TMA_WIDE_WARPS 0  // consumer warps of the store-staged kernel (two per tile row); 0: 18, q = 64: 14
 #endif
 #ifndef LB_TMA_WIDE_SMEM
-// ring + output tile of the store-staged kernel.  D2Q36-GH FP32 at 4096^2 (GLUPS): 224 KB
-// (8 stages) 17.2, 192 KB (6 stages: one tile ahead) 17.5; 9 velocities per stage instead of 6:
-// +0.2 %; 16 / 20 consumer warps instead of 18: 15.0 / 15.9
+// ring + output slots of the store-staged kernel (D2Q36-GH FP32 at 4096^2: 192 and 224 KB 774 us a level)
 #define LB_TMA_WIDE_SMEM (192 * 1024)
 #endif
 #ifndef LB_DIAG_PREFETCH
-// load sin/cos of the diagnostics before the collision: -1 per set and kernel (measured at
-// 4096^2 FP32, same box: TMA kernel with plain stores D2Q16-GH 35.7 -> 38.5 GLUPS, D2Q37
-// 12.6 -> 12.6, D2Q36-GH 14.8 -> 11.8; store-staged kernel D2Q36-GH 17.44 -> 17.91; so
-// D2Q16-GH and the store-staged kernel), 0 never, 1 always
+// load sin/cos of the diagnostics before the collision: -1 per set and kernel, 0 never, 1 always.  Taken
+// for D2Q16-GH (35.7 -> 38.5 GLUPS at 4096^2 when the stores were of single velocities) and the
+// store-staged kernel (17.4 -> 17.9); D2Q37 and D2Q64-GH lost 1 to 2 % by it
 #define LB_DIAG_PREFETCH -1
 #endif
 
@@ -523,12 +521,14 @@ struct Cfg {
 // UPW: second-order upwind streaming of a Lax-Wendroff set (one cell per lane): lanes
 // 0, 1 and 30, 31 compute the y pass of the two columns on either side of the 28 cells
 // that lanes 2..29 own, and the box carries two extra rows above and below.
-// WIDE: the store-staged variant of the Lax-Wendroff kernel (one cell per lane, halo
-// lanes): two warps share a tile row (30 cells each, 60 velocity pairs per row: whole 16-byte TMA
-// granules), the consumer warps write the relaxed populations of the tile (16-bit: stochastically
-// rounded) into a shared-memory output tile, and the producer warp writes it to HBM with
-// one TMA tensor store per tile (cp.async.bulk.tensor, shared -> global), so no thread
-// issues per-velocity global stores and every DRAM sector of the tile is written whole.
+// WIDE: the store-staged variant of the Lax-Wendroff kernel (one cell per lane, halo lanes): two warps
+// share a tile row (FP32: 30 cells each; 16-bit: 28 each, lanes 29 to 31 idle: a warp's row segment is
+// whole 16-byte TMA granules), and each consumer warp writes its relaxed populations (16-bit:
+// stochastically rounded) into a slot of its own in shared memory and from there to HBM with one TMA
+// tensor store (cp.async.bulk.tensor, shared -> global), so no lane issues per-velocity global stores.
+// A warp waits only for its own store of the tile before: one store of the whole tile by the producer
+// made every warp wait for the slowest one's tile and for that store.  D2Q36-GH FP32 at 4096^2: 820 -> 774 us
+// a level (5.89 -> 6.25 TB/s), 1024^2 69 -> 66.
 template <class VS, class S, bool UPW = false, bool WIDE = false>
 struct TmaCfg {
     static constexpr bool LW = !VS::kOnLattice;
@@ -556,12 +556,12 @@ struct TmaCfg {
     // (No per-tile barrier of the consumer warps, which would keep the ring's stages together: with
     // populations in pairs D2Q36-GH FP32 takes 965 us a level with it and 838 without at 4094 x 4096,
     // upwind at 2048^2 271 and 224.)
-    static constexpr int WCELLS = UPW ? 28 : (HALO ? 30 : TW);  // cells a warp produces
+    static constexpr int WCELLS = UPW || (WIDE && sizeof(S) == 2) ? 28 : (HALO ? 30 : TW);  // cells a warp produces
     static constexpr int TWO = WPR * WCELLS;            // cells a tile row produces
     static constexpr int GX = UPW ? 2 : 1;              // stencil reach (columns and rows) of the box
     static constexpr int BAND = LB_TMA_BAND >= 0 ? LB_TMA_BAND : (LW ? 0 : LB_TMA_BAND_SHIFT);  // tile order
     static constexpr int AL = 16 / EB;                  // TMA x coordinates are multiples of 16 bytes
-    static_assert(!WIDE || TWO % AL == 0, "store-staged tile rows are whole 16-byte granules");
+    static_assert(!WIDE || WCELLS % AL == 0, "store-staged row segments are whole 16-byte granules");
     static constexpr int BW = WIDE ? TWO + 2 * AL : (LW ? 32 + AL : TW + AL);
     static constexpr int BH = LW ? ROWS + 2 * GX : ROWS;
     static constexpr int BOX = BW * BH;                 // elements of one plane's box
@@ -573,7 +573,7 @@ struct TmaCfg {
     // D2Q36-GH 4096^2 6 / 12 / 18 / 36 889 / 819 / 814 / 811; D2Q16-GH 4096^2 6 / 8 / 16 453 / 432 /
     // 411), FP32 D2Q16-GH 8 (4096^2 and 2502 x 1251, 6 / 8 / 16: 388 / 364 / 361 and 83.7 / 79.2 / 80.0,
     // three tiles of stages), D2Q36-GH 12 (4094 x 4096, 6 / 12 / 18: 838 / 786 / 793), D2Q64-GH 16 (2048^2,
-    // 8 / 12 / 16: 391 / 372 / 369), store-staged D2Q36-GH 6 (4096^2, 6 / 12 / 18: 818 / 818 / 821).
+    // 8 / 12 / 16: 391 / 372 / 369), store-staged D2Q36-GH 6 (4096^2, 4 / 6 / 18: 820 / 774 / 804).
     static constexpr int K = LB_TMA_K > 0          ? LB_TMA_K
                              : !LW                 ? 18
                              : WIDE || UPW         ? (VS::Q > 40 ? 12 : 6)
@@ -584,8 +584,9 @@ struct TmaCfg {
     static constexpr int KE = K / VW;                   // planes per stage
     static constexpr int NG = (VS::Q + K - 1) / K;      // stages per tile
     static constexpr int STAGE_BYTES = (KE * SLOT * EB + 127) / 128 * 128;
-    // output tile of the store-staged kernel: [plane][row][TWO cells]
-    static constexpr int OUT_BYTES = WIDE ? (Layout<VS, S>::PLANES * ROWS * TWO * EB + 127) / 128 * 128 : 0;
+    // output slot of a warp of the store-staged kernel: [plane][WCELLS cells]
+    static constexpr int OUT_SLOT = (Layout<VS, S>::PLANES * WCELLS * EB + 127) / 128 * 128;
+    static constexpr int OUT_BYTES = WIDE ? CW * OUT_SLOT : 0;
     static constexpr int NS_FIT = ((WIDE ? LB_TMA_WIDE_SMEM - OUT_BYTES : LB_TMA_SMEM) - 512) / STAGE_BYTES;
     static constexpr int NS_TILES = LB_TMA_NS_TILES > 0 ? LB_TMA_NS_TILES
                                     : LW && !WIDE && !UPW && VS::Q == 16 ? (sizeof(S) == 2 ? 4 : 3) : 2;
@@ -596,8 +597,8 @@ struct TmaCfg {
     static constexpr int WARPS_PER_SMSP = (CW + 1 + 3) / 4;
     static constexpr int MAXREG_FIT = 16384 / (32 * WARPS_PER_SMSP) / 8 * 8;
     static constexpr int MAXREG = MAXREG_FIT > 255 ? 255 : MAXREG_FIT;
-    // ring, output tile, full/empty barriers of the ring, tile-done and output-free barriers
-    static constexpr int SMEM = NS * STAGE_BYTES + OUT_BYTES + 2 * NS * 8 + 16 + 128;  // + alignment slack
+    // ring, output slots, full/empty barriers of the ring
+    static constexpr int SMEM = NS * STAGE_BYTES + OUT_BYTES + 2 * NS * 8 + 128;  // + alignment slack
     static constexpr int BOX_D = LW ? KE : 1;           // planes per TMA box
 };
 
@@ -661,11 +662,11 @@ struct Lane {
 
 // TMA-staged Lax-Wendroff with one cell per lane: the warp's edge lanes are halo lanes
 // (columns x0 - 1 and x0 + 30), whose y-pass only feeds their neighbours' x-pass, so no
-// lane reads an extra column; lanes 1..30 own cells x0 .. x0 + 29.
-__device__ __forceinline__ Lane halo_lane_geometry(int lane, int x0, int tile_start, int nx) {
+// lane reads an extra column; lanes 1..own own cells x0 .. x0 + own - 1.
+__device__ __forceinline__ Lane halo_lane_geometry(int lane, int x0, int tile_start, int nx, int own = 30) {
     Lane g;
     g.x = x0 - 1 + lane;
-    g.own = lane >= 1 && lane <= 30 && g.x < nx && g.x >= tile_start;
+    g.own = lane >= 1 && lane <= own && g.x < nx && g.x >= tile_start;
     g.xl = g.x;
     return g;
 }
@@ -1100,15 +1101,15 @@ __device__ __forceinline__ CellOut<float> collide_cell_pairs(const Tab<float>& t
 // Collision and store (or the moment outputs) of the V cells (g.x .., y) whose
 // streamed populations are in ft.  Diagnostics are reduced over the warp in
 // FP32 and added to acc (lane 0) in FP64.
-// OSTRIDE > 0 (store-staged kernel, FP32): the relaxed populations go to the output tile in
-// shared memory, out[a * OSTRIDE] for velocity a, instead of to HBM (the periodic images in
-// the ghost rim are still written here, from that tile).
+// OSTRIDE > 0 (store-staged kernel): the relaxed populations go to the warp's output slot in shared
+// memory, out[m * OSTRIDE] for plane m, instead of to HBM (the periodic images in the ghost
+// rim are still written here).
 template <class VS, int N, class S, class R, int V, int KIND, class T, int OSTRIDE = 0>
 __device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], S* dst, int y,
                                               const Lane& g, bool diag, R (&acc)[6], int lane, long long lvl,
                                               R gt, typename Layout<VS, S>::E* out = nullptr) {
     constexpr int Q = VS::Q;
-    static_assert(OSTRIDE == 0 || V == 1, "output tile: one cell per lane");
+    static_assert(OSTRIDE == 0 || V == 1, "output slot: one cell per lane");
     // body force g_y(x_i, t_n) = gt sin(x_i), gt = A_f cos(phi t_n) (driven standing wave, Sec. 4);
     // compiled out of the unforced step kernels
     constexpr bool STEP = (KIND == kStep || KIND == kStepForced);
@@ -1182,7 +1183,7 @@ __device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], 
     }
     if constexpr (STEP) {
         // The relaxed populations, straight from registers: to the cell (OSTRIDE > 0: to the
-        // output tile) and, for the lanes of a boundary, to its periodic images in the ghost rim.
+        // output slot) and, for the lanes of a boundary, to its periodic images in the ghost rim.
         // put(p) writes all planes at offset p of the first; each call draws the 16-bit rounding
         // bits anew from the cell's own stream, so every image holds the cell's bits.
         using E = typename Layout<VS, S>::E;
@@ -1873,32 +1874,22 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
     }
 }
 
-// Store-staged kernel, producer side: wait (bounded) until every consumer warp has written
-// tile `ti` into the output tile, write it to the cells (x0.., y0..) of dst with one TMA
-// tensor store (velocities, rows and columns of the tile; the tensor map clips it at nx and
-// ny), wait until the store has read the output tile, and release it.  False on a timeout.
-__device__ __forceinline__ bool store_tile(const Args<float>& A, const void* otile, uint64_t* tdone, uint64_t* ofree,
-                                           int ti, int x0, int y0) {
-    if (!mbar_wait(tdone, (uint32_t)ti & 1u, A.status)) return false;
+// Store-staged kernel: the warp's output slot to the cells (x.., y) of dst, all planes, with one TMA
+// tensor store (the tensor map clips it at nx).  One lane calls it, once the warp's writes to the slot
+// have been made visible to the async proxy.
+__device__ __forceinline__ void store_strip(const Args<float>& A, const void* slot, int x, int y) {
     asm volatile(
         "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
             reinterpret_cast<uint64_t>(&A.tmap_st)),
-        "r"(smem_u32(otile)), "r"(x0), "r"(y0), "r"(0)
+        "r"(smem_u32(slot)), "r"(x), "r"(y), "r"(0)
         : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-    mbar_arrive(ofree);
-    return true;
 }
 
 // KIND = kStep: one level (store f*, diagnostics, level advance); kMoments: the per-cell
 // moments (and optionally f~) of the current level, nothing stored, no level advance.
 // WIDE (KIND = kStep only): the store-staged variant (see TmaCfg): consumer warp w owns half
-// w % 2 of tile row w / 2; at the end of a tile each consumer warp writes its relaxed cells
-// into the output tile, then arrives on the tile-done barrier; the producer, once it has
-// issued the next tile's loads, waits for that barrier, writes the tile to HBM with one TMA
-// tensor store, waits until the store has read the output tile and releases it (the
-// output-free barrier) for the consumers' next tile.
+// w % 2 of tile row w / 2, and stores it from a shared-memory slot of its own.
 template <class VS, int N, class S, bool UPW = false, int KIND = kStep, bool WIDE = false>
 __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
     lb_tma_step_kernel(const __grid_constant__ Args<float> A) {
@@ -1910,17 +1901,15 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
     constexpr int NS = C::NS, NG = C::NG, K = C::K, BW = C::BW, BOX = C::BOX, SLOT = C::SLOT;
     using E = typename C::E;
     constexpr int STAGE_ELEMS = C::STAGE_BYTES / C::EB, KE = C::KE;
-    constexpr int OSTRIDE = WIDE ? ROWS * C::TWO : 0;  // output tile: elements per plane
+    constexpr int OSTRIDE = WIDE ? C::WCELLS : 0;  // output slot: elements per plane
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     // TMA destinations must be 128-byte aligned: align the base explicitly
     unsigned char* const smem_raw =
         smem_dyn + ((128u - (smem_u32(smem_dyn) & 127u)) & 127u);
     E* const stages = reinterpret_cast<E*>(smem_raw);
-    E* const otile = reinterpret_cast<E*>(smem_raw + NS * C::STAGE_BYTES);
+    unsigned char* const slots = smem_raw + NS * C::STAGE_BYTES;  // store-staged: the warps' output slots
     uint64_t* const full = reinterpret_cast<uint64_t*>(smem_raw + NS * C::STAGE_BYTES + C::OUT_BYTES);
     uint64_t* const empty = full + NS;
-    uint64_t* const tdone = empty + NS;  // store-staged: the consumers have filled the output tile
-    uint64_t* const ofree = tdone + 1;   // store-staged: the output tile may be overwritten
     __shared__ int s_abort;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1929,13 +1918,8 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], CW);
         }
-        if constexpr (WIDE) {
-            mbar_init(tdone, CW);
-            mbar_init(ofree, 1);
-        }
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if constexpr (WIDE) mbar_arrive(ofree);  // phase 0: the output tile starts free
     }
     __syncthreads();
 
@@ -1954,7 +1938,6 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
         // ---------------- producer: one thread streams the boxes of every tile
         if (lane == 0) {
             uint32_t it = 0;
-            int ti = 0, px0 = 0, py0 = 0;  // store-staged: tiles issued, coordinates of the last
             for (int tile = blockIdx.x; tile < A.ntiles && !*abort_flag; tile += gridDim.x) {
                 int ty, tx;
                 tma_tile_coords<C::BAND>(tile, A.ntiles_x, A.ntiles, ty, tx);
@@ -1986,18 +1969,6 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                         }
                     }
                 }
-                if constexpr (WIDE) {
-                    // the previous tile's output, once this tile's loads are on their way
-                    if (ti > 0 && !*abort_flag && !store_tile(A, otile, tdone, ofree, ti - 1, px0, py0)) *abort_flag = 1;
-                    px0 = x0;
-                    py0 = y0;
-                    ++ti;
-                }
-            }
-            if constexpr (WIDE) {
-                if (ti > 0 && !*abort_flag && !store_tile(A, otile, tdone, ofree, ti - 1, px0, py0)) *abort_flag = 1;
-                // every store has written HBM before the block exits
-                asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
             }
             // drain: no box may still be in flight when the block exits
             if (*abort_flag) {
@@ -2013,7 +1984,7 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
         // store-staged: the warp's row of the tile and its half of the row
         const int trow = WIDE ? warp / C::WPR : warp;
         const int half = WIDE ? warp % C::WPR : 0;
-        uint32_t ti = 0;  // tiles processed (store-staged: phase of the output-free barrier)
+        uint32_t ti = 0;  // tiles processed
         for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x, ++ti) {
             int ty, tx;
             tma_tile_coords<C::BAND>(tile, A.ntiles_x, A.ntiles, ty, tx);
@@ -2021,7 +1992,7 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
             const int x0 = (!WIDE && tx == A.ntiles_x - 1) ? A.x0_last : tile_start;
             const int y = ty * ROWS + trow;
             const Lane g = UPW      ? upwind_lane_geometry(lane, x0, tile_start, A.nx)
-                           : C::HALO ? halo_lane_geometry(lane, x0, tile_start, A.nx)
+                           : C::HALO ? halo_lane_geometry(lane, x0, tile_start, A.nx, C::WCELLS)
                                      : lane_geometry<V>(lane, x0, tile_start, A.nx);
             using T = typename Pack<R, V>::T;
             T ft[Q];
@@ -2121,21 +2092,20 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                 }
             });
             if constexpr (WIDE) {
-                // the output tile is free once the producer's store of the previous tile has read it
-                if (ok) {
-                    ok = mbar_wait(ofree, ti & 1u, A.status);
-                    if (!ok) *abort_flag = 1;
-                }
-                if (ok && y < A.ny)
+                unsigned char* const slot = slots + warp * C::OUT_SLOT;
+                const bool stores = __all_sync(0xffffffffu, ok) && y < A.ny && tile_start < A.nx;  // warp-uniform
+                if (stores) {
+                    // the slot is free once the warp's store before has read it
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                    __syncwarp();
                     collide_store<VS, N, S, R, V, KIND, typename Pack<R, V>::T, OSTRIDE>(
                         A, ft, static_cast<S*>(A.dst), y, g, diag, acc, lane, lvl, R(0),
-                        otile + trow * C::TWO + (g.x - tx * C::TWO));
-                // the generic-proxy writes of the tile become visible to the TMA store; a warp
-                // whose wait ran out does not arrive, so the producer's bounded wait runs out
-                // too and no store of the tile is issued
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (ok && lane == 0) mbar_arrive(tdone);
+                        reinterpret_cast<E*>(slot) + (g.x - tile_start));
+                    // the generic-proxy writes of the slot become visible to the TMA store
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) store_strip(A, slot, tile_start, y);
+                }
             } else {
                 if (ok && y < A.ny)
                     collide_store<VS, N, S, R, V, KIND>(A, ft, static_cast<S*>(A.dst), y, g, diag, acc, lane, lvl,
@@ -2143,6 +2113,10 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
             }
             if (diag && (ti % kDiagFold) == kDiagFold - 1) fold_diag(acc, wsum[warp], lane);  // warp-uniform
             if (!ok) break;
+        }
+        if constexpr (WIDE) {  // the warp's stores have written HBM before the block exits
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+            __syncwarp();
         }
     }
     __syncthreads();
@@ -2272,14 +2246,16 @@ cudaError_t launch_typed(const Launch& L) {
                 if (e == cudaSuccess) {
                     sh->st = sh->st_occupancy > 0 ? 1 : 0;
                     sh->st_tw = TS::TWO;
+                    sh->st_cells = TS::WCELLS;
                     sh->st_rows = TS::ROWS;
                     sh->st_threads = TS::THREADS;
                     sh->st_smem = TS::SMEM;
                     sh->st_box_w = TS::BW;
                     sh->st_box_h = TS::BH;
                     sh->st_box_d = TS::BOX_D;
-                    // measured at 4096^2 (GLUPS, TMA-staged / store-staged): D2Q36-GH N = 3 13.8 /
-                    // 16.2, N = 2 11.4 / 16.9, N = 1 9.8 / 18.1; D2Q16-GH N = 2 38.2 / 31.5
+                    // D2Q16-GH and the 16-bit sets are faster with plain stores (4096^2, us a level, plain /
+                    // store-staged: D2Q16-GH FP32 364 / 421, D2Q36-GH FP16 811 / 1005), D2Q36-GH FP32 with
+                    // staged ones (788 at 4094 x 4096 / 774)
                     sh->st_auto = (sizeof(S) == 4 && VS::Q > 16) ? 1 : 0;
                 }
             }
