@@ -488,8 +488,9 @@ __device__ __forceinline__ typename PairOf<S>::E to_storage_pair(f2 v, f2 si, ui
 #define LB_TMA_WIDE_WARPS 0  // consumer warps of the store-staged kernel (two per tile row); 0: 18, q = 64: 14
 #endif
 #ifndef LB_TMA_WIDE_SMEM
-// ring + output slots of the store-staged kernel (D2Q36-GH FP32 at 4096^2: 192 and 224 KB 774 us a level)
-#define LB_TMA_WIDE_SMEM (192 * 1024)
+// ring + output slots of the store-staged kernel, bytes; 0: FP32 224 KB (D2Q36-GH at 4096^2, 192 / 224 KB
+// and 12 velocities a stage: 788 / 751 us a level), 16-bit 192 KB (D2Q64-GH at 2048^2 525 / 563)
+#define LB_TMA_WIDE_SMEM 0
 #endif
 #ifndef LB_DIAG_PREFETCH
 // load sin/cos of the diagnostics before the collision: -1 per set and kernel, 0 never, 1 always.  Taken
@@ -528,7 +529,7 @@ struct Cfg {
 // tensor store (cp.async.bulk.tensor, shared -> global), so no lane issues per-velocity global stores.
 // A warp waits only for its own store of the tile before: one store of the whole tile by the producer
 // made every warp wait for the slowest one's tile and for that store.  D2Q36-GH FP32 at 4096^2: 820 -> 774 us
-// a level (5.89 -> 6.25 TB/s), 1024^2 69 -> 66.
+// a level, with larger stages 751 (5.89 -> 6.43 TB/s).
 template <class VS, class S, bool UPW = false, bool WIDE = false>
 struct TmaCfg {
     static constexpr bool LW = !VS::kOnLattice;
@@ -573,10 +574,13 @@ struct TmaCfg {
     // D2Q36-GH 4096^2 6 / 12 / 18 / 36 889 / 819 / 814 / 811; D2Q16-GH 4096^2 6 / 8 / 16 453 / 432 /
     // 411), FP32 D2Q16-GH 8 (4096^2 and 2502 x 1251, 6 / 8 / 16: 388 / 364 / 361 and 83.7 / 79.2 / 80.0,
     // three tiles of stages), D2Q36-GH 12 (4094 x 4096, 6 / 12 / 18: 838 / 786 / 793), D2Q64-GH 16 (2048^2,
-    // 8 / 12 / 16: 391 / 372 / 369), store-staged D2Q36-GH 6 (4096^2, 4 / 6 / 18: 820 / 774 / 804).
+    // 8 / 12 / 16: 391 / 372 / 369), store-staged D2Q36-GH 12, a third of a tile
+    // (FP32 4096^2, 4 / 6 / 10 / 12 / 14 / 18: 820 / 774 / 758 / 751 / 784 / 804, 1024^2 6 / 12: 66 / 65; N = 1
+    // alone is faster with 6, 738 / 768; FP16 1005 / 947 with 6 / 12), upwind D2Q36-GH 12 (2048^2 6 / 12: 224 /
+    // 215, 4096^2 891 / 828).
     static constexpr int K = LB_TMA_K > 0          ? LB_TMA_K
                              : !LW                 ? 18
-                             : WIDE || UPW         ? (VS::Q > 40 ? 12 : 6)
+                             : WIDE || UPW         ? (VS::Q > 16 ? 12 : 6)
                              : sizeof(S) == 2      ? VS::Q
                              : VS::Q > 40          ? 16
                                                    : (VS::Q > 16 ? 12 : 8);
@@ -587,7 +591,8 @@ struct TmaCfg {
     // output slot of a warp of the store-staged kernel: [plane][WCELLS cells]
     static constexpr int OUT_SLOT = (Layout<VS, S>::PLANES * WCELLS * EB + 127) / 128 * 128;
     static constexpr int OUT_BYTES = WIDE ? CW * OUT_SLOT : 0;
-    static constexpr int NS_FIT = ((WIDE ? LB_TMA_WIDE_SMEM - OUT_BYTES : LB_TMA_SMEM) - 512) / STAGE_BYTES;
+    static constexpr int WIDE_SMEM = LB_TMA_WIDE_SMEM > 0 ? LB_TMA_WIDE_SMEM : (sizeof(S) == 4 ? 224 : 192) * 1024;
+    static constexpr int NS_FIT = ((WIDE ? WIDE_SMEM - OUT_BYTES : LB_TMA_SMEM) - 512) / STAGE_BYTES;
     static constexpr int NS_TILES = LB_TMA_NS_TILES > 0 ? LB_TMA_NS_TILES
                                     : LW && !WIDE && !UPW && VS::Q == 16 ? (sizeof(S) == 2 ? 4 : 3) : 2;
     static constexpr int NS = NS_FIT < NS_TILES * NG ? NS_FIT : NS_TILES * NG;
@@ -2254,8 +2259,8 @@ cudaError_t launch_typed(const Launch& L) {
                     sh->st_box_h = TS::BH;
                     sh->st_box_d = TS::BOX_D;
                     // D2Q16-GH and the 16-bit sets are faster with plain stores (4096^2, us a level, plain /
-                    // store-staged: D2Q16-GH FP32 364 / 421, D2Q36-GH FP16 811 / 1005), D2Q36-GH FP32 with
-                    // staged ones (788 at 4094 x 4096 / 774)
+                    // store-staged: D2Q16-GH FP32 364 / 421, D2Q36-GH FP16 811 / 947), D2Q36-GH FP32 with
+                    // staged ones (788 at 4094 x 4096 / 751)
                     sh->st_auto = (sizeof(S) == 4 && VS::Q > 16) ? 1 : 0;
                 }
             }
