@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kBatchMaxWarps * 32) lb_batch_kernel(const __g
         const BatchQueue& Qu = B.queue[kind];
         BatchGroup G;
         G.kind = kind;
-        const int per_cta = kind <= kBatchCta ? nwarp : (kind == kBatchQuad ? 4 : 1);  // warps of a group in a CTA
+        const int per_cta = batch_group_warps(kind, nwarp);  // warps of a group in a CTA
         if (kind == kBatchQuad && nwarp % 4 != 0) continue;  // (the host leaves that queue empty)
         G.ctas = kind == kBatchCluster ? (int)nc : 1;
         G.warps = per_cta * G.ctas;
@@ -359,9 +359,9 @@ __global__ void __launch_bounds__(kBatchMaxWarps * 32) lb_batch_kernel(const __g
         G.wid = (warp - G.first) * G.ctas + (kind == kBatchCluster ? (int)rank : 0);
         G.threads = 32 * per_cta;
         G.tid = threadIdx.x - 32 * G.first;
-        // each group's slice of the shared memory, 16-byte aligned
-        G.smem_cap = (int)((long long)B.smem_cap * per_cta / nwarp) & ~15;
-        void* const smem = bsm + (size_t)(G.first / per_cta) * G.smem_cap;
+        const BatchSlice slice = batch_slice(kind, G.first, B.smem_cap, nwarp);
+        G.smem_cap = slice.bytes;
+        void* const smem = bsm + slice.offset;
         if (!Qu.order) continue;
         const int n = *Qu.n;
         if (n == 0) continue;

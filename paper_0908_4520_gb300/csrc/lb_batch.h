@@ -1,6 +1,7 @@
 // Host/device descriptors of the persistent multi-instance kernel.
 #pragma once
 
+#include "lb_batch_slices.h"
 #include "lb_device.h"
 
 namespace lbk {
@@ -30,9 +31,6 @@ struct BatchInst {
     // conservation identities (see Tab)
     float ow[kMaxNA], owlo[kMaxNA], hn1lo[kMaxNA], whn1lo[kMaxNA];
 };
-
-// The work queues, by the width of the group of warps that advances an instance.
-enum BatchKind : int { kBatchCluster = 0, kBatchCta = 1, kBatchQuad = 2, kBatchWarp = 3, kBatchQueues = 4 };
 
 struct BatchQueue {
     const int* order;     // slots in processing order (null: no such queue)
