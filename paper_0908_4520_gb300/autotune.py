@@ -11,10 +11,13 @@ holds the whole mix up to 1024 instances: a trial must fill every SM the way the
 real launch does, or it times one instance's latency instead of the launch's
 throughput.  Results are
 cached in a JSON file keyed by the storage type and a signature of the mix
-(quadrature, order and grid-size classes), so later runs reuse them.
+(quadrature, order and grid-size classes), of the candidates and of what ran
+them (the library's code, the device, the trial's size), so later runs reuse
+them, and a library with other kernels or candidates tunes anew.
 """
 from __future__ import annotations
 
+import functools
 import hashlib
 import json
 import os
@@ -29,10 +32,23 @@ CANDIDATES = [(0, -1, -1)] + [(t, s, w) for t in (64, 128, 256) for s in (0, 48 
 _CACHE = os.path.join(os.path.expanduser("~"), ".cache", "paper_0908_4520_gb300", "autotune.json")
 
 
-def _signature(instances, precision):
+@functools.lru_cache(maxsize=None)
+def _library_digest():
+    """Digest of the loaded library: the kernels that a result was measured with."""
+    with open(capi.LIB_PATH, "rb") as fh:
+        return hashlib.file_digest(fh, "sha256").hexdigest()
+
+
+def _device_name():
+    import torch
+
+    return torch.cuda.get_device_name() if torch.cuda.is_available() else ""
+
+
+def _signature(instances, precision, sample=1024, chunk=32):
     classes = sorted({(d["quadrature"], d["n_eq"], d["nx"] * d["ny"]) for d in instances})
-    h = hashlib.sha256(json.dumps(["threads/smem/warp_cells", precision, classes]).encode()).hexdigest()[:16]
-    return f"{precision}:{h}"
+    key = ["threads/smem/warp_cells", precision, classes, CANDIDATES, _library_digest(), _device_name(), sample, chunk]
+    return f"{precision}:{hashlib.sha256(json.dumps(key).encode()).hexdigest()[:16]}"
 
 
 def _sample(instances, k):
@@ -72,7 +88,7 @@ def _trial(sample, precision, threads, smem, warp_cells, chunk):
 
 def tune(instances, precision: str = "f32", sample: int = 1024, chunk: int = 32, use_cache: bool = True) -> dict:
     """Best (threads, smem_bytes, warp_cells) for this mix; cached by mix signature."""
-    sig = _signature(instances, precision)
+    sig = _signature(instances, precision, sample, chunk)
     cache = {}
     if use_cache and os.path.exists(_CACHE):
         try:
