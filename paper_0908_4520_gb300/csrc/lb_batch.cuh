@@ -224,7 +224,7 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
                         static_for<0, Q / 2>([&](auto mc) {
                             constexpr int m = decltype(mc)::value, a = 2 * m;
                             auto pair = [&](const E* p) {
-                                f2 v = lds_pair<S>(p);  // (plain loads: the arena or shared memory)
+                                f2 v = ld_pair<S>(p);  // (plain loads: the arena or shared memory)
                                 if constexpr (Is16<S>::value)
                                     v = vmul(v, f2{t.sc[a] * scale, t.sc[a + 1] * scale});
                                 return v;

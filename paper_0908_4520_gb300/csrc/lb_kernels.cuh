@@ -62,78 +62,6 @@ struct Is16<__nv_bfloat16> : std::true_type {};
 template <>
 struct Is16<__half> : std::true_type {};
 
-// (loads of the populations do not take the read-only path: a step launch may have started, and its
-// caches filled, before the launch that writes them has ended; see await_previous_step)
-template <class S, class R>
-__device__ __forceinline__ R ld1(const S* p, R scale) {
-    if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        return __bfloat162float(*p) * scale;
-    } else if constexpr (std::is_same<S, __half>::value) {
-        return __half2float(*p) * scale;
-    } else {
-        (void)scale;
-        return *p;
-    }
-}
-
-// shared-memory loads (plain, no read-only path)
-template <class S, class R>
-__device__ __forceinline__ R sld1(const S* p, R scale) {
-    if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        return __bfloat162float(*p) * scale;
-    } else if constexpr (std::is_same<S, __half>::value) {
-        return __half2float(*p) * scale;
-    } else {
-        (void)scale;
-        return *p;
-    }
-}
-
-template <class S, class R>
-__device__ __forceinline__ void sld2(const S* p, R scale, R& v0, R& v1) {
-    if constexpr (std::is_same<S, float>::value) {
-        const float2 t = *reinterpret_cast<const float2*>(p);
-        v0 = t.x;
-        v1 = t.y;
-    } else if constexpr (std::is_same<S, double>::value) {
-        const double2 t = *reinterpret_cast<const double2*>(p);
-        v0 = t.x;
-        v1 = t.y;
-    } else if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
-        v0 = t.x * scale;
-        v1 = t.y * scale;
-    } else {
-        const float2 t = __half22float2(*reinterpret_cast<const __half2*>(p));
-        v0 = t.x * scale;
-        v1 = t.y * scale;
-    }
-    (void)scale;
-}
-
-// aligned pair p[0], p[1]
-template <class S, class R>
-__device__ __forceinline__ void ld2(const S* p, R scale, R& v0, R& v1) {
-    if constexpr (std::is_same<S, float>::value) {
-        const float2 t = *reinterpret_cast<const float2*>(p);
-        v0 = t.x;
-        v1 = t.y;
-    } else if constexpr (std::is_same<S, double>::value) {
-        const double2 t = *reinterpret_cast<const double2*>(p);
-        v0 = t.x;
-        v1 = t.y;
-    } else if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
-        v0 = t.x * scale;
-        v1 = t.y * scale;
-    } else {
-        const float2 t = __half22float2(*reinterpret_cast<const __half2*>(p));
-        v0 = t.x * scale;
-        v1 = t.y * scale;
-    }
-    (void)scale;
-}
-
 template <class S, class R>
 __device__ __forceinline__ void st1(S* p, R v, R scinv) {
     if constexpr (std::is_same<S, __nv_bfloat16>::value) {
@@ -228,20 +156,6 @@ __device__ __forceinline__ uint32_t sr_bits(uint32_t r) {
     return std::is_same<S, __half>::value ? (r >> 19) : (r >> 16);
 }
 
-// storage value of a deviation (16-bit: stochastic rounding with the random bits of r)
-template <class S, class R>
-__device__ __forceinline__ S to_storage(R v, R scinv, uint32_t r) {
-    if constexpr (std::is_same<S, __half>::value) {
-        return __float2half_rz(__uint_as_float(__float_as_uint(v * scinv) + sr_bits<S>(r)));
-    } else if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        return __float2bfloat16_rz(__uint_as_float(__float_as_uint(v * scinv) + sr_bits<S>(r)));
-    } else {
-        (void)scinv;
-        (void)r;
-        return v;
-    }
-}
-
 // Two scaled values (already multiplied by the storage scale) rounded stochastically
 // into one 16-bit pair word, the first in the low half (one conversion instruction).
 template <class S>
@@ -255,29 +169,6 @@ __device__ __forceinline__ uint32_t to_storage16x2(float h0, float h1, uint32_t 
         asm("cvt.rz.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
     }
     return d;
-}
-
-template <class S>
-__device__ __forceinline__ void store_raw(S* p, S a) {
-    *p = a;
-}
-template <class S>
-__device__ __forceinline__ void store_raw2(S* p, S a, S b) {
-    if constexpr (std::is_same<S, float>::value) {
-        __stcs(reinterpret_cast<float2*>(p), make_float2(a, b));
-    } else if constexpr (std::is_same<S, double>::value) {
-        __stcs(reinterpret_cast<double2*>(p), make_double2(a, b));
-    } else if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        __nv_bfloat162 t;
-        t.x = a;
-        t.y = b;
-        __stcs(reinterpret_cast<__nv_bfloat162*>(p), t);
-    } else {
-        __half2 t;
-        t.x = a;
-        t.y = b;
-        __stcs(reinterpret_cast<__half2*>(p), t);
-    }
 }
 
 // compile-time loop: f(integral_constant<int, a>) for a in [A_, Q)
@@ -394,7 +285,20 @@ struct Pack<float, 2> {
     using T = f2;
 };
 
-// A pair of velocities of one cell, unscaled (global memory; shared memory).
+// Loads of the populations, from global or shared memory.  None takes the read-only path: a step launch
+// may have started, and its caches filled, before the launch that writes them has ended (see
+// await_previous_step).
+// The cells of a lane: one value, or an aligned pair.
+template <class T, class R>
+__device__ __forceinline__ T ld_cells(const R* p) {
+    if constexpr (std::is_same<T, f2>::value) {
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        return f2{t.x, t.y};
+    } else {
+        return *p;
+    }
+}
+// A pair of velocities of one cell, unscaled.
 template <class S>
 __device__ __forceinline__ f2 unpack_pair(uint32_t u) {
     float2 t;
@@ -407,15 +311,6 @@ __device__ __forceinline__ f2 unpack_pair(uint32_t u) {
 }
 template <class S>
 __device__ __forceinline__ f2 ld_pair(const typename PairOf<S>::E* p) {
-    if constexpr (std::is_same<S, float>::value) {
-        const float2 t = *p;
-        return f2{t.x, t.y};
-    } else {
-        return unpack_pair<S>(*p);
-    }
-}
-template <class S>
-__device__ __forceinline__ f2 lds_pair(const typename PairOf<S>::E* p) {
     if constexpr (std::is_same<S, float>::value) {
         const float2 t = *p;
         return f2{t.x, t.y};
@@ -964,12 +859,6 @@ __device__ __forceinline__ R force_at_level(const Args<R>& A, long long lvl) {
     return A.force_amp != 0.0 ? (R)(A.force_amp * cos(A.force_freq * (double)lvl * A.dt)) : R(0);
 }
 
-// The same collision with one cell per lane and the velocities taken in pairs (a, a + 1)
-// of equal x node (a = ix NA + iy, iy even), each pair one packed f32x2 value: the
-// per-velocity work (moment sums, diagnostics, equilibrium, relaxation) runs at half the
-// instruction count.  Product-weight Gauss-Hermite sets (NA even), FP32 arithmetic.
-// Moments as in collide_cell, with the y-node sums kept as pairs and the x-node sums
-// reduced when the x node changes; H = sum_ix (1/W_ix) sum_iy d^2 / W_iy.
 // Tensor-product Lax-Wendroff of a velocity pair (a, a + 1) of one lane's cell: the y pass over
 // the lane's column (values of the rows y - 1, y, y + 1), then the x pass, whose neighbours'
 // columns come by shuffles.  The pair has one x node and two y nodes, so both passes run as
@@ -994,6 +883,12 @@ __device__ __forceinline__ f2 shfl_down2(f2 v) {
     return f2{__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1)};
 }
 
+// The collision of collide_cell with one cell per lane and the velocities taken in pairs (a, a + 1)
+// of equal x node (a = ix NA + iy, iy even), each pair one packed f32x2 value: the
+// per-velocity work (moment sums, diagnostics, equilibrium, relaxation) runs at half the
+// instruction count.  Product-weight Gauss-Hermite sets (NA even), FP32 arithmetic.
+// Moments as in collide_cell, with the y-node sums kept as pairs and the x-node sums
+// reduced when the x node changes; H = sum_ix (1/W_ix) sum_iy d^2 / W_iy.
 // ow, owlo, hn1lo, whn1lo: the relaxation tables of omega (Tab), the handle's own or, in a
 // batch, the instance's.
 template <class VS, int N, bool COLLIDE, class F>
@@ -1210,7 +1105,7 @@ __device__ __forceinline__ void collide_store(const Args<R>& A, T (&ft)[VS::Q], 
                 static_for<0, Q>([&](auto ac) {
                     constexpr int a = decltype(ac)::value;
                     if constexpr (V == 2) {
-                        store_raw2<S>(p, lane_get<0>(ft[a]), lane_get<1>(ft[a]));
+                        __stcs(reinterpret_cast<float2*>(p), make_float2(ft[a].x, ft[a].y));
                     } else {
                         *p = ft[a];
                     }
@@ -1470,29 +1365,18 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
             static_for<0, Q>([&](auto ac) {
                 constexpr int a = decltype(ac)::value;
                 constexpr int VW = Layout<VS, S>::VW;
-                const R sc = load_scale<S, R>(A.tab, a);
                 const S* pl = src + pop_index<VS, S>(a, A.plane, A.origin);
                 if (A.raw) {
                     const S* p = pl + VW * ((long long)y * A.pitch + g.xl);
-                    if constexpr (V == 2) {
-                        R v0, v1;
-                        ld2<S, R>(p, sc, v0, v1);
-                        ft[a] = pack_lanes<T, R>(v0, v1);
-                    } else {
-                        ft[a] = ld1<S, R>(p, sc);
-                    }
+                    ft[a] = ld_cells<T>(p);
                 } else if constexpr (VS::kOnLattice) {
                     // exact shift: f~_a(x, y) = f*_a(x - ex, y - ey)
                     constexpr int ex = VS::ex(a), ey = VS::ey(a);
                     const S* p = pl + (long long)(y - ey) * A.pitch + g.xl - ex;
-                    if constexpr (V == 2 && (ex % 2 == 0)) {
-                        R v0, v1;
-                        ld2<S, R>(p, sc, v0, v1);
-                        ft[a] = pack_lanes<T, R>(v0, v1);
-                    } else if constexpr (V == 2) {
-                        ft[a] = pack_lanes<T, R>(ld1<S, R>(p, sc), ld1<S, R>(p + 1, sc));
+                    if constexpr (V == 2 && ex % 2 != 0) {
+                        ft[a] = pack_lanes<T, R>(p[0], p[1]);
                     } else {
-                        ft[a] = ld1<S, R>(p, sc);
+                        ft[a] = ld_cells<T>(p);
                     }
                 } else if constexpr (UPW) {
                     // tensor-product second-order upwind (Beam-Warming), one cell per lane: y pass
@@ -1507,16 +1391,15 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
                     const S* r0 = pl + VW * (long long)y * A.pitch;
                     const S* rn = r0 - VW * (long long)sy * A.pitch;
                     const S* rf = r0 - VW * 2LL * sy * A.pitch;
-                    const R one = R(1);
                     // lanes past the grid read the images of columns 0 and 1 (nx, nx + 1)
                     const int xu = VW * min(g.x, A.nx + 1);
-                    const R gv = fma(yf, ld1<S, R>(rf + xu, one), fma(yn, ld1<S, R>(rn + xu, one),
-                                                                     ys * ld1<S, R>(r0 + xu, one)));
+                    const R gv = fma(yf, rf[xu], fma(yn, rn[xu],
+                                                                     ys * r0[xu]));
                     // extra column: x0 - 2 + (lane & 1) (lanes 30, 31) for sx > 0,
                     // x0 + 32 + (lane & 1) (lanes 0, 1) for sx < 0, clamped into the rim
                     const int xe = VW * (sx > 0 ? x0 - 2 + (lane & 1) : min(x0 + 32 + (lane & 1), A.nx + 1));
-                    const R ge = fma(yf, ld1<S, R>(rf + xe, one), fma(yn, ld1<S, R>(rn + xe, one),
-                                                                     ys * ld1<S, R>(r0 + xe, one)));
+                    const R ge = fma(yf, rf[xe], fma(yn, rn[xe],
+                                                                     ys * r0[xe]));
                     R g1, g2;
                     if constexpr (sx > 0) {
                         g1 = __shfl_up_sync(0xffffffffu, gv, 1);
@@ -1544,12 +1427,11 @@ __global__ void __launch_bounds__(Cfg<VS, S>::THREADS, Cfg<VS, S>::MINB)
                     const S* r0 = pl + (long long)y * A.pitch;
                     const S* rm = r0 - A.pitch;
                     const S* rp = r0 + A.pitch;
-                    const R one = R(1);
                     const int xe = (lane == 31) ? min(x0 + TW, A.nx) : x0 - 1;
-                    const R ge = fma(ly0, ld1<S, R>(rm + xe, one), fma(ly1, ld1<S, R>(r0 + xe, one), ly2 * ld1<S, R>(rp + xe, one)));
-                    const R f0 = ld1<S, R>(r0 + g.xl, one);
-                    const R fm = ld1<S, R>(rm + g.xl, one);
-                    const R fp = ld1<S, R>(rp + g.xl, one);
+                    const R ge = fma(ly0, rm[xe], fma(ly1, r0[xe], ly2 * rp[xe]));
+                    const R f0 = r0[g.xl];
+                    const R fm = rm[g.xl];
+                    const R fp = rp[g.xl];
                     const R gv = fma(ly0, fm, fma(ly1, f0, ly2 * fp));
                     R gl = __shfl_up_sync(0xffffffffu, gv, 1);
                     R gr = __shfl_down_sync(0xffffffffu, gv, 1);
@@ -2035,14 +1917,14 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                                     const E* r0 = box + (trow + 2) * BW + c;
                                     auto upstream = [&](int k) {
                                         if constexpr (sa == sb) {
-                                            return lds_pair<S>(r0 - k * sa * BW);
+                                            return ld_pair<S>(r0 - k * sa * BW);
                                         } else {
                                             return f2{reinterpret_cast<const float*>(r0 - k * sa * BW)[0],
                                                       reinterpret_cast<const float*>(r0 - k * sb * BW)[1]};
                                         }
                                     };
                                     auto uw = [&](int k) { return f2{A.tab.uw[iy][k], A.tab.uw[iy + 1][k]}; };
-                                    const f2 gv = vfma(uw(0), upstream(2), vfma(uw(1), upstream(1), vmul(uw(2), lds_pair<S>(r0))));
+                                    const f2 gv = vfma(uw(0), upstream(2), vfma(uw(1), upstream(1), vmul(uw(2), ld_pair<S>(r0))));
                                     const f2 g1 = sx > 0 ? shfl_up2(gv) : shfl_down2(gv);
                                     f2 g2;
                                     if constexpr (sx > 0) {
@@ -2055,8 +1937,8 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                                 } else {
                                     auto column = [&](int c) {
                                         const E* rm = box + trow * BW + c;  // row y - 1
-                                        return lw_y_pair<VS, a>(A.tab, lds_pair<S>(rm), lds_pair<S>(rm + BW),
-                                                                lds_pair<S>(rm + 2 * BW));
+                                        return lw_y_pair<VS, a>(A.tab, ld_pair<S>(rm), ld_pair<S>(rm + BW),
+                                                                ld_pair<S>(rm + 2 * BW));
                                     };
                                     const f2 gv = column(c_lw), gl = shfl_up2(gv), gr = shfl_down2(gv);
                                     v = lw_x_pair<VS, a>(A.tab, gl, gv, gr);
@@ -2073,17 +1955,12 @@ __global__ void __maxnreg__((TmaCfg<VS, S, UPW, WIDE>::MAXREG))
                             constexpr int a = grp * K + j;
                             if constexpr (a < Q) {
                                 constexpr int ex = VS::ex(a);
-                                const R sc = load_scale<S, R>(A.tab, a);
                                 const int r = (x0 - ex + kGhostX) & (AL - 1);
                                 const S* p = reinterpret_cast<const S*>(st + j * SLOT) + trow * BW + r + lane * V;
-                                if constexpr (V == 2 && (ex % 2 == 0)) {
-                                    R v0, v1;
-                                    sld2<S, R>(p, sc, v0, v1);
-                                    ft[a] = pack_lanes<T, R>(v0, v1);
-                                } else if constexpr (V == 2) {
-                                    ft[a] = pack_lanes<T, R>(sld1<S, R>(p, sc), sld1<S, R>(p + 1, sc));
+                                if constexpr (V == 2 && ex % 2 != 0) {
+                                    ft[a] = pack_lanes<T, R>(p[0], p[1]);
                                 } else {
-                                    ft[a] = sld1<S, R>(p, sc);
+                                    ft[a] = ld_cells<T>(p);
                                 }
                             }
                         });
