@@ -167,6 +167,8 @@ typedef struct {
     double c_lattice;   /* xi = c e for on-lattice sets, else 0 */
     long long time_level;   /* n: the state is f~(n dt) */
     int tma_staged;         /* 1: steps run the TMA-staged kernel, 2: its store-staged variant */
+    int node_split;         /* 1: steps run the node-split FP64 kernel (small grids); lies in what was
+                               padding, so the struct's layout is unchanged */
     long long records;      /* diagnostics records produced so far (n + 1 after init) */
     size_t bytes_per_cell_update; /* algorithmic HBM bytes: 2 q sizeof(storage) */
     size_t device_bytes;    /* device memory held by the handle */

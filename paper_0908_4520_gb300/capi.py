@@ -62,7 +62,7 @@ class lb_info_t(ctypes.Structure):
         ("q", ctypes.c_int), ("degree", ctypes.c_int), ("on_lattice", ctypes.c_int), ("halo", ctypes.c_int),
         ("dx", ctypes.c_double), ("dt", ctypes.c_double), ("tau", ctypes.c_double), ("omega", ctypes.c_double),
         ("c_lattice", ctypes.c_double), ("time_level", ctypes.c_longlong), ("tma_staged", ctypes.c_int),
-        ("records", ctypes.c_longlong),
+        ("node_split", ctypes.c_int), ("records", ctypes.c_longlong),
         ("bytes_per_cell_update", ctypes.c_size_t), ("device_bytes", ctypes.c_size_t),
         ("storage_scale", ctypes.c_double),
     ]

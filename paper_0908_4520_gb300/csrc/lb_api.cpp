@@ -1032,6 +1032,7 @@ lb_status lb_get_info(const lb_handle* h, lb_info_t* o) {
     o->c_lattice = h->vs.c;
     o->time_level = h->level;
     o->tma_staged = h->use_st ? 2 : h->use_tma ? 1 : 0;
+    o->node_split = h->use_split ? 1 : 0;
     o->records = h->initialized ? h->level + 1 : 0;
     o->bytes_per_cell_update = 2 * (size_t)h->vs.q * storage_bytes(h->p.precision);
     o->device_bytes = h->device_bytes;
