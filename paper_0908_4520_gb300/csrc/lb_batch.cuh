@@ -20,8 +20,9 @@
 // those kernels.
 //
 // The sums of a level (A, S, H) are taken over 64 slots: strip s belongs to slot s % 64, a slot to
-// one warp, which sums its strips in order; after the level's barrier every warp sums the slots in
-// the same order and so knows for itself whether the instance has stopped.  Neither a cell's
+// one warp, which sums its strips in order in FP32; after the level's barrier every warp adds the
+// slots in the same order, with what each addition rounds off (Sum2), and so knows for itself
+// whether the instance has stopped; the history is rounded to FP32 once.  Neither a cell's
 // operations nor the sums' order depend on the group or the memory path, so an instance's
 // populations and history are bitwise the same whichever path runs it and whatever else shares the
 // launch.  Lax-Wendroff streaming only: the batch serves the Gauss-Hermite product sets.
@@ -44,7 +45,7 @@ constexpr int kBatchSlots = 64;     // partial sums of a level
 
 // the kernel's static shared memory; what belongs to a group lies at the index of its first warp
 struct BatchShared {
-    float red[kBatchMaxWarps / 4][2][3][kBatchSlots];  // A, S, H by slot, two levels (groups of four warps and more)
+    float red[kBatchMaxWarps][3][kBatchSlots];     // A, S, H by slot: of two levels in turn (one warp: of one)
     float relax[kBatchMaxWarps][4][kMaxNA];        // relaxation tables of the group's instance
     int next[kBatchMaxWarps];                      // queue position of the group's instance
 };
@@ -111,6 +112,29 @@ __device__ __forceinline__ float warp_sum3(float a, float b, float c, int lane) 
     return x;
 }
 
+// A sum of FP32 values as its FP32 rounding and what that left out: the slots' sums are exact to 2^-46
+// of their terms' size.  FP64 additions, of which an SM does two a clock, cost a level of a small
+// instance up to half as much again (152 of D2Q16-GH 256 x 1, us a level: plain FP32 sums, whose
+// rounding the history then has, 3.27, FP64 5.06, these 3.56; 512 uneven instances the same with all
+// three, 66 to 67 ms).
+struct Sum2 {
+    float hi, lo;
+};
+__device__ __forceinline__ Sum2 add2(Sum2 a, Sum2 b) {
+    // Knuth's two-sum of the leading parts (exact); the parts left out add up
+    const float s = __fadd_rn(a.hi, b.hi), t = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
+    return {s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
+}
+__device__ __forceinline__ Sum2 shfl_xor2(Sum2 v, int o) {
+    return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+// hi the FP32 rounding of the whole sum (a sum that is not finite stays as it is)
+__device__ __forceinline__ Sum2 normal2(Sum2 v) {
+    const float s = __fadd_rn(v.hi, v.lo);
+    return isfinite(v.hi) ? Sum2{s, __fsub_rn(v.lo, __fsub_rn(s, v.hi))} : Sum2{v.hi, 0.f};
+}
+
 // Advance instance `id` by up to B.chunk levels with the group's warps (smem: the group's share of
 // the CTA's shared memory).
 template <class VS, int SET, int N, class S>
@@ -164,9 +188,14 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
     const int isothermal = in.isothermal, max_level = in.max_level;
     const float stop_ratio2 = in.stop_ratio2;
     // stop rule sqrt(H / H0) <= stop_ratio (none for stop_ratio = 0, also where H is 0): the largest
-    // FP32 value of H that meets it
-    auto threshold = [&](float h) { return __double2float_rd((double)stop_ratio2 * (double)h); };
-    float hstop = threshold(h0);
+    // value of H that meets it, as a sum
+    auto threshold = [&](float h) {
+        const double t = (double)stop_ratio2 * (double)h;
+        const float hi = __double2float_rn(t);
+        return Sum2{hi, __double2float_rd(t - (double)hi)};
+    };
+    Sum2 hstop = threshold(h0);
+    const double norm = 2.0 / (double)ncell;
 
     // 16-bit storage: deviation = stored * sc[a] * scale; sc (tables built with S = 1) and
     // scale are powers of two, so the load and store scales are exact inverses
@@ -176,8 +205,7 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
     for (; level <= stop && !done; ++level) {
         const E* src = buf[cur];
         E* dst = buf[level == 0 ? 0 : 1 - cur];
-        float(*red)[kBatchSlots] = sh.red[G.first / 4][level & 1];
-        float tot[3] = {0.f, 0.f, 0.f};  // lane l: the sums of slots l and l + 32
+        float(*red)[kBatchSlots] = sh.red[G.kind == kBatchWarp ? G.first : G.first + (level & 1)];
         for (int slot = G.wid; slot < nslot; slot += G.warps) {
             float pa = 0.f, ps = 0.f, ph = 0.f;
             // strips of up to 30 cells of one row: lanes 1..w own cells x0 .. x0 + w - 1, lanes 0
@@ -273,47 +301,54 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
                 }
             }
             const float v = warp_sum3(pa, ps, ph, lane);
-            if (G.kind == kBatchWarp) {  // the warp has every slot itself
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const float r = __shfl_sync(0xffffffffu, v, 8 * k);
-                    if (lane == (slot & 31)) tot[k] += r;
-                }
-            } else if (lane == 0 || lane == 8 || lane == 16) {
-                red[lane >> 3][slot] = v;
-            }
+            if (lane == 0 || lane == 8 || lane == 16) red[lane >> 3][slot] = v;
         }
         G.sync();
-        // every warp sums the slots
-        if (G.kind != kBatchWarp) {
+        // every warp sums the slots: eight lanes each A, S and H, lane j of them slots j, j + 8, ..
+        const float* const mine = red[min(lane >> 3, 2)] + (lane & 7);
+        Sum2 tot = {0.f, 0.f};
+        auto take = [&](auto i0, auto i1) {
+            constexpr int I0 = decltype(i0)::value, I1 = decltype(i1)::value;
+            float part[I1 - I0];
+            if (G.ctas == 1) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k)
+                for (int i = I0; i < I1; ++i) part[i - I0] = mine[8 * i];
+            } else {  // (slot s lies in CTA s % 2)
+                const uint32_t at = cluster_addr(mine, lane % G.ctas);
 #pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    const int slot = lane + 32 * s;
-                    if (slot < nslot)
-                        tot[k] += G.ctas == 1 ? red[k][slot] : cluster_ld(cluster_addr(&red[k][slot], slot % G.ctas));
-                }
+                for (int i = I0; i < I1; ++i) part[i - I0] = cluster_ld(at + 32 * i);
+            }
+#pragma unroll
+            for (int i = I0; i < I1; ++i) {
+                const float v = 8 * i + (lane & 7) < nslot ? part[i - I0] : 0.f;
+                tot = i == 0 ? Sum2{v, 0.f} : add2(tot, Sum2{v, 0.f});
+            }
+        };
+        using I = std::integral_constant<int, 1>;
+        take(std::integral_constant<int, 0>{}, I{});
+        if (nslot > 8) take(I{}, std::integral_constant<int, 2>{});
+        if (nslot > 16) take(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
+        if (nslot > 32) take(std::integral_constant<int, 4>{}, std::integral_constant<int, kBatchSlots / 8>{});
+        if (nslot > 1) {
+            if (nslot > 4) tot = add2(tot, shfl_xor2(tot, 4));
+            if (nslot > 2) tot = add2(tot, shfl_xor2(tot, 2));
+            tot = normal2(add2(tot, shfl_xor2(tot, 1)));
         }
-        const float v = warp_sum3(tot[0], tot[1], tot[2], lane);
-        const float H = __shfl_sync(0xffffffffu, v, 16);
+        if (G.kind == kBatchWarp) __syncwarp();  // (before the next level's slots)
+        const Sum2 H = {__shfl_sync(0xffffffffu, tot.hi, 16), __shfl_sync(0xffffffffu, tot.lo, 16)};
         if (level == 0) {
-            h0 = H;
+            h0 = H.hi;
             hstop = threshold(h0);
         }
-        if (!isfinite(H)) {
+        if (!isfinite(H.hi)) {
             status = 1;
             done = true;
         }
-        if (level > 0 && stop_ratio2 > 0.f && H <= hstop) done = true;
+        if (level > 0 && stop_ratio2 > 0.f && (H.hi < hstop.hi || (H.hi == hstop.hi && H.lo <= hstop.lo))) done = true;
         if (level == max_level) done = true;
-        if (G.wid == 0) {
-            const float Sx = __shfl_sync(0xffffffffu, v, 8);
-            if (lane == 0) {
-                const double norm = 2.0 / (double)ncell;
-                hist[level] = make_float2((float)((double)v * norm), (float)((double)Sx * norm));
-            }
-        }
+        // the history, by the group's last warp (none has fewer strips)
+        if (G.wid == G.warps - 1 && (lane == 0 || lane == 8))
+            reinterpret_cast<float*>(hist + level)[lane >> 3] = (float)fma((double)tot.lo, norm, (double)tot.hi * norm);
         cur = (level == 0) ? 0 : 1 - cur;
     }
     if (onchip && level > first_level)
