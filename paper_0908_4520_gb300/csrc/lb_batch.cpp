@@ -108,6 +108,7 @@ struct lb_batch {
     std::vector<std::vector<std::pair<size_t, size_t>>> ranges_of;
     std::vector<double> tau;
     int threads = lbk::kBatchThreads, smem = 96 * 1024, grid = 0;
+    int l2_bytes = 0;           // of the device's second-level cache
     cudaGraphExec_t graph = nullptr;
     int graph_chunk = -1;
     bool in_flight = false;
@@ -158,6 +159,52 @@ cudaError_t batch_setup(lb_precision prec, int threads, int* smem, int* grid) {
         case LB_BF16: return lbk::batch_setup_bf16(threads, lbk::kBatchClusterCtas, smem, grid);
         default: return cudaErrorInvalidValue;
     }
+}
+
+// Whether a CTA of nw warps has groups of four beside the whole CTA.
+bool quads(int nw) { return nw > 4 && nw % 4 == 0; }
+
+// The group width for a launch of instances that are alike (their strips x velocities within a quarter
+// of one another), -1 where they are not: n instances on g groups take ceil(n / g) waves of
+// ceil(strips / warps) rounds each, and about three quarters of a round (a cluster: one) for the level's
+// barrier and sums.  The mean load says nothing there: 152 equal instances on 152 SMs have it exactly,
+// and the rule of half the mean put them on clusters, two waves where whole CTAs take one.  A width whose
+// instances at work together take more than three quarters of the L2 is used only if every width's do.
+// us a level, half the mean / this rule (FP32): 152 of D2Q16-GH 256 x 4 13.9 / 8.1, of D2Q64-GH 256 x 4
+// 39.3 / 28.5; 1000 of D2Q16-GH 256 x 1 19.1 / 12.7; 608 of D2Q36-GH 256 x 1 15.9 / 12.4.
+int alike_width(const lb_batch* b, const std::vector<long long>& strips) {
+    const int nw = b->threads / 32;
+    long long n = 0, most = 0, lo = 0, hi = 0;
+    double bytes = 0.0;
+    for (int s = 0; s < b->p.max_slots; ++s) {
+        if (!b->live[s] || b->inst[s].done) continue;
+        const lbk::BatchInst& in = b->inst[s];
+        const long long c = strips[s] * b->sets[in.set].q;
+        lo = n ? std::min(lo, c) : c;
+        hi = std::max(hi, c);
+        most = std::max(most, strips[s]);
+        bytes = std::max(bytes, 2.0 * b->sets[in.set].q * in.nx * in.ny * elem_bytes(b->p.precision));
+        ++n;
+    }
+    if (n == 0 || 4 * hi > 5 * lo) return -1;
+    const long long warps[lbk::kBatchQueues] = {(long long)nw * lbk::kBatchClusterCtas, nw, 4, 1};
+    const long long groups[lbk::kBatchQueues] = {b->grid / lbk::kBatchClusterCtas, b->grid,
+                                                 quads(nw) ? (long long)b->grid * (nw / 4) : 0,
+                                                 (long long)b->grid * nw};
+    int best = -1;
+    for (int fits = 1; fits >= 0 && best < 0; --fits) {
+        double t_best = 0.0;
+        for (int k = lbk::kBatchWarp; k >= lbk::kBatchCluster; --k) {
+            if (groups[k] == 0 || (fits && (double)std::min(n, groups[k]) * bytes > 0.75 * b->l2_bytes)) continue;
+            const double rounds = (double)((most + warps[k] - 1) / warps[k]) + (k == lbk::kBatchCluster ? 1.0 : 0.75);
+            const double t = (double)((n + groups[k] - 1) / groups[k]) * rounds;
+            if (best < 0 || t < t_best) {
+                best = k;
+                t_best = t;
+            }
+        }
+    }
+    return best;
 }
 
 }  // namespace
@@ -241,6 +288,10 @@ lb_status lb_batch_create(const lb_batch_params* pin, lb_batch** out) {
     if ((e = batch_setup(P.precision, b->threads, &b->smem, &b->grid)) != cudaSuccess || b->grid < 1)
         return bail(LB_ERR_ARG, std::string("kernel configuration does not fit: ") +
                                     (e != cudaSuccess ? cudaGetErrorString(e) : "zero occupancy"));
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&b->l2_bytes, cudaDevAttrL2CacheSize, dev)) != cudaSuccess)
+        return bail(LB_ERR_CUDA, std::string("device query: ") + cudaGetErrorString(e));
     if (cudaMalloc(&b->arena, P.budget_bytes) != cudaSuccess) return bail(LB_ERR_NOMEM, "arena allocation");
     if (cudaMalloc(&b->inst_d, sizeof(lbk::BatchInst) * P.max_slots) != cudaSuccess ||
         cudaMalloc(&b->order_d, sizeof(int) * lbk::kBatchQueues * (size_t)P.max_slots) != cudaSuccess ||
@@ -430,9 +481,11 @@ lb_status lb_batch_run(lb_batch* b, int chunk) {
         cost[s] = levels * (double)strips[s] * b->sets[in.set].q;
         total += cost[s];
     }
+    const int alike = b->warp_cells < 0 ? alike_width(b, strips) : -1;
     // An instance takes cost x (warps of a CTA) / (warps of its group) of an SM's time when the SM is
-    // full.  It goes to the narrowest group that takes at most half of the launch's mean time an SM,
-    // or that has a warp for every strip.  With warp_cells given: at most that many cells to a
+    // full.  Where the instances differ, each goes to the narrowest group that takes at most half of the
+    // launch's mean time an SM, or that has a warp for every strip; where they are alike, all go to the
+    // width whose waves end first (alike_width).  With warp_cells given: at most that many cells to a
     // warp, else to a CTA.  (Results do not depend on the choice.)
     const double mean = total / b->grid;
     const int width[lbk::kBatchQueues] = {nw * lbk::kBatchClusterCtas, nw, 4, 1};
@@ -441,9 +494,11 @@ lb_status lb_batch_run(lb_batch* b, int chunk) {
         int k = lbk::kBatchWarp;
         if (b->warp_cells >= 0) {
             if ((long long)b->inst[s].nx * b->inst[s].ny > b->warp_cells) k = lbk::kBatchCta;
+        } else if (alike >= 0) {
+            k = alike;
         } else {
             while (k > lbk::kBatchCluster && strips[s] > width[k] && cost[s] * nw / width[k] > 0.5 * mean) --k;
-            if (k == lbk::kBatchQuad && (nw <= 4 || nw % 4)) k = lbk::kBatchCta;
+            if (k == lbk::kBatchQuad && !quads(nw)) k = lbk::kBatchCta;
         }
         order[k].push_back(s);
     }
