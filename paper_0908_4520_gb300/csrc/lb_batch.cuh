@@ -20,9 +20,9 @@
 // those kernels.
 //
 // The sums of a level (A, S, H) are taken over 64 slots: strip s belongs to slot s % 64, a slot to
-// one warp, which sums its strips in order in FP32; after the level's barrier every warp adds the
-// slots in the same order, with what each addition rounds off (Sum2), and so knows for itself
-// whether the instance has stopped; the history is rounded to FP32 once.  Neither a cell's
+// one warp, which sums its strips in order in FP32; after the level's barrier every warp finds out
+// for itself whether the instance has stopped, and the last one adds the slots in a fixed order, with
+// what each addition rounds off (Sum2): the history is rounded to FP32 once.  Neither a cell's
 // operations nor the sums' order depend on the group or the memory path, so an instance's
 // populations and history are bitwise the same whichever path runs it and whatever else shares the
 // launch.  Lax-Wendroff streaming only: the batch serves the Gauss-Hermite product sets.
@@ -114,9 +114,9 @@ __device__ __forceinline__ float warp_sum3(float a, float b, float c, int lane) 
 
 // A sum of FP32 values as its FP32 rounding and what that left out: the slots' sums are exact to 2^-46
 // of their terms' size.  FP64 additions, of which an SM does two a clock, cost a level of a small
-// instance up to half as much again (152 of D2Q16-GH 256 x 1, us a level: plain FP32 sums, whose
-// rounding the history then has, 3.27, FP64 5.06, these 3.56; 512 uneven instances the same with all
-// three, 66 to 67 ms).
+// instance up to half as much again.  152 of D2Q16-GH 256 x 1, us a level: plain FP32 sums, whose
+// roundings the history then has, 3.29, FP64 5.06, these in every warp 3.56, in the last warp alone, the
+// others deciding by a plain sum, 2.75; 512 uneven instances 66 to 67 ms with all of them but the last, 65.
 struct Sum2 {
     float hi, lo;
 };
@@ -128,6 +128,21 @@ __device__ __forceinline__ Sum2 add2(Sum2 a, Sum2 b) {
 }
 __device__ __forceinline__ Sum2 shfl_xor2(Sum2 v, int o) {
     return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+// the same of one more value
+__device__ __forceinline__ Sum2 add1(Sum2 a, float b) {
+    const float s = __fadd_rn(a.hi, b), t = __fsub_rn(s, a.hi);
+    return {s, __fadd_rn(__fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b, t)), a.lo)};
+}
+// a b, rounded to FP32 once (a product that is not finite stays as it is)
+__device__ __forceinline__ float mul2(Sum2 a, Sum2 b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    const float r = fmaf(a.hi, b.hi, -p) + fmaf(a.hi, b.lo, a.lo * b.hi);
+    return isfinite(p) ? __fadd_rn(p, r) : p;
+}
+__device__ __forceinline__ Sum2 split2(double v) {
+    const float hi = __double2float_rn(v);
+    return {hi, __double2float_rd(v - (double)hi)};
 }
 // hi the FP32 rounding of the whole sum (a sum that is not finite stays as it is)
 __device__ __forceinline__ Sum2 normal2(Sum2 v) {
@@ -165,6 +180,7 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
     const int spr = ring ? 1 : (nx + kStrip - 1) / kStrip;  // strips per row
     const int nstrip = spr * ny;
     const int nslot = min(nstrip, kBatchSlots);
+    const bool solo = nstrip == 1 && G.warps == 1;  // one strip, one warp: no slots to add
 
     const int first_level = in.level;
     int level = first_level;
@@ -189,13 +205,9 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
     const float stop_ratio2 = in.stop_ratio2;
     // stop rule sqrt(H / H0) <= stop_ratio (none for stop_ratio = 0, also where H is 0): the largest
     // value of H that meets it, as a sum
-    auto threshold = [&](float h) {
-        const double t = (double)stop_ratio2 * (double)h;
-        const float hi = __double2float_rn(t);
-        return Sum2{hi, __double2float_rd(t - (double)hi)};
-    };
+    auto threshold = [&](float h) { return split2((double)stop_ratio2 * (double)h); };
     Sum2 hstop = threshold(h0);
-    const double norm = 2.0 / (double)ncell;
+    const Sum2 norm = split2(2.0 / (double)ncell);
 
     // 16-bit storage: deviation = stored * sc[a] * scale; sc (tables built with S = 1) and
     // scale are powers of two, so the load and store scales are exact inverses
@@ -206,6 +218,7 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
         const E* src = buf[cur];
         E* dst = buf[level == 0 ? 0 : 1 - cur];
         float(*red)[kBatchSlots] = sh.red[G.kind == kBatchWarp ? G.first : G.first + (level & 1)];
+        float one = 0.f;  // A, S and H of the warp's last slot in lanes 0, 8 and 16
         for (int slot = G.wid; slot < nslot; slot += G.warps) {
             float pa = 0.f, ps = 0.f, ph = 0.f;
             // strips of up to 30 cells of one row: lanes 1..w own cells x0 .. x0 + w - 1, lanes 0
@@ -300,55 +313,76 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
                     ph += co.h;
                 }
             }
-            const float v = warp_sum3(pa, ps, ph, lane);
-            if (lane == 0 || lane == 8 || lane == 16) red[lane >> 3][slot] = v;
+            one = warp_sum3(pa, ps, ph, lane);
+            if (!solo && (lane == 0 || lane == 8 || lane == 16)) red[lane >> 3][slot] = one;
         }
         G.sync();
-        // every warp sums the slots: eight lanes each A, S and H, lane j of them slots j, j + 8, ..
-        const float* const mine = red[min(lane >> 3, 2)] + (lane & 7);
-        Sum2 tot = {0.f, 0.f};
-        auto take = [&](auto i0, auto i1) {
-            constexpr int I0 = decltype(i0)::value, I1 = decltype(i1)::value;
-            float part[I1 - I0];
-            if (G.ctas == 1) {
-#pragma unroll
-                for (int i = I0; i < I1; ++i) part[i - I0] = mine[8 * i];
-            } else {  // (slot s lies in CTA s % 2)
-                const uint32_t at = cluster_addr(mine, lane % G.ctas);
-#pragma unroll
-                for (int i = I0; i < I1; ++i) part[i - I0] = cluster_ld(at + 32 * i);
-            }
-#pragma unroll
-            for (int i = I0; i < I1; ++i) {
-                const float v = 8 * i + (lane & 7) < nslot ? part[i - I0] : 0.f;
-                tot = i == 0 ? Sum2{v, 0.f} : add2(tot, Sum2{v, 0.f});
-            }
+        // Every warp finds out whether the instance has stopped, the group's last warp (none has fewer
+        // strips) also writes the history.  A plain FP32 sum of H's slots, none of them negative, is
+        // within 2^-21 of itself of the exact one and decides unless the threshold is nearer than twice that.
+        const uint32_t at = G.ctas > 1 ? cluster_addr(&red[0][0], lane % G.ctas) : 0u;  // (slot s lies in CTA s % 2)
+        auto value = [&](int k, int slot) {  // (slots past the last one are read, not used)
+            const int i = k * kBatchSlots + slot;
+            const float v = G.ctas > 1 ? cluster_ld(at + 4 * i) : (&red[0][0])[i];
+            return slot < nslot ? v : 0.f;
         };
-        using I = std::integral_constant<int, 1>;
-        take(std::integral_constant<int, 0>{}, I{});
-        if (nslot > 8) take(I{}, std::integral_constant<int, 2>{});
-        if (nslot > 16) take(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
-        if (nslot > 32) take(std::integral_constant<int, 4>{}, std::integral_constant<int, kBatchSlots / 8>{});
-        if (nslot > 1) {
-            if (nslot > 4) tot = add2(tot, shfl_xor2(tot, 4));
-            if (nslot > 2) tot = add2(tot, shfl_xor2(tot, 2));
-            tot = normal2(add2(tot, shfl_xor2(tot, 1)));
+        const bool writes = G.wid == G.warps - 1;
+        bool bad = false, near = true;
+        float h = 0.f;
+        if (G.warps > 1) {
+            h = value(2, lane);
+            bad = !isfinite(h);
+            if (nslot > 32) {
+                const float more = value(2, lane + 32);
+                bad |= !isfinite(more);
+                h += more;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (nslot > o) h += __shfl_xor_sync(0xffffffffu, h, o);
+            h = __shfl_sync(0xffffffffu, h, 0);
+            near = !(fabsf(h - hstop.hi) > 0x1p-20f * h);
         }
-        if (G.kind == kBatchWarp) __syncwarp();  // (before the next level's slots)
-        const Sum2 H = {__shfl_sync(0xffffffffu, tot.hi, 16), __shfl_sync(0xffffffffu, tot.lo, 16)};
-        if (level == 0) {
-            h0 = H.hi;
-            hstop = threshold(h0);
+        bool below = h < hstop.hi;
+        if (writes || level == 0 || near) {
+            // the exact sums: eight lanes each A, S and H, lane j of them slots j, j + 8, ..
+            const int k = min(lane >> 3, 2), j = lane & 7;
+            Sum2 tot = {solo ? one : value(k, j), 0.f};
+            bad |= k == 2 && !isfinite(tot.hi);
+            auto take = [&](auto first, auto last) {
+                constexpr int I0 = decltype(first)::value, I1 = decltype(last)::value;
+                float part[I1 - I0];
+#pragma unroll
+                for (int i = I0; i < I1; ++i) part[i - I0] = value(k, 8 * i + j);
+#pragma unroll
+                for (int i = I0; i < I1; ++i) {
+                    bad |= k == 2 && !isfinite(part[i - I0]);
+                    tot = add1(tot, part[i - I0]);
+                }
+            };
+            if (nslot > 8) take(std::integral_constant<int, 1>{}, std::integral_constant<int, 2>{});
+            if (nslot > 16) take(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
+            if (nslot > 32) take(std::integral_constant<int, 4>{}, std::integral_constant<int, kBatchSlots / 8>{});
+            if (nslot > 1) {
+                if (nslot > 4) tot = add2(tot, shfl_xor2(tot, 4));
+                if (nslot > 2) tot = add2(tot, shfl_xor2(tot, 2));
+                tot = normal2(add2(tot, shfl_xor2(tot, 1)));
+            }
+            const Sum2 H = {__shfl_sync(0xffffffffu, tot.hi, 16), __shfl_sync(0xffffffffu, tot.lo, 16)};
+            if (level == 0) {
+                h0 = H.hi;
+                hstop = threshold(h0);
+            }
+            below = H.hi < hstop.hi || (H.hi == hstop.hi && H.lo <= hstop.lo);
+            if (writes && (lane == 0 || lane == 8)) reinterpret_cast<float*>(hist + level)[lane >> 3] = mul2(tot, norm);
         }
-        if (!isfinite(H.hi)) {
+        if (__any_sync(0xffffffffu, bad)) {
             status = 1;
             done = true;
         }
-        if (level > 0 && stop_ratio2 > 0.f && (H.hi < hstop.hi || (H.hi == hstop.hi && H.lo <= hstop.lo))) done = true;
+        if (G.kind == kBatchWarp) __syncwarp();  // (its next level's slots go to the same place)
+        if (level > 0 && stop_ratio2 > 0.f && below) done = true;
         if (level == max_level) done = true;
-        // the history, by the group's last warp (none has fewer strips)
-        if (G.wid == G.warps - 1 && (lane == 0 || lane == 8))
-            reinterpret_cast<float*>(hist + level)[lane >> 3] = (float)fma((double)tot.lo, norm, (double)tot.hi * norm);
         cur = (level == 0) ? 0 : 1 - cur;
     }
     if (onchip && level > first_level)
