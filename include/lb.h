@@ -278,8 +278,9 @@ lb_status lb_quadrature_info(lb_quadrature quad, int *q, int *degree, double *xi
  * added and removed between runs (continuous batching); admission is by the
  * device-memory budget of the batch arena.  Lax-Wendroff product sets only.
  * Each instance starts from the shear wave u_y = u0 sin(x_i) (rho = T = 1) and
- * records A(n), S(n) (as in lb_diag, summed in FP32) for every level it
- * processes.  The per-cell arithmetic is the single-lattice one (the same
+ * records A(n), S(n) (as in lb_diag; FP32 sums over each of up to 64 parts of the
+ * grid, the parts added to 2^-46 of their size, rounded to FP32 once) for every level
+ * it processes.  The per-cell arithmetic is the single-lattice one (the same
  * collision function): an instance's results are bitwise the same alone or in
  * any mix, and agree with an lb_handle run of the same problem to FP32 rounding.
  * ------------------------------------------------------------------------- */
@@ -353,14 +354,14 @@ const char *lb_batch_last_error(const lb_batch *b);
  *   dG/dt + xi_k dG/dx = (u - G)/tau,  u = sum_k w_k G_k,
  * at the nodes xi_k of the n_nodes-point Gauss-Hermite rule, started from G = u0 sin x.
  * Strang splitting of the exact relaxation around one Lax-Wendroff step,
- * dt = cfl dx / max|xi_k|, dx = 2 pi / nx, FP64 on the GPU, one CTA per collision
- * time.  For the same-quadrature cross-check of the lattice runs (Sec. 3.2).
+ * dt = cfl dx / max|xi_k|, dx = 2 pi / nx, FP64 on the GPU, a cluster of one to eight
+ * CTAs per collision time.  For the same-quadrature cross-check of the lattice runs (Sec. 3.2).
  *   tau          n_inst collision times (host array)
  *   amp, shear   caller host arrays of n_inst x (nsteps + 1) doubles: A(n) and S(n)
  *                (as in lb_diag, sigma = sum_k w_k xi_k G) of instance i at [i*(nsteps+1) + n]
  *   stream       cudaStream_t (NULL = default); returns after the run.
- * Errors: LB_ERR_ARG; LB_ERR_UNSUPPORTED if n_nodes x nx does not fit one CTA's shared
- * memory (8 (n_nodes + 2) nx bytes); LB_ERR_NOMEM; LB_ERR_CUDA (lb_last_error(NULL)).
+ * Errors: LB_ERR_ARG; LB_ERR_UNSUPPORTED if 8 (n_nodes + 2) nx bytes are more than the shared
+ * memory a CTA may have (227 KB); LB_ERR_NOMEM; LB_ERR_CUDA (lb_last_error(NULL)).
  * ------------------------------------------------------------------------- */
 lb_status lb_dvm_run(int n_inst, const double *tau, int n_nodes, int nx, double cfl, double u0,
                      int nsteps, double *amp, double *shear, void *stream);

@@ -681,9 +681,9 @@ lb_status lb_create_ex(const lb_params* pin, lb_handle** out) {
         const bool big = P.nx >= ttw && h->tma_ntiles >= nsm;
         h->use_tma = P.step_kernel >= 2 || (P.step_kernel == 0 && big);
         // the store-staged kernel (Lax-Wendroff sets): automatic on the same grids where it is
-        // the faster.  Its stores cover whole 16-byte granules of a row, so nx must be a multiple
-        // of 16 / (bytes per population) (else the store of the last tile would reach the
-        // periodic images past nx)
+        // the faster.  It takes nx that are multiples of 16 / (bytes per population), the widths of
+        // whole 16-byte granules in a layout of one velocity a plane (in pairs, FP32 rows of
+        // any even nx would be whole granules; the others run the TMA-staged kernel)
         if (h->shape.st && !upwind && P.nx % (int)(16 / storage_bytes(P.precision)) == 0) {
             h->st_ntiles_x = (P.nx + h->shape.st_tw - 1) / h->shape.st_tw;
             h->st_ntiles = h->st_ntiles_x * ((P.ny + h->shape.st_rows - 1) / h->shape.st_rows);

@@ -38,7 +38,8 @@ cudaError_t setup_s(int threads, int cluster, int* smem, int* grid) {
     cudaError_t e = cudaFuncGetAttributes(&attr, lb_batch_kernel<S>);
     if (e != cudaSuccess) return e;
     const int room = optin - (int)attr.sharedSizeBytes;
-    // a budget within a kilobyte or so of the limit is one that the kernel's own part reaches into
+    // budgets up to 1156 bytes below the device's limit are taken (what a kernel with 1156 bytes of its
+    // own would leave) and brought down to what this kernel leaves; larger ones are refused
     if (*smem > optin - 1156) return cudaErrorInvalidValue;
     if (*smem > room) *smem = room;
     e = cudaFuncSetAttribute(lb_batch_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
