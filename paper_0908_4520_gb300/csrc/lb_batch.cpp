@@ -170,8 +170,8 @@ bool quads(int nw) { return nw > 4 && nw % 4 == 0; }
 // barrier and sums.  The mean load says nothing there: 152 equal instances on 152 SMs have it exactly,
 // and the rule of half the mean put them on clusters, two waves where whole CTAs take one.  A width whose
 // instances at work together take more than three quarters of the L2 is used only if every width's do.
-// us a level, half the mean / this rule (FP32): 152 of D2Q16-GH 256 x 4 13.9 / 8.1, of D2Q64-GH 256 x 4
-// 39.3 / 28.5; 1000 of D2Q16-GH 256 x 1 19.1 / 12.7; 608 of D2Q36-GH 256 x 1 15.9 / 12.4.
+// us a level, half the mean / this rule (FP32): 152 of D2Q16-GH 256 x 4 13.9 / 7.4, of D2Q64-GH 256 x 4
+// 37.8 / 27.3; 1000 of D2Q16-GH 256 x 1 18.9 / 12.6; 608 of D2Q36-GH 256 x 1 16.0 / 12.5.
 int alike_width(const lb_batch* b, const std::vector<long long>& strips) {
     const int nw = b->threads / 32;
     long long n = 0, most = 0, lo = 0, hi = 0;

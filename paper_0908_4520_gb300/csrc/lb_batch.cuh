@@ -201,11 +201,12 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
     int status = 0;
     float h0 = in.h0;
     const double u0 = in.u0;
-    const int isothermal = in.isothermal, max_level = in.max_level;
-    const float stop_ratio2 = in.stop_ratio2;
+    const int isothermal = in.isothermal;
+    // (what is wanted once a level is read from the descriptor there: in registers it cost the strips'
+    // loop spills, D2Q64-GH FP32 N = 4 1024 x 4 44.2 for 41.7 us a level)
     // stop rule sqrt(H / H0) <= stop_ratio (none for stop_ratio = 0, also where H is 0): the largest
     // value of H that meets it, as a sum
-    auto threshold = [&](float h) { return split2((double)stop_ratio2 * (double)h); };
+    auto threshold = [&](float h) { return split2((double)in.stop_ratio2 * (double)h); };
     Sum2 hstop = threshold(h0);
     const Sum2 norm = split2(2.0 / (double)ncell);
 
@@ -341,6 +342,7 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
             for (int o = 16; o > 0; o >>= 1)
                 if (nslot > o) h += __shfl_xor_sync(0xffffffffu, h, o);
             h = __shfl_sync(0xffffffffu, h, 0);
+            bad = __any_sync(0xffffffffu, bad);
             near = !(fabsf(h - hstop.hi) > 0x1p-20f * h);
         }
         bool below = h < hstop.hi;
@@ -348,27 +350,33 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
             // the exact sums: eight lanes each A, S and H, lane j of them slots j, j + 8, ..
             const int k = min(lane >> 3, 2), j = lane & 7;
             Sum2 tot = {solo ? one : value(k, j), 0.f};
-            bad |= k == 2 && !isfinite(tot.hi);
-            auto take = [&](auto first, auto last) {
-                constexpr int I0 = decltype(first)::value, I1 = decltype(last)::value;
-                float part[I1 - I0];
-#pragma unroll
-                for (int i = I0; i < I1; ++i) part[i - I0] = value(k, 8 * i + j);
-#pragma unroll
-                for (int i = I0; i < I1; ++i) {
-                    bad |= k == 2 && !isfinite(part[i - I0]);
-                    tot = add1(tot, part[i - I0]);
-                }
-            };
-            if (nslot > 8) take(std::integral_constant<int, 1>{}, std::integral_constant<int, 2>{});
-            if (nslot > 16) take(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
-            if (nslot > 32) take(std::integral_constant<int, 4>{}, std::integral_constant<int, kBatchSlots / 8>{});
             if (nslot > 1) {
+                bool inf = k == 2 && !isfinite(tot.hi);
+                auto take = [&](auto first, auto last) {
+                    constexpr int I0 = decltype(first)::value, I1 = decltype(last)::value;
+                    float part[I1 - I0];
+#pragma unroll
+                    for (int i = I0; i < I1; ++i) part[i - I0] = value(k, 8 * i + j);
+#pragma unroll
+                    for (int i = I0; i < I1; ++i) {
+                        inf |= k == 2 && !isfinite(part[i - I0]);
+                        tot = add1(tot, part[i - I0]);
+                    }
+                };
+                if (nslot > 8) {
+                    take(std::integral_constant<int, 1>{}, std::integral_constant<int, 2>{});
+                    if (nslot > 16) {
+                        take(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{});
+                        if (nslot > 32) take(std::integral_constant<int, 4>{}, std::integral_constant<int, kBatchSlots / 8>{});
+                    }
+                }
                 if (nslot > 4) tot = add2(tot, shfl_xor2(tot, 4));
                 if (nslot > 2) tot = add2(tot, shfl_xor2(tot, 2));
                 tot = normal2(add2(tot, shfl_xor2(tot, 1)));
+                if (G.warps == 1) bad = __any_sync(0xffffffffu, inf);
             }
             const Sum2 H = {__shfl_sync(0xffffffffu, tot.hi, 16), __shfl_sync(0xffffffffu, tot.lo, 16)};
+            if (nslot == 1) bad = !isfinite(H.hi);
             if (level == 0) {
                 h0 = H.hi;
                 hstop = threshold(h0);
@@ -376,13 +384,13 @@ __device__ __forceinline__ void batch_run(const BatchArgs& B, int id, void* smem
             below = H.hi < hstop.hi || (H.hi == hstop.hi && H.lo <= hstop.lo);
             if (writes && (lane == 0 || lane == 8)) reinterpret_cast<float*>(hist + level)[lane >> 3] = mul2(tot, norm);
         }
-        if (__any_sync(0xffffffffu, bad)) {
+        if (bad) {
             status = 1;
             done = true;
         }
         if (G.kind == kBatchWarp) __syncwarp();  // (its next level's slots go to the same place)
-        if (level > 0 && stop_ratio2 > 0.f && below) done = true;
-        if (level == max_level) done = true;
+        if (level > 0 && in.stop_ratio2 > 0.f && below) done = true;
+        if (level == in.max_level) done = true;
         cur = (level == 0) ? 0 : 1 - cur;
     }
     if (onchip && level > first_level)
